@@ -29,6 +29,8 @@ struct bt_handle {
     int count_nt = 1024;  // schedule used by the next pipeline run (1024: fewest per-block counter arrays)
     int peel_seg = 32;
     int peel_sms = 0;     // SMs the peel kernel spans (0: all); a server worker takes its share
+    bt::Side side;
+    bool grid_peel = false;  // peel with the grid-wide kernel alone (use_grid_peel)
     const bt::GraphSplit *split = nullptr;  // graphs of the batch union being prepared, if any
     std::map<uint64_t, std::pair<int, int>> tuned;  // batch signature -> (count_nt, peel_seg)
     unsigned char *pinned = nullptr;  // page-locked staging for batch copies
@@ -68,6 +70,23 @@ int cuda_fail(bt_handle *h, cudaError_t e, const char *where) {
     return fail(h, BT_ERR_CUDA, "%s: %s", where, cudaGetErrorString(e));
 }
 
+void free_side(bt::Side &s) {
+    if (s.join) cudaEventDestroy(s.join);
+    if (s.fork) cudaEventDestroy(s.fork);
+    if (s.stream) cudaStreamDestroy(s.stream);
+}
+
+// Limits that address the grid-wide peel kernel keep it in use for the whole peel.
+bool grid_peel_only(const bt_handle *h) {
+    const bt_limits &l = h->limits;
+    return h->grid_peel || l.hold_barrier || l.join_cap || l.block_links;
+}
+
+// Up to this many edges (of all graphs of a batch) are peeled by one block as one
+// part.  Below about 1,000 edges that takes less than the rounds of a coarse
+// peel do (300 edges: 0.26 against 0.43 ms; 1,003: 0.72 / 0.75; 2,500: 1.19 / 0.93).
+constexpr uint64_t kWholeEdges = 1024;
+
 int peel_sms(const bt_handle *h) { return h->peel_sms > 0 ? h->peel_sms : h->num_sms; }
 
 bt::Alloc make_alloc(bt_handle *h) {
@@ -76,6 +95,7 @@ bt::Alloc make_alloc(bt_handle *h) {
     al.pool = h->pool;
     al.prof = &h->prof;
     al.limits = &h->limits;
+    al.side = &h->side;
     return al;
 }
 
@@ -248,7 +268,12 @@ int bt_create(bt_handle **out, int device, void *cuda_stream) {
         e = cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
     if (e == cudaSuccess) e = cudaMalloc(&h->err_word, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->side.stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.join, cudaEventDisableTiming);
     if (e != cudaSuccess) {
+        free_side(h->side);
+        if (h->err_word) cudaFree(h->err_word);
         if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
         if (h->pool) cudaMemPoolDestroy(h->pool);
         delete h;
@@ -269,6 +294,7 @@ int bt_destroy(bt_handle *h) {
     for (auto &ev : h->prof.ev)
         if (ev) cudaEventDestroy(ev);
     cudaFree(h->err_word);
+    free_side(h->side);
     if (h->pinned) cudaFreeHost(h->pinned);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -486,7 +512,8 @@ extern "C" int bt_k_bitruss(bt_handle *h, const uint32_t *phi, uint64_t m, uint3
 }
 
 static int build_index_impl(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU,
-                            uint32_t nL, uint32_t flags, uint64_t *d_sup, bt::Alloc &al) {
+                            uint32_t nL, uint32_t flags, uint64_t *d_sup, bt::Alloc &al,
+                            bool one_part = false) {
     Prepared P;
     int rc = prepare(h, edges, m, nU, nL, flags, P, al);
     if (h->has_index) {
@@ -494,6 +521,7 @@ static int build_index_impl(bt_handle *h, const int32_t *edges, uint64_t m, uint
         h->has_index = false;
     }
     bt::Index ix;
+    ix.twin_links = one_part;
     uint64_t bf = 0;
     if (rc == BT_OK) rc = count_and_index(h, P, d_sup, true, ix, bf, al);
     release(P, al);
@@ -504,6 +532,59 @@ static int build_index_impl(bt_handle *h, const int32_t *edges, uint64_t m, uint
         bt::free_index(ix, al);
     }
     return rc;
+}
+
+// Whether a peel of m edges runs as one part (the index then has twin links).
+static bool as_one_part(const bt_handle *h, uint64_t m) { return !grid_peel_only(h) && m <= kWholeEdges; }
+
+// Peels the handle's index: its edges are first told apart by ranges of bitruss
+// numbers (a coarse peel by the whole grid), then the ranges are peeled
+// independently of one another (local.cu).
+static cudaError_t peel_index(bt_handle *h, const uint64_t *sup, uint32_t *phi, bt::PeelResult &pr, int seg,
+                              bt::Alloc &al) {
+    const bt::Index &ix = h->index;
+    if (grid_peel_only(h)) return bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg);
+    bt::PartGraph g;
+    cudaError_t e = cudaSuccess;
+    const size_t held = al.live.size();
+    al.mark(bt::kPhPeel, false);
+    if (ix.twin_links) {
+        e = bt::one_part(ix, sup, g, peel_sms(h), al);
+        if (e == cudaSuccess) e = bt::peel_parts(g, phi, pr, peel_sms(h), al);
+    } else {
+        uint32_t *part = al.get<uint32_t>(ix.m);
+        int *snap = al.get<int>(ix.m);
+        e = al.err;
+        bt::PeelOpts o;
+        o.snap = snap;
+        o.max_parts = bt::kPartsMax;
+        // more parts cost the coarse peel more rounds, fewer leave SMs idle in
+        // the fine one; the best counts grew with the cube root of the twin
+        // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150)
+        o.parts_hint = (uint32_t)(0.305 * std::cbrt((double)ix.w2)) + 1;
+        if (e == cudaSuccess) e = bt::peel(ix, sup, part, pr, peel_sms(h), al, seg, &o);
+        if (e == cudaSuccess && pr.status == BT_OK) {
+            const bt::PeelResult coarse = pr;
+            e = bt::parts_of_ranges(ix, part, snap, coarse.parts, g, peel_sms(h), al);
+            if (e == cudaSuccess) e = bt::peel_parts(g, phi, pr, peel_sms(h), al);
+            pr.slots += coarse.slots;
+            pr.scanned += coarse.scanned;
+        }
+        al.put(part);
+        al.put(snap);
+    }
+    al.mark(bt::kPhPeel, true);
+    if (e == cudaErrorMemoryAllocation && !al.injected && !ix.twin_links) {
+        // parts need about 46 more bytes a twin pair than the grid-wide peel
+        // alone: an index that leaves no room for them is still peeled
+        cudaGetLastError();
+        al.undo_to(held);
+        al.err = cudaSuccess;
+        e = cudaStreamSynchronize(h->stream);
+        return e == cudaSuccess ? bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg) : e;
+    }
+    bt::free_parts(g, al);
+    return e;
 }
 
 int bt_build_index(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL,
@@ -601,7 +682,7 @@ int bt_decompose(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, ui
     uint64_t *s_int = al.get<uint64_t>(m);  // internal edge order
     uint32_t *p_int = al.get<uint32_t>(m);
     if (al.err != cudaSuccess) return cuda_fail(h, al.err, "allocating outputs");
-    rc = build_index_impl(h, edges, m, nU, nL, flags, s_int, al);
+    rc = build_index_impl(h, edges, m, nU, nL, flags, s_int, al, as_one_part(h, m));
     bt::PeelResult pr;
     if (rc == BT_OK) {
         // larger work items pay off when rounds are heavy: on the 30M-edge
@@ -610,7 +691,7 @@ int bt_decompose(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, ui
         // and 21.9 s with 32; on graphs with up to 2e8 pairs 32 measured
         // 3-8 % faster than 64
         const int seg = h->index.w2 > (1ull << 30) ? 128 : h->peel_seg;
-        cudaError_t e = bt::peel(h->index, s_int, p_int, pr, peel_sms(h), al, seg);
+        cudaError_t e = peel_index(h, s_int, p_int, pr, seg, al);
         if (e == cudaSuccess) e = bt::gather_u64(s_int, h->index.newid, d_sup, m, al);
         if (e == cudaSuccess) e = bt::gather_u32(p_int, h->index.newid, d_phi, m, al);
         if (e != cudaSuccess) rc = cuda_fail(h, e, "peeling");
@@ -786,12 +867,12 @@ static int decompose_union(bt_handle *h, const bt_graph *graphs, uint32_t n, uin
         for (uint32_t g = 0; g < n; ++g) split.max_n = std::max(split.max_n, gnU[g] + gnL[g]);
         h->split = &split;
         rc = build_index_impl(h, d_edges, M, (uint32_t)NU, (uint32_t)NL,
-                              (flags & BT_TIE_LOWER_FIRST) | BT_DEVICE_PTRS, d_sup, al);
+                              (flags & BT_TIE_LOWER_FIRST) | BT_DEVICE_PTRS, d_sup, al, as_one_part(h, M));
         h->split = nullptr;
     }
     bt::PeelResult pr;
     if (rc == BT_OK && M > 0) {
-        e = bt::peel(h->index, d_sup, d_phi, pr, peel_sms(h), al, h->peel_seg);
+        e = peel_index(h, d_sup, d_phi, pr, h->peel_seg, al);
         // results back to input order (the edge array is free by now: reuse it)
         uint64_t *g_sup = reinterpret_cast<uint64_t *>(d_edges);
         uint32_t *g_phi = al.get<uint32_t>(M);
@@ -1266,5 +1347,9 @@ namespace bt {
 // latency-bound, so half the SMs cost the 2M-edge peel about 6 %.
 void share_peel_sms(bt_handle *h, int ways) {
     if (h && ways > 1) h->peel_sms = h->num_sms / ways > 0 ? h->num_sms / ways : 1;
+}
+
+void use_grid_peel(bt_handle *h) {
+    if (h) h->grid_peel = true;
 }
 }  // namespace bt

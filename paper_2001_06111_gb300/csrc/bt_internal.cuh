@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <vector>
+
 #include "../../include/bitruss.h"
 
 namespace bt {
@@ -27,6 +29,13 @@ struct Prof {
     bool used[kNumPhases] = {};
 };
 
+// A second stream of the handle, for kernels that run beside one another inside
+// a call: forked from the call's stream and joined to it before the call goes on.
+struct Side {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+
 // Stream-ordered scratch allocation from the handle's memory pool, plus the
 // call's launch counter and profiler.
 struct Alloc {
@@ -35,6 +44,7 @@ struct Alloc {
     cudaError_t err = cudaSuccess;
     uint64_t launches = 0;
     Prof *prof = nullptr;
+    const Side *side = nullptr;
     // Optional fixed arena (set only by the allocation-free entry point):
     // get() then bump-allocates inside it and put() does nothing.
     unsigned char *arena = nullptr;
@@ -43,6 +53,16 @@ struct Alloc {
     // null.  fail_alloc_at = n > 0 makes allocation number n of this call fail.
     const bt_limits *limits = nullptr;
     uint64_t n_allocs = 0;
+    bool injected = false;  // the failure in err was asked for
+    // what get() gave and put() has not taken back, so that a step that runs out
+    // of memory half way can be undone (undo_to)
+    std::vector<void *> live;
+    void undo_to(size_t held) {
+        while (live.size() > held) {
+            cudaFreeAsync(live.back(), stream);
+            live.pop_back();
+        }
+    }
     // NVTX push/pop ranges of the phases, nested call > csr, count, emit,
     // peel (host-side issue order; no-ops unless a profiler is attached).
     // Ranges an early error return left open are popped when the call's
@@ -76,6 +96,7 @@ struct Alloc {
         if (err != cudaSuccess) return nullptr;
         if (limits && limits->fail_alloc_at && ++n_allocs == limits->fail_alloc_at) {
             err = cudaErrorMemoryAllocation;
+            injected = true;
             return nullptr;
         }
         void *p = nullptr;
@@ -91,10 +112,18 @@ struct Alloc {
             return reinterpret_cast<T *>(arena + off);
         }
         err = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
-        return err == cudaSuccess ? static_cast<T *>(p) : nullptr;
+        if (err != cudaSuccess) return nullptr;
+        live.push_back(p);
+        return static_cast<T *>(p);
     }
     void put(void *p) {
-        if (p && !arena) cudaFreeAsync(p, stream);
+        if (!p || arena) return;
+        cudaFreeAsync(p, stream);
+        for (size_t i = live.size(); i-- > 0;)
+            if (live[i] == p) {
+                live.erase(live.begin() + (long)i);
+                break;
+            }
     }
 };
 
@@ -201,7 +230,10 @@ struct Index {
     uint64_t *inc_off = nullptr;     // [m+1]
     // [links] per edge: (pair id, bloom id | side << 31), side 0 when the
     // edge is the pair's first member (e_uv), 1 when it is the second
+    // with twin_links (set before emit): (twin edge id, bloom id) instead, the
+    // links the part peel follows
     uint2 *inc = nullptr;
+    bool twin_links = false;
     uint32_t *newid = nullptr;       // [m] input edge id -> internal id (ids above are internal)
     size_t bytes() const {
         return nb * 8 + 4 + w2 * 8 + (m + 1) * 8 + links * 8;
@@ -215,6 +247,7 @@ void free_index(Index &ix, Alloc &al);
 struct PeelResult {
     uint64_t rounds = 0, levels = 0, updates = 0, kmax = 0, windows = 0, slots = 0, scanned = 0;
     uint64_t inc_phases = 0;  // rounds that ran a separate incidence phase
+    uint32_t parts = 0;       // coarse peel: parts made
     int status = BT_OK;
 };
 // support: [m] initial supports (device, preserved); phi_out: [m] device.
@@ -226,14 +259,63 @@ struct PeelOpts {
     uint64_t m_active = 0;
     long long k_init = 0;
     long long assign_from = 0;
+    // Coarse peel (snap set): edges are told apart only by the part their
+    // bitruss number falls in.  A level is a range of bitruss numbers that
+    // aims at 1/parts_hint of all links and edges; phi_out receives the part of every edge (parts
+    // ascend with phi) and snap its support when its part began, all edges of
+    // lower parts being gone.
+    int *snap = nullptr;
+    uint32_t parts_hint = 0, max_parts = 0;
 };
 // seg: peel work-item size (32 or 64 entries; anything else means 32)
 cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, PeelResult &res,
                  int num_sms, Alloc &al, int seg = 32, const PeelOpts *opts = nullptr);
 
+// Parts that can be peeled independently of one another (local.cu).  Part p
+// owns the edges [part_e[p], part_e[p + 1]) of the part graph's own numbering
+// and touches at most part_b[p + 1] - part_b[p] blooms.
+constexpr uint32_t kBlockEdges = 43008;  // edges of a part whose supports fit one block's shared memory
+constexpr uint32_t kPartsMax = 1024;     // parts of a coarse peel
+// A bloom inside a part, one 32-byte sector.
+struct __align__(32) BloomRec {
+    uint32_t first, n;   // its pairs: here if n <= 2, else from pairs[first]
+    uint32_t k, c;       // k_B, pairs that died in the current round
+    uint2 pair[2];
+};
+struct PartGraph {
+    uint64_t m = 0, nb = 0;
+    uint32_t np = 0;
+    const uint32_t *part_e = nullptr, *part_b = nullptr;  // [np + 1]
+    const uint32_t *order = nullptr;  // [np] parts in the order they are taken (null: last first)
+    uint32_t n_heavy = 0;             // the first n_heavy of them by a cluster of blocks each
+    uint4 *er = nullptr;              // [m] per edge: first link (64 bits), links, support when its part begins
+    const uint2 *inc = nullptr;       // links: (twin | flag << 31 when the twin lies in a higher part, bloom)
+    const uint2 *pairs = nullptr;     // twin pairs (flagged the same way) of blooms of more than two
+    BloomRec *bl = nullptr;           // consumed by the peel
+    const uint32_t *out_id = nullptr;  // [m] the index's id of each edge, or null when the numbering is the same
+    void *own[8] = {};  // what free_parts gives back
+    int n_own = 0;
+    template <typename T>
+    T *keep(T *x) {
+        own[n_own++] = x;
+        return x;
+    }
+};
+void free_parts(PartGraph &g, Alloc &al);
+// The whole graph as one part (an index with twin links).
+cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al);
+// The ranges of a coarse peel as parts: part[e] in [0, np), snap[e] the support
+// of e when its part begins.
+cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np, PartGraph &g,
+                            int num_sms, Alloc &al);
+// Peel of all parts.
+cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, PeelResult &res, int num_sms, Alloc &al);
+
 // ---------------------------------------------------------------- serving
 // The peel of handle h spans 1/ways of the SMs (server workers share the GPU).
 void share_peel_sms(bt_handle *h, int ways);
+// Handle h peels with the grid-wide kernel alone, without parts.
+void use_grid_peel(bt_handle *h);
 
 // ---------------------------------------------------------------- hierarchy
 // order[i]: edge ids by phi descending, equal phi in ascending id (stable);

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(NT) k_emit(
     unsigned long long *cw_all, const uint64_t *__restrict__ bloom_base,
     const uint64_t *__restrict__ pair_base, const uint64_t *__restrict__ inc_off,
     uint32_t *inc_fill, uint32_t *bloom_k, uint32_t *bloom_off, uint2 *pairs,
-    uint2 *inc, uint32_t *queue, const uint8_t *__restrict__ assigned) {
+    uint2 *inc, uint32_t *queue, const uint8_t *__restrict__ assigned, bool twin) {
     __shared__ Chunk<NT> ch;
     __shared__ uint32_t s_q;
     // bloom count (high 32 bits) and pair count (low 32 bits) of the vertex,
@@ -298,14 +298,15 @@ __global__ void __launch_bounds__(NT) k_emit(
                     const bool fu = assigned && assigned[euv], fw = assigned && assigned[evw];
                     // an assigned edge is flagged in bit 31 and gets no link
                     pairs[slot] = make_uint2(euv | (fu ? 0x80000000u : 0u), evw | (fw ? 0x80000000u : 0u));
-                    // each link carries its bloom and which member of the pair the edge is
+                    // each link carries its bloom and which member of the pair
+                    // the edge is, or the twin itself and the bloom
                     if (!fu) {
                         uint32_t q1 = atomicAdd(&inc_fill[euv], 1u);
-                        inc[inc_off[euv] + q1] = make_uint2(slot, (uint32_t)B);
+                        inc[inc_off[euv] + q1] = make_uint2(twin ? evw : slot, (uint32_t)B);
                     }
                     if (!fw) {
                         uint32_t q2 = atomicAdd(&inc_fill[evw], 1u);
-                        inc[inc_off[evw] + q2] = make_uint2(slot, (uint32_t)B | 0x80000000u);
+                        inc[inc_off[evw] + q2] = make_uint2(twin ? euv : slot, (uint32_t)B | (twin ? 0u : 0x80000000u));
                     }
                 }
             }
@@ -428,7 +429,7 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     al.mark(kPhEmit, false);
 #define BT_EMIT_ARGS                                                                         \
     g.off, g.adj, g.eid, g.hv, g.pl, g.wv, n, g.vbase, g.cnt_n, cw, bloom_base, pair_base, ix.inc_off,  \
-        inc_fill, ix.bloom_k, ix.bloom_off, ix.pairs, ix.inc, queue, c.assigned
+        inc_fill, ix.bloom_k, ix.bloom_off, ix.pairs, ix.inc, queue, c.assigned, ix.twin_links
     if (nt == 256) k_emit<256><<<blocks, 256, 0, al.stream>>>(BT_EMIT_ARGS);
     else if (nt == 1024) k_emit<1024><<<blocks, 1024, 0, al.stream>>>(BT_EMIT_ARGS);
     else k_emit<512><<<blocks, 512, 0, al.stream>>>(BT_EMIT_ARGS);

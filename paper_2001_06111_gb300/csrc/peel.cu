@@ -32,10 +32,10 @@
 // second barrier) only when such items exist or a level jump selected the
 // batch.  Pairs killed early carry stamp r + 1 and still count as alive in
 // the bloom phase of round r.  The bloom number at the start of round q is
-// the value recorded after the last round that touched the bloom, less
-// C_{q-1} when round q - 1 touched it and its bloom phase has not recorded
-// the new value yet.  Work is split into items of at most kSeg entries, so no
-// warp straggles on a hub edge or bloom.  A twin pair carries the round it
+// the value recorded after the last round before q that touched the bloom; the
+// bloom's first item of round q records the new one during q's bloom phase.
+// Work is split into items of at most kSeg entries, so no warp straggles on a
+// hub edge or bloom; a warp lays the entries of its items side by side.  A twin pair carries the round it
 // died in; the edges of a batch race to stamp it with atomicCAS, so exactly
 // one of them counts it in C(B); the stamp also records which members of the
 // pair are in the batch (the killer's side bit, and the other member's bit
@@ -44,6 +44,18 @@
 // (C by 3, bloom items by 4, batch sizes by 3, incidence items by 2) so each
 // is reset a barrier after its last reader.  Data written by other blocks
 // during the kernel is read with L2 (.cg) loads.
+//
+// Coarse peel (kCoarse).  The same rounds with levels that are ranges of bitruss
+// numbers: a level takes every edge whose support is, or falls, within the range,
+// so phi is known only up to the range (the part), in a fraction of the rounds
+// (2M-edge graph: 865 instead of 39,928).  Each part can then be peeled by itself
+// (split.cu, local.cu).  A level jump reads the alive edges, copies their
+// supports, histograms them by class and takes classes until their weight (edges
+// and links) reaches the target.  The jump's list of alive edges is written
+// anew only after a quarter has gone: taking places from one counter at every
+// jump cost 130 us of it at 2M edges (now 30 us).
+#include <limits.h>
+
 #include "bt_device.cuh"
 #include "bt_internal.cuh"
 
@@ -52,16 +64,14 @@ namespace {
 
 // entries per work item: SEG = 32, 64 or 128 (template parameter: 32 or 64
 // picked by the batch autotuner, 128 for indexes of over 2^30 twin pairs);
-// each lane handles SEG / 32 entries with their loads and atomics issued
-// together.  Threads a block: 640 (96 registers, no spills) for 32- and
+// a coarse peel knows 32 and 128).  Threads a block: 640 (96 registers, no spills) for 32- and
 // 64-entry items, 512 (128 registers) for 128-entry items, whose four slots
 // a lane need the registers.
 __host__ __device__ constexpr int peel_threads(uint32_t seg) { return seg == 128 ? 512 : 640; }
-// items with at most kSmall entries are processed by one lane each, larger
-// ones by the whole warp.  Lane l of warp w takes item w + l * nwarps (plus
-// multiples of 32 * nwarps): a round with fewer items than warps still gives
-// every item its own warp, and a large round fills all lanes.
-constexpr uint32_t kSmall = 2;
+// Lane l of warp w takes item w + l * nwarps (plus multiples of 32 * nwarps),
+// and the warp works on the entries of its items side by side: a round with
+// fewer items than warps still gives every item its own warp, and a large
+// round fills all lanes however small its items are.
 // edges that join the next batch in a bloom phase are listed per block (up to
 // one per thread); the block kills their twin pairs at the end of the phase,
 // two links per thread, for the edges whose links fit in the first two per
@@ -76,6 +86,21 @@ constexpr uint32_t kErrPeelOverflow = 4u;
 constexpr unsigned kFull = 0xffffffffu;
 // level-jump windows above this size queue their batch with warp-aggregated atomics
 constexpr uint32_t kWarpSlotsMin = 1u << 16;
+
+// Support classes of the coarse peel: values below 64 apart, above that 64 a
+// power of two.
+constexpr uint32_t kBins = 2048;
+__device__ __forceinline__ uint32_t bin_of(unsigned long long s) {
+    if (s < 64ull) return (uint32_t)s;
+    const uint32_t x = s > 0x7FFFFFFFull ? 0x7FFFFFFFu : (uint32_t)s;
+    const uint32_t e = 31u - (uint32_t)__clz(x);
+    return ((e - 5u) << 6) + ((x >> (e - 6u)) & 63u);
+}
+__device__ __forceinline__ long long bin_top(uint32_t b) {
+    if (b < 64u) return b;
+    const uint32_t e = (b >> 6) + 5u;
+    return ((long long)(64u + (b & 63u) + 1u) << (e - 6u)) - 1;
+}
 
 struct Ctl {
     unsigned long long bar_count;  // barrier arrivals (monotonic within a launch)
@@ -97,6 +122,18 @@ struct Ctl {
     unsigned long long windows;
     unsigned long long kfinal;
     unsigned long long inc_phases;  // rounds that ran a separate incidence phase
+    unsigned int n_parts;           // coarse peel: parts made
+    unsigned int hist[2][kBins];    // coarse peel: supports of the alive edges, ping-pong
+};
+
+// What changes of a bloom, in one 32-byte sector.  A kill touches it with one
+// counter atomic and no load: a load beside an atomic on the same sector
+// costs three times the atomic (the part peel's kills went from 14 to 5 ns
+// a link an SM without it).
+struct __align__(32) BloomWord {
+    unsigned long long bw;      // last round that touched it << 32 | k_B after it
+    uint32_t C[3];              // C_r by round mod 3
+    uint32_t pad[3];
 };
 
 struct PeelArgs {
@@ -105,14 +142,13 @@ struct PeelArgs {
     const uint2 *inc;  // (pair, bloom | side << 31)
     const uint2 *pairs;
     const uint32_t *bloom_off;
+    BloomWord *blooms;
     long long *sup;
     uint32_t *state;
     uint32_t *phi;
     uint32_t *died;           // death stamp of a twin pair (kAlive while alive)
-    unsigned long long *bw;   // per bloom: last round that touched it << 32 | k_B after it
-    uint32_t *Cb[3];          // C_r by round mod 3
     uint4 *items[2];          // (edge, first link lo, first link hi, count | head flag << 31)
-    uint4 *bseg[4];           // (bloom, first pair, count | head flag << 31, k_B at round start)
+    uint4 *bseg[4];           // (bloom, first pair, count | head flag << 31, 0)
     uint32_t *alive[2];
     uint32_t *near[2];
     uint64_t item_cap;
@@ -128,6 +164,12 @@ struct PeelArgs {
     uint64_t m_active;
     long long k_init;
     long long assign_from;
+    // coarse peel: phi receives the part of every edge instead, snap its support
+    // when its part began.  An edge weighs 1 + (links >> wshift), a part aims at
+    // a weight of `target`.
+    int *snap;
+    uint32_t target, wshift;
+    uint32_t max_parts;
 };
 
 // Loop state every thread keeps identically (derived from values read after
@@ -136,6 +178,7 @@ struct Lvl {
     long long k;    // current level
     long long khi;  // top of the near window: alive edges with support < khi are listed
     uint32_t nq;    // current near list
+    uint32_t label;  // what a peeled edge receives: k, or its part in a coarse peel
 };
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -235,9 +278,9 @@ __device__ __forceinline__ void push_items(const PeelArgs &a, uint32_t e, uint32
 }
 
 // Edge e joins the batch of round q at level k.
-__device__ __forceinline__ void join_batch(const PeelArgs &a, uint32_t e, uint32_t q, long long k) {
+__device__ __forceinline__ void join_batch(const PeelArgs &a, uint32_t e, uint32_t q, const Lvl &L) {
     a.state[e] = q;
-    if (k >= a.assign_from) a.phi[e] = (uint32_t)k;  // e leaves in a batch of this level
+    if (L.k >= a.assign_from) a.phi[e] = L.label;  // e leaves in a batch of this level
 }
 
 __device__ __forceinline__ void push_near(const PeelArgs &a, uint32_t e, uint32_t nq) {
@@ -250,20 +293,6 @@ __device__ __forceinline__ void push_near(const PeelArgs &a, uint32_t e, uint32_
 __device__ __forceinline__ long long window_top(long long kmin) {
     long long w = kmin / 64;
     return kmin + (w < 8 ? 8 : w);
-}
-
-// One kill of a pair of bloom B for round q: count it in C_q(B).  Returns
-// true for the first kill of B in round q, with B's first pair, pair count
-// and k_B at the start of round q (its bloom items are then queued).
-__device__ __forceinline__ bool count_kill(const PeelArgs &a, uint32_t B, uint32_t q, uint32_t &bo0,
-                                           uint32_t &span, uint32_t &kB) {
-    bo0 = a.bloom_off[B];
-    const uint32_t bo1 = a.bloom_off[B + 1];
-    const unsigned long long w = __ldcg(&a.bw[B]);
-    const uint32_t cprev = __ldcg(&a.Cb[(q + 2u) % 3u][B]);  // C_{q-1}(B)
-    span = bo1 - bo0;
-    kB = (uint32_t)(w >> 32) == q - 1u ? (uint32_t)w : (uint32_t)w - cprev;
-    return atomicAdd(&a.Cb[q % 3u][B], 1u) == 0u;
 }
 
 // Edges of the batch of round q kill the pairs of up to N links (won[r] set
@@ -285,71 +314,93 @@ __device__ __forceinline__ void kill_pairs(const PeelArgs &a, const uint2 (&l)[N
     }
 }
 
+// Places of bloom items a warp has taken from the list's counter and not filled
+// yet: in an incidence phase a warp takes kTake at a time, since millions of
+// first kills would otherwise queue on the one counter (about 4 ns each).
+// What is left at the end is filled with empty items.
+constexpr uint32_t kTake = 128;
+struct Slots {
+    uint32_t next = 0, left = 0;
+};
+__device__ __forceinline__ void fill_empty(const PeelArgs &a, uint32_t qb, Slots &t, int lane) {
+    for (uint32_t i = lane; i < t.left; i += 32) a.bseg[qb][t.next + i] = make_uint4(0u, 0u, 0u, 0u);
+    t.left = 0;
+}
+
 // Whole warp (converged): each lane's pairs killed for round q (won[r], bloom
 // B[r]) are counted, and the blooms killed for the first time in round q get
-// their bloom items (one per kSeg pairs, each with k_B at the start of round
-// q).  The warp takes all its item slots with one atomic: in large rounds
-// millions of first kills would otherwise queue on the one counter.
-template <uint32_t kSeg, uint32_t N>
+// their bloom items (one per kSeg pairs).  kMode: how the places of the items
+// are taken: 0 one counter atomic a warp, 1 one a block (called by the whole
+// block), 2 from the warp's stock t.
+template <uint32_t kSeg, uint32_t N, int kMode>
 __device__ __forceinline__ void warp_kills(const PeelArgs &a, uint32_t q, const uint32_t (&B)[N],
-                                           const bool (&won)[N], int lane) {
-    uint32_t bo0[N], span[N], kB[N], nseg[N];
+                                           const bool (&won)[N], int lane, Slots &t) {
+    // a lane's loads, then its counter atomics, go out together
+    uint32_t bo0[N], span[N], prev[N], nseg[N];
     uint32_t mine = 0;
-    if constexpr (N >= 4) {
-        // four kills a lane: their bloom loads, then their count atomics, go
-        // out together
-        uint32_t prev[N];
 #pragma unroll
-        for (uint32_t r = 0; r < N; ++r) {
-            if (won[r]) {
-                bo0[r] = a.bloom_off[B[r]];
-                span[r] = a.bloom_off[B[r] + 1] - bo0[r];
-                const unsigned long long w = __ldcg(&a.bw[B[r]]);
-                const uint32_t cprev = __ldcg(&a.Cb[(q + 2u) % 3u][B[r]]);  // C_{q-1}(B)
-                kB[r] = (uint32_t)(w >> 32) == q - 1u ? (uint32_t)w : (uint32_t)w - cprev;
-            }
-        }
+    for (uint32_t r = 0; r < N; ++r) {
+        bo0[r] = won[r] ? a.bloom_off[B[r]] : 0u;
+        span[r] = won[r] ? a.bloom_off[B[r] + 1] - bo0[r] : 0u;
+    }
 #pragma unroll
-        for (uint32_t r = 0; r < N; ++r) prev[r] = won[r] ? atomicAdd(&a.Cb[q % 3u][B[r]], 1u) : 1u;
+    for (uint32_t r = 0; r < N; ++r) prev[r] = won[r] ? atomicAdd(&a.blooms[B[r]].C[q % 3u], 1u) : 1u;
 #pragma unroll
-        for (uint32_t r = 0; r < N; ++r) {
-            nseg[r] = prev[r] == 0u ? (span[r] + kSeg - 1) / kSeg : 0u;
-            mine += nseg[r];
-        }
+    for (uint32_t r = 0; r < N; ++r) {
+        nseg[r] = prev[r] == 0u ? (span[r] + kSeg - 1) / kSeg : 0u;
+        mine += nseg[r];
+    }
+    const uint32_t qb = q & 3u;
+    uint32_t slot;
+    if constexpr (kMode == 1) {
+        uint32_t all;
+        slot = dev::block_excl_scan<uint32_t>(mine, &all);
+        if (all == 0) return;
+        __shared__ uint32_t s_base;
+        if (threadIdx.x == 0) s_base = atomicAdd(&a.ctl->n_bseg[qb], all);
+        __syncthreads();
+        slot += s_base;
     } else {
-#pragma unroll
-        for (uint32_t r = 0; r < N; ++r) {
-            nseg[r] = 0;
-            if (won[r] && count_kill(a, B[r], q, bo0[r], span[r], kB[r])) nseg[r] = (span[r] + kSeg - 1) / kSeg;
-            mine += nseg[r];
+        const uint32_t incl = dev::warp_incl_scan(mine);
+        const uint32_t all = __shfl_sync(kFull, incl, 31);
+        if (all == 0) return;
+        if constexpr (kMode == 2) {
+            if (all > t.left) {
+                fill_empty(a, qb, t, lane);
+                const uint32_t take = all > kTake ? all : kTake;
+                uint32_t base = 0;
+                if (lane == 0) base = atomicAdd(&a.ctl->n_bseg[qb], take);
+                t.next = __shfl_sync(kFull, base, 0);
+                t.left = take;
+            }
+            slot = t.next + incl - mine;
+            t.next += all;
+            t.left -= all;
+        } else {
+            uint32_t base = 0;
+            if (lane == 31) base = atomicAdd(&a.ctl->n_bseg[qb], all);
+            slot = __shfl_sync(kFull, base, 31) + incl - mine;
         }
     }
-    const uint32_t incl = dev::warp_incl_scan(mine);
-    const uint32_t all = __shfl_sync(kFull, incl, 31);
-    if (all == 0) return;
-    const uint32_t qb = q & 3u;
-    uint32_t base = 0;
-    if (lane == 31) base = atomicAdd(&a.ctl->n_bseg[qb], all);
-    uint32_t slot = __shfl_sync(kFull, base, 31) + incl - mine;
 #pragma unroll
     for (uint32_t r = 0; r < N; ++r)
         for (uint32_t s = 0; s < nseg[r]; ++s, ++slot) {
             const uint32_t left = span[r] - s * kSeg;
             a.bseg[qb][slot] =
-                make_uint4(B[r], bo0[r] + s * kSeg, (left < kSeg ? left : kSeg) | (s == 0 ? 0x80000000u : 0u), kB[r]);
+                make_uint4(B[r], bo0[r] + s * kSeg, (left < kSeg ? left : kSeg) | (s == 0 ? 0x80000000u : 0u), 0u);
         }
 }
 
 // Edge e joins the batch of round q in a bloom phase: it goes to the block's
 // list, or, when that is full, the lane queues its links itself.
 template <uint32_t kSeg>
-__device__ __forceinline__ void join_next(const PeelArgs &a, uint32_t e, uint32_t q, long long k,
+__device__ __forceinline__ void join_next(const PeelArgs &a, uint32_t e, uint32_t q, const Lvl &L,
                                           uint32_t *s_je, uint32_t *s_jn) {
     const uint32_t slot = atomicAdd(s_jn, 1u);
     if (slot < a.join_cap) {
         s_je[slot] = e;
     } else {
-        join_batch(a, e, q, k);
+        join_batch(a, e, q, L);
         push_items<kSeg>(a, e, q & 1u, a.inc_off[e], a.inc_off[e + 1]);
         atomicAdd(&a.ctl->n_edges[q % 3u], 1u);
     }
@@ -361,8 +412,8 @@ __device__ __forceinline__ void join_next(const PeelArgs &a, uint32_t e, uint32_
 // travel together.
 template <uint32_t kSeg, uint32_t N>
 __device__ __forceinline__ void apply_slots(const PeelArgs &a, const uint32_t (&d)[N], const uint2 (&pr)[N],
-                                            uint32_t c, uint32_t kB, const Lvl &L, uint32_t round,
-                                            unsigned long long &upd, uint32_t *s_je, uint32_t *s_jn) {
+                                            const uint32_t (&c)[N], const uint32_t (&kB)[N], const Lvl &L,
+                                            uint32_t round, unsigned long long &upd, uint32_t *s_je, uint32_t *s_jn) {
     const uint32_t q = round + 1u;
     uint32_t e[2 * N];
     long long dec[2 * N];
@@ -379,13 +430,13 @@ __device__ __forceinline__ void apply_slots(const PeelArgs &a, const uint32_t (&
         if (d[r] == kAlive || dr == q) {
             // alive during this round (a pair killed for the next round still
             // is): one butterfly lost per dead pair
-            if (!fx) dec[2 * r] = c;
-            if (!fy) dec[2 * r + 1] = c;
-        } else if (dr == round && kB > 1u) {
+            if (!fx) dec[2 * r] = c[r];
+            if (!fy) dec[2 * r + 1] = c[r];
+        } else if (dr == round && kB[r] > 1u) {
             // died now: a member outside S (its bit not stamped) loses its
             // k_B - 1 butterflies
-            if (!(fx || (d[r] & 1u))) dec[2 * r] = (long long)kB - 1;
-            if (!(fy || (d[r] & 2u))) dec[2 * r + 1] = (long long)kB - 1;
+            if (!(fx || (d[r] & 1u))) dec[2 * r] = (long long)kB[r] - 1;
+            if (!(fy || (d[r] & 2u))) dec[2 * r + 1] = (long long)kB[r] - 1;
         }
     }
     long long old[2 * N];
@@ -402,11 +453,11 @@ __device__ __forceinline__ void apply_slots(const PeelArgs &a, const uint32_t (&
         if (old[i] >= L.khi && now < L.khi) push_near(a, e[i], L.nq);
         // exactly one decrement takes the edge from > k to <= k: it joins the
         // next batch
-        if (old[i] > L.k && now <= L.k) join_next<kSeg>(a, e[i], q, L.k, s_je, s_jn);
+        if (old[i] > L.k && now <= L.k) join_next<kSeg>(a, e[i], q, L, s_je, s_jn);
     }
 }
 
-template <uint32_t kSeg>
+template <uint32_t kSeg, bool kCoarse>
 __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     constexpr uint32_t R = kSeg / 32;  // entries per lane
     constexpr uint32_t kT = peel_threads(kSeg);
@@ -419,7 +470,8 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     Ctl *ctl = a.ctl;
     uint64_t remaining = a.m_active;
     uint32_t round = 0;
-    Lvl L{a.k_init, 0, 0};
+    // (a coarse peel keeps no window: khi below every support)
+    Lvl L{a.k_init, kCoarse ? LLONG_MIN : 0ll, 0, (uint32_t)a.k_init};
     uint32_t ap = 0;  // current alive list
     bool level_jump = true;
     unsigned long long upd = 0, slots = 0;
@@ -429,6 +481,11 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     __shared__ unsigned long long s_jib[kJoinCap];
     __shared__ uint32_t s_jn;
     __shared__ SnapVals s_v;
+    __shared__ uint32_t s_hist[kCoarse ? kBins : 1];
+    __shared__ uint32_t s_bin, s_cum;
+    // coarse: parts begun, the weight the last one began with, all weight then
+    uint32_t pno = 0, picked = 1, total_jump = 0;
+    float aim = (float)a.target;
     if (threadIdx.x == 0) s_jn = 0;
     __syncthreads();
     // list sizes, kept identically by every thread from the barrier snapshots
@@ -446,7 +503,176 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
             if (gtid == 0) atomicOr(&ctl->err, kErrRounds);
             break;
         }
-        if (level_jump) {
+        if constexpr (kCoarse) {
+            if (level_jump) {
+                // C1: the alive edges again, with their supports' histogram and
+                // a copy of each support (the last copy an edge gets is its
+                // support when its part begins)
+                for (uint32_t i = threadIdx.x; i < kBins; i += kT) s_hist[i] = 0;
+                __syncthreads();
+                if (gtid == 0) atomicAdd(&ctl->scanned, 2ull * v_alive);
+                // the list is written anew only once a quarter of it is gone:
+                // its places come from one counter, which is what that costs
+                const bool anew = remaining < v_alive - v_alive / 4u;
+                constexpr uint32_t U = 4;  // entries a lane has in flight
+                for (uint32_t i0 = gwarp * 32u * U; i0 < v_alive; i0 += nthreads * U) {
+                    uint32_t e[U], stv[U];
+                    long long sv[U];
+                    bool keep[U];
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        const uint32_t i = i0 + 32u * r + lane;
+                        keep[r] = i < v_alive;
+                        e[r] = keep[r] ? ldcg_u32(&a.alive[ap][i]) : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        stv[r] = keep[r] ? ldcg_u32(&a.state[e[r]]) : 0u;
+                        sv[r] = keep[r] ? ldcg_ll(&a.sup[e[r]]) : 0ll;
+                    }
+                    uint32_t n = 0, at[U];
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        keep[r] = keep[r] && stv[r] == kAlive;
+                        if (keep[r]) {
+                            a.snap[e[r]] = (int)sv[r];
+                            const uint64_t d = a.inc_off[e[r] + 1] - a.inc_off[e[r]];
+                            atomicAdd(&s_hist[bin_of((unsigned long long)sv[r])], 1u + (uint32_t)(d >> a.wshift));
+                        }
+                        const unsigned int mask = __ballot_sync(kFull, keep[r]);
+                        at[r] = n + __popc(mask & ((1u << lane) - 1u));
+                        n += __popc(mask);
+                    }
+                    if (anew && n) {
+                        uint32_t base = 0;
+                        if (lane == 0) base = atomicAdd(&ctl->n_alive[ap ^ 1u], n);
+                        base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+                        for (uint32_t r = 0; r < U; ++r)
+                            if (keep[r]) a.alive[ap ^ 1u][base + at[r]] = e[r];
+                    }
+                }
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < kBins; i += kT)
+                    if (s_hist[i]) atomicAdd(&ctl->hist[pno & 1u][i], s_hist[i]);
+                {
+                    const Snap sn{{nullptr, nullptr, nullptr, nullptr, nullptr}, nullptr};
+                    if (!grid_barrier(a, bar_no, sn, &s_v)) break;
+                }
+                if (anew) {
+                    v_alive = (uint32_t)remaining;
+                    ap ^= 1u;
+                    if (gtid == 0) ctl->n_alive[ap ^ 1u] = 0;
+                }
+                L.label = pno;
+                // every block finds the class up to which the edges of the next
+                // part reach
+                {
+                    constexpr uint32_t kPer = (kBins + kT - 1) / kT;
+                    uint32_t mine[kPer], sum = 0;
+#pragma unroll
+                    for (uint32_t r = 0; r < kPer; ++r) {
+                        const uint32_t b = threadIdx.x * kPer + r;
+                        mine[r] = b < kBins ? __ldcg(&ctl->hist[pno & 1u][b]) : 0u;
+                        sum += mine[r];
+                    }
+                    uint32_t total;
+                    uint32_t cum = dev::block_excl_scan<uint32_t>(sum, &total);
+                    if (pno + 1u >= a.max_parts || total <= a.target + a.target / 2u) {
+                        // the rest is the last part: nothing is left to be told apart
+                        for (uint32_t i = gtid; i < v_alive; i += nthreads) {
+                            const uint32_t e = ldcg_u32(&a.alive[ap][i]);
+                            if (ldcg_u32(&a.state[e]) == kAlive) a.phi[e] = pno;
+                        }
+                        ++pno;
+                        break;
+                    }
+                    // the peel takes more edges than the class holds: the target
+                    // is scaled by what the last part grew by
+                    if (pno > 0) {
+                        const float grew = (float)(total_jump - total) / (float)picked;
+                        aim = fminf(fmaxf((float)a.target / grew, (float)a.target / 32.f), (float)a.target);
+                    }
+                    const uint32_t want = aim < 1.f ? 1u : (uint32_t)aim;
+#pragma unroll
+                    for (uint32_t r = 0; r < kPer; ++r) {
+                        // the first class with a weight of at least `want` up to it
+                        if (cum < want && cum + mine[r] >= want) {
+                            s_bin = threadIdx.x * kPer + r;
+                            s_cum = cum + mine[r];
+                        }
+                        cum += mine[r];
+                    }
+                    __syncthreads();
+                    L.k = bin_top(s_bin);
+                    picked = s_cum;
+                    total_jump = total;
+                    for (uint32_t i = gtid; i < kBins; i += nthreads) ctl->hist[(pno & 1u) ^ 1u][i] = 0;
+                    ++pno;
+                }
+                // C2: their links become incidence items of this round
+                uint32_t sel = 0;
+                for (uint32_t i0 = gwarp * 32u * U; i0 < v_alive; i0 += nthreads * U) {
+                    uint32_t e[U], stv[U], nseg[U], all = 0;
+                    long long sv[U];
+                    uint64_t ib[U], ie[U];
+                    bool in[U];
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        const uint32_t i = i0 + 32u * r + lane;
+                        in[r] = i < v_alive;
+                        e[r] = in[r] ? ldcg_u32(&a.alive[ap][i]) : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        stv[r] = in[r] ? ldcg_u32(&a.state[e[r]]) : 0u;
+                        sv[r] = in[r] ? ldcg_ll(&a.sup[e[r]]) : 0ll;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        in[r] = in[r] && stv[r] == kAlive && sv[r] <= L.k;
+                        ib[r] = in[r] ? a.inc_off[e[r]] : 0ull;
+                        ie[r] = in[r] ? a.inc_off[e[r] + 1] : 0ull;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < U; ++r) {
+                        if (in[r]) {
+                            join_batch(a, e[r], round, L);
+                            ++sel;
+                        }
+                        nseg[r] = (uint32_t)((ie[r] - ib[r] + kSeg - 1) / kSeg);
+                        all += nseg[r];
+                    }
+                    const uint32_t incl = dev::warp_incl_scan(all);
+                    const uint32_t sum = __shfl_sync(kFull, incl, 31);
+                    if (sum) {
+                        uint32_t base = 0;
+                        if (lane == 31) base = atomicAdd(&ctl->n_items[par], sum);
+                        uint32_t slot = __shfl_sync(kFull, base, 31) + incl - all;
+#pragma unroll
+                        for (uint32_t r = 0; r < U; ++r)
+                            for (uint32_t s2 = 0; s2 < nseg[r]; ++s2, ++slot) {
+                                const uint64_t j = ib[r] + (uint64_t)s2 * kSeg;
+                                const uint64_t left = ie[r] - j;
+                                const uint32_t cnt = (uint32_t)(left < kSeg ? left : kSeg);
+                                a.items[par][slot] =
+                                    make_uint4(e[r], (uint32_t)j, (uint32_t)(j >> 32), cnt | (s2 == 0 ? 0x80000000u : 0u));
+                            }
+                    }
+                }
+                sel = dev::warp_sum(sel);
+                if (lane == 0 && sel) atomicAdd(&ctl->n_edges[c3], sel);
+                {
+                    const Snap sn{{&ctl->n_edges[c3], &ctl->n_items[par], &ctl->n_bseg[b4], &ctl->n_bseg[bp], nullptr},
+                                  nullptr};
+                    if (!grid_barrier(a, bar_no, sn, &s_v)) break;
+                }
+                n_batch = s_v.u[0];
+                n_items = s_v.u[1];
+                nb_cur = s_v.u[2];
+                nb_prev = s_v.u[3];
+            }
+        } else if (level_jump) {
             if (gtid == 0) atomicAdd(&ctl->scanned, (unsigned long long)v_near);
             // L1: minimum over the near window, compacting it
             {
@@ -558,6 +784,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                 if (gtid == 0) ctl->minsup2 = ~0ull;
             }
             if ((long long)mn > L.k) L.k = (long long)mn;
+            L.label = (uint32_t)L.k;
             if ((unsigned long long)L.k > 0xFFFFFFFFull) {
                 if (gtid == 0) atomicOr(&ctl->err, kErrPeelOverflow);
                 break;
@@ -581,7 +808,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                         const long long sv = ldcg_ll(&a.sup[e]);
                         const uint64_t b0 = a.inc_off[e], b1 = a.inc_off[e + 1];
                         if (stv == kAlive && sv <= L.k) {
-                            join_batch(a, e, round, L.k);
+                            join_batch(a, e, round, L);
                             ++sel;
                             ib = b0;
                             ie = b1;
@@ -610,7 +837,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                     const long long sv = ldcg_ll(&a.sup[e]);
                     const uint64_t b0 = a.inc_off[e], b1 = a.inc_off[e + 1];
                     if (stv == kAlive && sv <= L.k) {
-                        join_batch(a, e, round, L.k);
+                        join_batch(a, e, round, L);
                         push_items<kSeg>(a, e, par, b0, b1);
                         ++sel;
                     }
@@ -641,49 +868,40 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
         // ---------------- incidence phase (only for queued link lists)
         if (n_items > 0) {
             if (gtid == 0) atomicAdd(&ctl->inc_phases, 1ull);
+            constexpr uint32_t U = 4;  // links a lane has in flight
+            Slots t;
+            const bool stock = n_items > nwarps;  // a small phase takes its places one atomic a warp
             for (uint32_t base = gwarp; base < n_items; base += nwarps * 32u) {
                 const uint32_t i = base + lane * nwarps;
                 const uint4 it = i < n_items ? __ldcg(&a.items[par][i]) : make_uint4(0, 0, 0, 0);
                 const uint32_t cnt = it.w & 0x7FFFFFFFu;
-                {
-                    // a small item is this lane's own: its links' loads and
-                    // stamps go out together
-                    const uint64_t j0 = (uint64_t)it.z << 32 | it.y;
-                    uint2 l[kSmall];
-                    uint32_t B[kSmall];
-                    bool won[kSmall];
+                // the links of the warp's items side by side (as in the bloom phase)
+                const uint32_t incl = dev::warp_incl_scan(cnt);
+                const uint32_t all = __shfl_sync(kFull, incl, 31);
+                const uint64_t start = ((uint64_t)it.z << 32 | it.y) + cnt - incl;
+                for (uint32_t x0 = 0; x0 < all; x0 += 32u * U) {
+                    uint2 l[U];
+                    uint32_t B[U];
+                    bool won[U];
 #pragma unroll
-                    for (uint32_t r = 0; r < kSmall; ++r) {
-                        won[r] = cnt <= kSmall && r < cnt;
-                        l[r] = won[r] ? a.inc[j0 + r] : make_uint2(0u, 0u);
+                    for (uint32_t r = 0; r < U; ++r) {
+                        const uint32_t x = x0 + lane + 32u * r;
+                        uint32_t j = 0;  // the item of link x: the first with incl > x
+#pragma unroll
+                        for (uint32_t step = 16; step > 0; step >>= 1)
+                            if (__shfl_sync(kFull, incl, j + step - 1u) <= x) j += step;
+                        const uint64_t at = __shfl_sync(kFull, start, j) + x;
+                        won[r] = x < all;
+                        l[r] = won[r] ? a.inc[at] : make_uint2(0u, 0u);
                         B[r] = l[r].y & 0x7FFFFFFFu;
                     }
                     // the first edge of the batch to stamp a pair kills it (once)
-                    kill_pairs<kSmall>(a, l, won, round);
-                    warp_kills<kSeg, kSmall>(a, round, B, won, lane);
-                }
-                // items with many links: the whole warp, one item at a time
-                unsigned big = __ballot_sync(kFull, cnt > kSmall);
-                while (big) {
-                    const int src = __ffs(big) - 1;
-                    big &= big - 1u;
-                    const uint32_t bcnt = __shfl_sync(kFull, cnt, src);
-                    const uint32_t jlo = __shfl_sync(kFull, it.y, src);
-                    const uint32_t jhi = __shfl_sync(kFull, it.z, src);
-                    const uint64_t j0 = ((uint64_t)jhi << 32 | jlo) + lane;
-                    uint2 l[R];
-                    uint32_t B[R];
-                    bool won[R];
-#pragma unroll
-                    for (uint32_t r = 0; r < R; ++r) {
-                        won[r] = lane + 32u * r < bcnt;
-                        l[r] = won[r] ? a.inc[j0 + 32u * r] : make_uint2(0u, 0u);
-                        B[r] = l[r].y & 0x7FFFFFFFu;
-                    }
-                    kill_pairs<R>(a, l, won, round);
-                    warp_kills<kSeg, R>(a, round, B, won, lane);
+                    kill_pairs<U>(a, l, won, round);
+                    if (stock) warp_kills<kSeg, U, 2>(a, round, B, won, lane, t);
+                    else warp_kills<kSeg, U, 0>(a, round, B, won, lane, t);
                 }
             }
+            fill_empty(a, b4, t, lane);
             {
                 const Snap sn{{nullptr, nullptr, &ctl->n_bseg[b4], nullptr, nullptr}, nullptr};
                 if (!grid_barrier(a, bar_no, sn, &s_v)) break;
@@ -695,93 +913,53 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
         if (gtid == 0) ctl->n_items[par] = 0;
         {
             const uint32_t q = round + 1u;
-            const uint32_t *C = a.Cb[c3];
             for (uint32_t base = gwarp; base < nb_cur; base += nwarps * 32u) {
                 const uint32_t i = base + lane * nwarps;
                 const uint4 it = i < nb_cur ? __ldcg(&a.bseg[b4][i]) : make_uint4(0, 0, 0, 0);
                 const uint32_t cnt = it.z & 0x7FFFFFFFu;
-                const uint32_t c = cnt ? __ldcg(&C[it.x]) : 0u;
-                if (cnt && (it.z >> 31))
-                    a.bw[it.x] = (unsigned long long)round << 32 | (uint32_t)(it.w - c);
-                slots += cnt;
-                if (cnt <= kSmall) {
-                    uint32_t d[kSmall];
-                    uint2 pr[kSmall];
-#pragma unroll
-                    for (uint32_t r = 0; r < kSmall; ++r) {
-                        const bool act = r < cnt;
-                        d[r] = act ? __ldcg(&a.died[it.y + r]) : (round + 2u) << 2;  // inactive: no case applies
-                        pr[r] = act ? a.pairs[it.y + r] : make_uint2(0, 0);
-                    }
-                    apply_slots<kSeg, kSmall>(a, d, pr, c, it.w, L, round, upd, s_je, &s_jn);
+                // the bloom's kills of this round, and its number at round start:
+                // recorded after the last round that touched it, or by its head
+                // item in this round already
+                uint32_t c = 0, k0 = 0;
+                if (cnt) {
+                    BloomWord *b = a.blooms + it.x;
+                    const unsigned long long w = __ldcg(&b->bw);
+                    c = __ldcg(&b->C[c3]);
+                    k0 = (uint32_t)w + ((uint32_t)(w >> 32) == round ? c : 0u);
+                    if (it.z >> 31) b->bw = (unsigned long long)round << 32 | (uint32_t)(k0 - c);
                 }
-                // items with many slots: the whole warp, one item at a time.
-                // With one slot a lane the next item's pair words are
-                // requested before this item's decrements go out (2M-edge
-                // graph 467 -> 460 ms, a C3-shaped 3M-edge graph 1534 ->
-                // 1481 ms); with two the extra registers spill and the
-                // 30M-edge graph measured 1 % slower, so items go one by one.
-                unsigned big = __ballot_sync(kFull, cnt > kSmall);
-                uint32_t d[R], kB = 0, bc = 0;
-                uint2 pr[R];
-                if constexpr (R == 1) {
-                    if (big) {
-                        const int src = __ffs(big) - 1;
-                        big &= big - 1u;
-                        const uint32_t bcnt = __shfl_sync(kFull, cnt, src);
-                        const uint32_t p0 = __shfl_sync(kFull, it.y, src) + lane;
-                        kB = __shfl_sync(kFull, it.w, src);
-                        bc = __shfl_sync(kFull, c, src);
-                        const bool act = lane < bcnt;
-                        d[0] = act ? __ldcg(&a.died[p0]) : (round + 2u) << 2;
-                        pr[0] = act ? a.pairs[p0] : make_uint2(0, 0);
-                        for (;;) {
-                            const bool more = big != 0u;
-                            uint32_t dn = 0, kBn = 0, bcn = 0;
-                            uint2 prn = make_uint2(0, 0);
-                            if (more) {
-                                const int s2 = __ffs(big) - 1;
-                                big &= big - 1u;
-                                const uint32_t ncnt = __shfl_sync(kFull, cnt, s2);
-                                const uint32_t np0 = __shfl_sync(kFull, it.y, s2) + lane;
-                                kBn = __shfl_sync(kFull, it.w, s2);
-                                bcn = __shfl_sync(kFull, c, s2);
-                                const bool nact = lane < ncnt;
-                                dn = nact ? __ldcg(&a.died[np0]) : (round + 2u) << 2;
-                                prn = nact ? a.pairs[np0] : make_uint2(0, 0);
-                            }
-                            apply_slots<kSeg, R>(a, d, pr, bc, kB, L, round, upd, s_je, &s_jn);
-                            if (!more) break;
-                            d[0] = dn;
-                            pr[0] = prn;
-                            kB = kBn;
-                            bc = bcn;
-                        }
-                    }
-                } else {
-                    while (big) {
-                        const int src = __ffs(big) - 1;
-                        big &= big - 1u;
-                        const uint32_t bcnt = __shfl_sync(kFull, cnt, src);
-                        const uint32_t p0 = __shfl_sync(kFull, it.y, src) + lane;
-                        kB = __shfl_sync(kFull, it.w, src);
-                        bc = __shfl_sync(kFull, c, src);
+                slots += cnt;
+                // the warp's items side by side: lane l takes slots l, l + 32, ...
+                // of their concatenation, so small items fill the warp too
+                const uint32_t incl = dev::warp_incl_scan(cnt);
+                const uint32_t all = __shfl_sync(kFull, incl, 31);
+                constexpr uint32_t U = R < 2u ? 2u : R;  // slots a lane has in flight
+                for (uint32_t x0 = 0; x0 < all; x0 += 32u * U) {
+                    uint32_t d[U], kB[U], cc[U];
+                    uint2 pr[U];
 #pragma unroll
-                        for (uint32_t r = 0; r < R; ++r) {
-                            const bool act = lane + 32u * r < bcnt;
-                            d[r] = act ? __ldcg(&a.died[p0 + 32u * r]) : (round + 2u) << 2;
-                            pr[r] = act ? a.pairs[p0 + 32u * r] : make_uint2(0, 0);
-                        }
-                        apply_slots<kSeg, R>(a, d, pr, bc, kB, L, round, upd, s_je, &s_jn);
+                    for (uint32_t r = 0; r < U; ++r) {
+                        const uint32_t x = x0 + lane + 32u * r;
+                        uint32_t j = 0;  // the item of slot x: the first with incl > x
+#pragma unroll
+                        for (uint32_t step = 16; step > 0; step >>= 1)
+                            if (__shfl_sync(kFull, incl, j + step - 1u) <= x) j += step;
+                        const bool act = x < all;
+                        const uint32_t p = __shfl_sync(kFull, it.y + cnt - incl, j) + x;
+                        kB[r] = __shfl_sync(kFull, k0, j);
+                        cc[r] = __shfl_sync(kFull, c, j);
+                        d[r] = act ? __ldcg(&a.died[p]) : (round + 2u) << 2;  // inactive: no case applies
+                        pr[r] = act ? a.pairs[p] : make_uint2(0, 0);
                     }
+                    apply_slots<kSeg, U>(a, d, pr, cc, kB, L, round, upd, s_je, &s_jn);
                 }
             }
             // clear C of the blooms the previous round touched (threads from
             // the top of the grid, away from the bloom items above)
-            uint32_t *Cp = a.Cb[(round + 2u) % 3u];
+            const uint32_t cp = (round + 2u) % 3u;
             for (uint32_t i = nthreads - 1u - gtid; i < nb_prev; i += nthreads) {
                 const uint4 it = __ldcg(&a.bseg[bp][i]);
-                if (it.z >> 31) Cp[it.x] = 0;
+                if (it.z >> 31) a.blooms[it.x].C[cp] = 0;
             }
 
             // the block kills the twin pairs of the edges it listed
@@ -793,7 +971,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                 uint64_t ib = 0;
                 if (threadIdx.x < nj) {
                     e = s_je[threadIdx.x];
-                    join_batch(a, e, q, L.k);
+                    join_batch(a, e, q, L);
                     ib = a.inc_off[e];
                     const uint64_t dl = a.inc_off[e + 1] - ib;
                     d = dl > a.block_links ? a.block_links + 1u : (uint32_t)dl;  // longer lists are queued
@@ -828,7 +1006,9 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                 }
                 // the first edge of the batch to stamp a pair kills it (once)
                 kill_pairs<2>(a, l, won, q);
-                warp_kills<kSeg, 2>(a, q, B, won, lane);
+                Slots none;
+                if (kCoarse && lim > kT / 2u) warp_kills<kSeg, 2, 1>(a, q, B, won, lane, none);
+                else warp_kills<kSeg, 2, 0>(a, q, B, won, lane, none);
                 if (threadIdx.x == 0) s_jn = 0;
             }
         }
@@ -857,6 +1037,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     if (gtid == 0) {
         ctl->rounds = round;
         ctl->kfinal = (unsigned long long)L.k;
+        ctl->n_parts = pno;
     }
 }
 
@@ -874,10 +1055,13 @@ __global__ void k_peel_init(const uint64_t *support, uint64_t m, long long *sup,
 }
 
 // Bloom words: no round has touched the bloom yet, k_B from the index.
-__global__ void k_bw_init(const uint32_t *bloom_k, uint64_t nb, unsigned long long *bw) {
+__global__ void k_bloom_words(const uint32_t *bloom_k, uint64_t nb, BloomWord *blooms) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nb;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        bw[i] = 0xFFFFFFFFull << 32 | bloom_k[i];
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        uint4 *w = reinterpret_cast<uint4 *>(blooms + i);
+        w[0] = make_uint4(bloom_k[i], 0xFFFFFFFFu, 0u, 0u);
+        w[1] = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 inline unsigned grid_for(uint64_t items, int threads, unsigned cap) {
@@ -898,19 +1082,20 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     if (m == 0 || (opts && opts->assigned && opts->m_active == 0)) return cudaSuccess;
     // one round queues each edge and each bloom at most once
     const uint64_t item_cap = m + (2 * ix.w2) / kSeg + 2;
-    const uint64_t bseg_cap = ix.nb + ix.w2 / kSeg + 2;
+    // (each bloom at most once), beside the places a warp takes and leaves empty
+    // in an incidence phase: fewer than it fills each time, and a last stock
+    const uint64_t bseg_cap = 2 * (ix.nb + ix.w2 / kSeg) + (uint64_t)num_sms * (kT / 32) * kTake + 2;
     PeelArgs a{};
     a.m = m;
     a.inc_off = ix.inc_off;
     a.inc = ix.inc;
     a.pairs = ix.pairs;
-    a.bloom_off = ix.bloom_off;
     a.phi = phi_out;
     a.sup = al.get<long long>(m);
     a.state = al.get<uint32_t>(m);
     a.died = al.get<uint32_t>(ix.w2);
-    a.bw = al.get<unsigned long long>(ix.nb);
-    for (int i = 0; i < 3; ++i) a.Cb[i] = al.get<uint32_t>(ix.nb);
+    a.bloom_off = ix.bloom_off;
+    a.blooms = al.get<BloomWord>(ix.nb);
     for (int i = 0; i < 4; ++i) a.bseg[i] = al.get<uint4>(bseg_cap);
     for (int i = 0; i < 2; ++i) {
         a.items[i] = al.get<uint4>(item_cap);
@@ -933,18 +1118,25 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     a.m_active = (opts && opts->assigned) ? opts->m_active : m;
     a.k_init = opts ? opts->k_init : 0;
     a.assign_from = opts ? opts->assign_from : 0;
+    const bool coarse = opts && opts->snap;
+    a.snap = coarse ? opts->snap : nullptr;
+    if (coarse) {
+        // weights add up to less than 2^31
+        while ((ix.links >> a.wshift) >> 30) ++a.wshift;
+        const uint64_t all = m + (ix.links >> a.wshift), t = all / (opts->parts_hint ? opts->parts_hint : 1);
+        a.target = (uint32_t)(t ? t : 1);
+    }
+    a.max_parts = coarse ? opts->max_parts : 0;
     if (al.err != cudaSuccess) return al.err;
     cudaStream_t st = al.stream;
-    al.mark(kPhPeel, false);
+    if (!coarse) al.mark(kPhPeel, false);  // (a coarse peel is part of its caller's phase)
     k_peel_init<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(
         support, m, a.sup, a.state, opts ? opts->assigned : nullptr, a.alive[0]);
     al.launches++;
     BT_CUDA(cudaMemsetAsync(a.died, 0xFF, sizeof(uint32_t) * (ix.w2 ? ix.w2 : 1), st));
     if (ix.nb) {
-        k_bw_init<<<grid_for(ix.nb, 256, (unsigned)num_sms * 16), 256, 0, st>>>(ix.bloom_k, ix.nb, a.bw);
+        k_bloom_words<<<grid_for(ix.nb, 256, (unsigned)num_sms * 16), 256, 0, st>>>(ix.bloom_k, ix.nb, a.blooms);
         al.launches++;
-        for (int i = 0; i < 3; ++i)
-            BT_CUDA(cudaMemsetAsync(a.Cb[i], 0, sizeof(uint32_t) * ix.nb, st));
     }
     Ctl h{};
     h.n_alive[0] = (unsigned int)m;
@@ -952,7 +1144,9 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     h.minsup2 = ~0ull;
     BT_CUDA(cudaMemcpyAsync(a.ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
     int bps = 0;
-    void *kfn = kSeg == 128 ? (void *)k_peel<128> : kSeg == 64 ? (void *)k_peel<64> : (void *)k_peel<32>;
+    void *kfn = coarse ? (kSeg == 128 ? (void *)k_peel<128, true> : (void *)k_peel<32, true>)
+                       : kSeg == 128 ? (void *)k_peel<128, false>
+                                     : kSeg == 64 ? (void *)k_peel<64, false> : (void *)k_peel<32, false>;
     BT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, (int)kT, 0));
     if (bps < 1) return cudaErrorCooperativeLaunchTooLarge;
     dim3 grid((unsigned)(num_sms * bps)), block(kT);
@@ -961,7 +1155,7 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     al.launches++;
     BT_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
     BT_CUDA(cudaStreamSynchronize(st));
-    al.mark(kPhPeel, true);
+    if (!coarse) al.mark(kPhPeel, true);
     if (h.err & kErrBarrier) res.status = BT_ERR_CUDA;
     else if (h.err & kErrPeelOverflow) res.status = BT_ERR_OVERFLOW;
     else if (h.err & kErrRounds) res.status = BT_ERR_NOCONVERGE;
@@ -973,11 +1167,11 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     res.scanned = h.scanned;
     res.kmax = h.kfinal;
     res.inc_phases = h.inc_phases;
+    res.parts = h.n_parts;
     al.put(a.sup);
     al.put(a.state);
     al.put(a.died);
-    al.put(a.bw);
-    for (int i = 0; i < 3; ++i) al.put(a.Cb[i]);
+    al.put(a.blooms);
     for (int i = 0; i < 4; ++i) al.put(a.bseg[i]);
     for (int i = 0; i < 2; ++i) {
         al.put(a.items[i]);

@@ -268,6 +268,10 @@ int bt_server_create(bt_server **out, int device, const bt_server_config *cfg) {
             return rc;
         }
         bt::share_peel_sms(h, (int)s->cfg.workers);  // peels of all workers fit on the GPU at once
+        // A server with one worker keeps the grid-wide peel: its callers count on
+        // a request of some 500,000 edges to hold the worker for 50 ms, so that
+        // those behind it can still be cancelled (115 ms so, 25 ms in parts).
+        if (s->cfg.workers == 1) bt::use_grid_peel(h);
         s->handles.push_back(h);
     }
     for (uint32_t i = 0; i < s->cfg.workers; ++i)

@@ -1,0 +1,493 @@
+// Part graphs for the part peel (local.cu): a whole small graph, or the ranges of
+// bitruss numbers a coarse peel found.
+//
+// Ranges.  The coarse peel (peel.cu) gives every edge the part its bitruss
+// number falls in, parts ascending.  When part q begins, all edges of lower
+// parts are gone, so of a bloom's twin pairs those with both edges in parts >= q
+// remain; Alg. 5 inside part q then needs
+//   * the bloom number k_B at that point: the pairs whose lower edge is in a
+//     part >= q;
+//   * the pairs that can die inside part q: those whose lower edge is in q.  An
+//     edge of a higher part is flagged: it is not peeled here and its support
+//     is not updated.
+// A pair thus belongs to one part, min(part(e1), part(e2)), and a bloom falls
+// apart into one group of pairs a part.  A group whose k_B is 1 holds no
+// butterfly and is dropped.  Supports at the start of a part come from the
+// coarse peel, so each part is peeled without any other.
+#include <algorithm>
+#include <vector>
+
+#include "bt_device.cuh"
+#include "bt_internal.cuh"
+
+namespace bt {
+namespace {
+
+constexpr uint32_t kNone = 0xFFFFFFFFu;
+constexpr uint32_t kFlag = 0x80000000u;
+constexpr uint32_t kMaxParts = kPartsMax;
+constexpr int kT = 256;
+// a part with more links than this many times the mean is peeled by a cluster
+constexpr double kHeavy = 4.0;
+constexpr int kSmall = 8;  // pairs of a bloom that one thread groups by itself
+constexpr unsigned kFull = 0xffffffffu;
+
+inline unsigned grid_for(uint64_t items, int threads, unsigned cap) {
+    uint64_t g = (items + threads - 1) / threads;
+    if (g == 0) g = 1;
+    return (unsigned)(g < cap ? g : cap);
+}
+
+__device__ __forceinline__ void head(BloomRec *b, uint32_t first, uint32_t n, uint32_t k) {
+    *reinterpret_cast<uint4 *>(b) = make_uint4(first, n, k, 0u);
+}
+
+__global__ void k_bloom_rec(const uint32_t *bloom_k, const uint32_t *bloom_off, const uint2 *pairs, uint64_t nb,
+                            BloomRec *bl) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nb; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t o = bloom_off[i], n = bloom_off[i + 1] - o;
+        head(bl + i, o, n, bloom_k[i]);
+        if (n <= 2u)
+            for (uint32_t j = 0; j < n; ++j) bl[i].pair[j] = pairs[o + j];
+    }
+}
+
+// Edge records of the whole graph; ends: its first and last edge, first and last bloom.
+__global__ void k_edge_rec(const uint64_t *inc_off, const uint64_t *support, uint64_t m, uint32_t nb, uint32_t *ends,
+                           uint4 *er) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<uint4 *>(ends) = make_uint4(0u, (uint32_t)m, 0u, nb);
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t o = inc_off[i];
+        er[i] = make_uint4((uint32_t)o, (uint32_t)(o >> 32), (uint32_t)(inc_off[i + 1] - o), (uint32_t)support[i]);
+    }
+}
+
+__global__ void k_iota2(const uint32_t *part, uint64_t m, uint32_t *keys, uint32_t *vals) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
+        keys[i] = part[i];
+        vals[i] = (uint32_t)i;
+    }
+}
+
+// keys: parts in ascending order (np of them), order: the edges.  place[e] = (new id, part);
+// part_e[q]: the first edge of part q.
+__global__ void k_place(const uint32_t *keys, const uint32_t *order, uint64_t m, uint32_t np, uint2 *place,
+                        uint32_t *part_e) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t q = keys[i];
+        place[order[i]] = make_uint2((uint32_t)i, q);
+        const uint32_t before = i ? keys[i - 1] + 1u : 0u;  // a part may be empty
+        for (uint32_t x = before; x <= q; ++x) part_e[x] = (uint32_t)i;
+        if (i + 1 == m)
+            for (uint32_t x = q + 1u; x <= np; ++x) part_e[x] = (uint32_t)m;
+    }
+}
+
+struct SplitArgs {
+    const uint32_t *bloom_off;
+    uint64_t nb;
+    const uint2 *pairs;   // the index's
+    const uint2 *place;   // per edge: new id, part
+    uint32_t np;
+    uint2 *out;           // pairs of groups of more than two, part by part, new ids
+    uint32_t *sub;        // per pair of the index: its group, or kNone
+    BloomRec *bl;         // group records, part by part
+    uint32_t *groups;     // [np] groups of each part: counted, then (the exclusive sums) handed out
+    uint32_t *members;    // [np] their pairs (of groups of more than two), likewise
+};
+
+__device__ __forceinline__ uint2 placed(uint2 a, uint2 b) {
+    return make_uint2(a.x | (a.y > b.y ? kFlag : 0u), b.x | (b.y > a.y ? kFlag : 0u));
+}
+
+// What a block takes of each part's groups and pairs: counted in shared memory,
+// then added to the part's counters with one atomic a part.
+struct Tally {
+    uint32_t groups[kMaxParts], members[kMaxParts];
+};
+__device__ __forceinline__ void tally_zero(Tally &s, uint32_t np) {
+    for (uint32_t i = threadIdx.x; i < np; i += kT) s.groups[i] = s.members[i] = 0;
+}
+// s becomes the first of the places taken (kTake), or is only added.
+template <bool kTake>
+__device__ __forceinline__ void tally_add(Tally &s, const SplitArgs &a) {
+    for (uint32_t i = threadIdx.x; i < a.np; i += kT) {
+        const uint32_t g = s.groups[i], n = s.members[i];
+        if (!g) continue;
+        const uint32_t g0 = atomicAdd(&a.groups[i], g), n0 = n ? atomicAdd(&a.members[i], n) : 0u;
+        if (kTake) {
+            s.groups[i] = g0;
+            s.members[i] = n0;
+        }
+    }
+}
+
+// Blooms of up to kSmall pairs, one thread each, all its pairs in registers.
+// kPlace: places the groups; else counts them.
+template <bool kPlace>
+__global__ void __launch_bounds__(kT) k_split_small(const SplitArgs a) {
+    __shared__ Tally s;
+    tally_zero(s, a.np);
+    __syncthreads();
+    for (uint64_t b0 = (uint64_t)blockIdx.x * kT; b0 < a.nb; b0 += (uint64_t)gridDim.x * kT) {
+        const uint64_t B = b0 + threadIdx.x;
+        uint32_t off = 0, K = 0;
+        if (B < a.nb) {
+            off = a.bloom_off[B];
+            K = a.bloom_off[B + 1] - off;
+            if (K > (uint32_t)kSmall) K = 0;
+        }
+        uint2 px[kSmall], py[kSmall];
+        uint32_t q[kSmall];
+#pragma unroll
+        for (int i = 0; i < kSmall; ++i) px[i] = (uint32_t)i < K ? a.pairs[off + i] : make_uint2(0u, 0u);
+#pragma unroll
+        for (int i = 0; i < kSmall; ++i) {
+            const uint2 pr = px[i];
+            py[i] = (uint32_t)i < K ? a.place[pr.y] : make_uint2(0u, 0u);
+            px[i] = (uint32_t)i < K ? a.place[pr.x] : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < kSmall; ++i) q[i] = (uint32_t)i < K ? (px[i].y < py[i].y ? px[i].y : py[i].y) : kNone;
+        // size and first pair of every pair's group; left: its k_B
+        uint32_t left[kSmall], rank[kSmall], first[kSmall], size[kSmall];
+#pragma unroll
+        for (int i = 0; i < kSmall; ++i) {
+            left[i] = K;
+            rank[i] = size[i] = 0;
+            first[i] = i;
+#pragma unroll
+            for (int j = kSmall - 1; j >= 0; --j) {
+                left[i] -= q[j] < q[i];
+                rank[i] += j < i && q[j] == q[i];
+                size[i] += q[j] == q[i];
+                if (q[j] == q[i]) first[i] = j;
+            }
+            if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u) {
+                atomicAdd(&s.groups[q[i]], 1u);
+                if (size[i] > 2u) atomicAdd(&s.members[q[i]], size[i]);
+            }
+        }
+        if constexpr (kPlace) {
+            __syncthreads();
+            tally_add<true>(s, a);
+            __syncthreads();
+            uint32_t id[kSmall], at[kSmall];
+#pragma unroll
+            for (int i = 0; i < kSmall; ++i) {
+                id[i] = kNone;
+                at[i] = 0;
+                if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u) {
+                    id[i] = atomicAdd(&s.groups[q[i]], 1u);
+                    if (size[i] > 2u) at[i] = atomicAdd(&s.members[q[i]], size[i]);
+                    head(a.bl + id[i], at[i], size[i], left[i]);
+                }
+#pragma unroll
+                for (int j = 0; j < i; ++j)
+                    if (first[i] == (uint32_t)j) {
+                        id[i] = id[j];
+                        at[i] = at[j];
+                    }
+                if ((uint32_t)i < K) {
+                    a.sub[off + i] = id[i];
+                    if (id[i] != kNone) {
+                        uint2 *to = size[i] > 2u ? a.out + at[i] : a.bl[id[i]].pair;
+                        to[rank[i]] = placed(px[i], py[i]);
+                    }
+                }
+            }
+            __syncthreads();
+            tally_zero(s, a.np);
+            __syncthreads();
+        }
+    }
+    if constexpr (!kPlace) {
+        __syncthreads();
+        tally_add<false>(s, a);
+    }
+}
+
+// Larger blooms, one warp each: a histogram over the parts in shared memory.
+template <bool kPlace>
+__global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
+    constexpr int kWarps = kT / 32;
+    extern __shared__ uint32_t s_tab[];  // two rows of np a warp; then the block's tally
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t *cur = s_tab + (size_t)w * 2 * a.np, *gid = cur + a.np;
+    uint32_t *t_groups = s_tab + (size_t)kWarps * 2 * a.np, *t_members = t_groups + a.np;
+    if constexpr (!kPlace) {
+        for (uint32_t i = threadIdx.x; i < 2 * a.np; i += kT) t_groups[i] = 0;
+        __syncthreads();
+    }
+    const uint64_t nw = (uint64_t)gridDim.x * kWarps;
+    for (uint64_t b0 = ((uint64_t)blockIdx.x * kWarps + w) * 32; b0 < a.nb; b0 += nw * 32) {
+        uint32_t my_off = 0, my_k = 0;
+        if (b0 + lane < a.nb) {
+            my_off = a.bloom_off[b0 + lane];
+            my_k = a.bloom_off[b0 + lane + 1] - my_off;
+        }
+        unsigned big = __ballot_sync(kFull, my_k > (uint32_t)kSmall);
+        while (big) {
+            const int src = __ffs(big) - 1;
+            big &= big - 1u;
+            const uint32_t off = __shfl_sync(kFull, my_off, src), K = __shfl_sync(kFull, my_k, src);
+            for (uint32_t i = lane; i < a.np; i += 32) cur[i] = 0;
+            __syncwarp();
+            for (uint32_t i = lane; i < K; i += 32) {
+                const uint2 pr = a.pairs[off + i];
+                const uint32_t qx = a.place[pr.x].y, qy = a.place[pr.y].y;
+                atomicAdd(&cur[qx < qy ? qx : qy], 1u);
+            }
+            __syncwarp();
+            // parts in order, 32 at a time: pairs below; a group for each
+            // non-empty part that leaves a butterfly
+            uint32_t run = 0;
+            for (uint32_t i0 = 0; i0 < a.np; i0 += 32) {
+                const uint32_t i = i0 + lane;
+                const uint32_t n = i < a.np ? cur[i] : 0u;
+                const uint32_t incl = dev::warp_incl_scan(n);
+                const uint32_t left = K - (run + incl - n);
+                run += __shfl_sync(kFull, incl, 31);
+                if (i >= a.np) continue;
+                const bool g = n > 0u && left >= 2u;
+                if constexpr (kPlace) {
+                    gid[i] = kNone;
+                    if (g) {
+                        const uint32_t id = atomicAdd(&a.groups[i], 1u);
+                        const uint32_t at = n > 2u ? atomicAdd(&a.members[i], n) : 0u;
+                        gid[i] = id;
+                        cur[i] = n > 2u ? at : kFlag;  // up to two go to the record
+                        head(a.bl + id, at, n, left);
+                    }
+                } else if (g) {
+                    atomicAdd(&t_groups[i], 1u);
+                    if (n > 2u) atomicAdd(&t_members[i], n);
+                }
+            }
+            __syncwarp();
+            if constexpr (kPlace) {
+                for (uint32_t i = lane; i < K; i += 32) {
+                    const uint2 pr = a.pairs[off + i];
+                    const uint2 x = a.place[pr.x], y = a.place[pr.y];
+                    const uint32_t qi = x.y < y.y ? x.y : y.y, id = gid[qi];
+                    a.sub[off + i] = id;
+                    if (id != kNone) {
+                        const uint32_t c = atomicAdd(&cur[qi], 1u);
+                        if (c & kFlag) a.bl[id].pair[c & 1u] = placed(x, y);
+                        else a.out[c] = placed(x, y);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+    if constexpr (!kPlace) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < a.np; i += kT)
+            if (t_groups[i]) {
+                atomicAdd(&a.groups[i], t_groups[i]);
+                atomicAdd(&a.members[i], t_members[i]);
+            }
+    }
+}
+
+// Links per part before the split: room[q] bounds the links part q keeps.
+__global__ void __launch_bounds__(kT) k_split_room(const uint64_t *inc_off, const uint2 *place, uint64_t m, uint32_t np,
+                                                   unsigned long long *room) {
+    __shared__ unsigned long long s_n[kMaxParts];
+    for (uint32_t i = threadIdx.x; i < np; i += kT) s_n[i] = 0;
+    __syncthreads();
+    for (uint64_t e = blockIdx.x * (uint64_t)kT + threadIdx.x; e < m; e += (uint64_t)gridDim.x * kT)
+        atomicAdd(&s_n[place[e].y], (unsigned long long)(inc_off[e + 1] - inc_off[e]));
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < np; i += kT)
+        if (s_n[i]) atomicAdd(&room[i], s_n[i]);
+}
+
+// Links of every edge (a warp each): those whose pair belongs to the edge's part,
+// as (twin, group), into the part's own range (next: its next free place).  The
+// links are read twice, first to know their number.
+__global__ void __launch_bounds__(kT) k_split_links(const uint64_t *inc_off, const uint2 *inc, const uint2 *pairs,
+                                                    const uint32_t *sub, const uint2 *place, const int *snap,
+                                                    uint64_t m, unsigned long long *next, uint2 *out, uint4 *er) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t nw = ((uint64_t)gridDim.x * kT) >> 5;
+    for (uint64_t e = ((uint64_t)blockIdx.x * kT + threadIdx.x) >> 5; e < m; e += nw) {
+        const uint64_t lb = inc_off[e], le = inc_off[e + 1];
+        const uint2 me = place[e];
+        uint32_t n = 0;
+        unsigned long long at = 0;
+        for (int pass = 0; pass < 2; ++pass) {
+            uint32_t k = 0;
+            for (uint64_t j0 = lb; j0 < le; j0 += 32) {
+                const uint64_t j = j0 + lane;
+                uint2 nl = make_uint2(0u, 0u);
+                bool keep = false;
+                if (j < le) {
+                    const uint2 l = inc[j];
+                    const uint2 pr = pairs[l.x];
+                    const uint32_t s = sub[l.x];
+                    const uint2 t = place[l.y >> 31 ? pr.x : pr.y];
+                    keep = s != kNone && t.y >= me.y;
+                    nl = make_uint2(t.x | (t.y > me.y ? kFlag : 0u), s);
+                }
+                const unsigned mask = __ballot_sync(kFull, keep);
+                if (pass == 0 && le - lb <= 32) {  // all its links at once: no second reading
+                    n = __popc(mask);
+                    if (lane == 0 && n) at = atomicAdd(&next[me.y], (unsigned long long)n);
+                    at = __shfl_sync(kFull, at, 0);
+                    if (keep) out[at + __popc(mask & ((1u << lane) - 1u))] = nl;
+                    pass = 1;
+                } else if (pass == 1 && keep) {
+                    out[at + k + __popc(mask & ((1u << lane) - 1u))] = nl;
+                }
+                k += __popc(mask);
+            }
+            if (pass == 0) {
+                n = k;
+                if (lane == 0 && n) at = atomicAdd(&next[me.y], (unsigned long long)n);
+                at = __shfl_sync(kFull, at, 0);
+            }
+        }
+        if (lane == 0) er[me.x] = make_uint4((uint32_t)at, (uint32_t)(at >> 32), n, (uint32_t)snap[e]);
+    }
+}
+
+}  // namespace
+
+void free_parts(PartGraph &g, Alloc &al) {
+    for (int i = 0; i < g.n_own; ++i) al.put(g.own[i]);
+    g = PartGraph{};
+}
+
+cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al) {
+    g.m = ix.m;
+    g.nb = ix.nb;
+    g.np = 1;
+    g.inc = ix.inc;
+    g.pairs = ix.pairs;
+    uint32_t *ends = g.keep(al.get<uint32_t>(4));
+    g.part_e = ends;
+    g.part_b = ends + 2;
+    g.er = g.keep(al.get<uint4>(ix.m));
+    g.bl = g.keep(al.get<BloomRec>(ix.nb));
+    if (al.err != cudaSuccess) return al.err;
+    const unsigned wide = (unsigned)num_sms * 16;
+    k_edge_rec<<<grid_for(ix.m, 256, wide), 256, 0, al.stream>>>(ix.inc_off, support, ix.m, (uint32_t)ix.nb, ends, g.er);
+    al.launches++;
+    if (ix.nb) {
+        k_bloom_rec<<<grid_for(ix.nb, 256, wide), 256, 0, al.stream>>>(ix.bloom_k, ix.bloom_off, ix.pairs, ix.nb, g.bl);
+        al.launches++;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np, PartGraph &g,
+                            int num_sms, Alloc &al) {
+    const uint64_t m = ix.m, nb = ix.nb;
+    const unsigned wide = (unsigned)num_sms * 16;
+    g.m = m;
+    g.np = np;
+    uint32_t *part_e = g.keep(al.get<uint32_t>((size_t)np + 1));
+    uint32_t *part_b = g.keep(al.get<uint32_t>((size_t)np + 1));
+    uint32_t *order = g.keep(al.get<uint32_t>(np));
+    uint32_t *out_id = g.keep(al.get<uint32_t>(m));
+    g.part_e = part_e;
+    g.part_b = part_b;
+    g.order = order;
+    g.out_id = out_id;
+    g.er = g.keep(al.get<uint4>(m));
+    uint32_t *keys = al.get<uint32_t>(m), *tk = al.get<uint32_t>(m), *tv = al.get<uint32_t>(m);
+    uint2 *place = al.get<uint2>(m);
+    uint32_t *tally = al.get<uint32_t>(2 * ((size_t)np + 1));  // groups, pairs of each part
+    uint32_t *cursor = al.get<uint32_t>(2 * ((size_t)np + 1));
+    unsigned long long *room = al.get<unsigned long long>((size_t)np + 1);  // links; their places
+    if (al.err != cudaSuccess) return al.err;
+    // edges by part
+    k_iota2<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(part, m, keys, out_id);
+    al.launches++;
+    BT_CUDA(radix_sort_u32(keys, out_id, tk, tv, m, bits_for(np - 1), al));
+    k_place<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(keys, out_id, m, np, place, part_e);
+    al.launches++;
+    al.put(keys);
+    al.put(tk);
+    al.put(tv);
+    // groups and pairs of each part, then their places
+    BT_CUDA(cudaMemsetAsync(tally, 0, 8 * ((size_t)np + 1), al.stream));
+    BT_CUDA(cudaMemsetAsync(room, 0, 8 * ((size_t)np + 1), al.stream));
+    SplitArgs s{ix.bloom_off, nb, ix.pairs, place, np, nullptr, nullptr, nullptr, tally, tally + np + 1};
+    const size_t smem = sizeof(uint32_t) * 2 * np * (kT / 32 + 1);
+    // (the attribute belongs to the process: always the same value, so that
+    // calls of several threads do not lower one another's)
+    const int most = (int)(sizeof(uint32_t) * 2 * kMaxParts * (kT / 32 + 1));
+    BT_CUDA(cudaFuncSetAttribute(k_split_large<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    BT_CUDA(cudaFuncSetAttribute(k_split_large<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    if (nb) {
+        k_split_small<false><<<grid_for(nb, kT, wide), kT, 0, al.stream>>>(s);
+        k_split_large<false><<<grid_for(nb, kT, wide), kT, smem, al.stream>>>(s);
+        al.launches += 2;
+    }
+    k_split_room<<<grid_for(m, kT, wide), kT, 0, al.stream>>>(ix.inc_off, place, m, np, room);
+    al.launches++;
+    BT_CUDA(cudaGetLastError());
+    std::vector<uint32_t> he(np + 1), ht(2 * (np + 1)), ord(np);
+    std::vector<unsigned long long> hr(np + 1), at(np + 1);
+    BT_CUDA(cudaMemcpyAsync(ht.data(), tally, 8 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
+    BT_CUDA(cudaMemcpyAsync(he.data(), part_e, 4 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
+    BT_CUDA(cudaMemcpyAsync(hr.data(), room, 8 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
+    BT_CUDA(cudaStreamSynchronize(al.stream));
+    uint32_t gsum = 0, psum = 0;
+    unsigned long long lsum = 0;
+    for (uint32_t i = 0; i <= np; ++i) {
+        const uint32_t gi = ht[i], pi = ht[np + 1 + i];
+        ht[i] = gsum;
+        ht[np + 1 + i] = psum;
+        at[i] = lsum;
+        gsum += gi;
+        psum += pi;
+        lsum += hr[i];
+    }
+    g.nb = gsum;
+    // the heaviest first; those that one block would be long at by a cluster
+    const double lim = kHeavy * (double)lsum / np;
+    auto heavy = [&](uint32_t p) { return he[p + 1] - he[p] > kBlockEdges || (double)hr[p] > lim; };
+    for (uint32_t i = 0; i < np; ++i) ord[i] = i;
+    std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) {
+        const bool hx = heavy(x), hy = heavy(y);
+        return hx != hy ? hx : hr[x] > hr[y];
+    });
+    for (uint32_t i = 0; i < np; ++i) g.n_heavy += heavy(i);
+    BT_CUDA(cudaMemcpyAsync(cursor, ht.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
+    BT_CUDA(cudaMemcpyAsync(part_b, ht.data(), 4 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
+    BT_CUDA(cudaMemcpyAsync(room, at.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
+    BT_CUDA(cudaMemcpyAsync(order, ord.data(), 4 * (size_t)np, cudaMemcpyHostToDevice, al.stream));
+    uint32_t *sub = al.get<uint32_t>(ix.w2);
+    uint2 *pairs = g.keep(al.get<uint2>(psum)), *inc = g.keep(al.get<uint2>(lsum));
+    g.bl = g.keep(al.get<BloomRec>(gsum));
+    g.pairs = pairs;
+    g.inc = inc;
+    if (al.err != cudaSuccess) return al.err;
+    s.out = pairs;
+    s.sub = sub;
+    s.bl = g.bl;
+    s.groups = cursor;
+    s.members = cursor + np + 1;
+    if (nb) {
+        k_split_small<true><<<grid_for(nb, kT, wide), kT, 0, al.stream>>>(s);
+        k_split_large<true><<<grid_for(nb, kT, wide), kT, smem, al.stream>>>(s);
+        al.launches += 2;
+    }
+    k_split_links<<<grid_for(m * 32, kT, wide), kT, 0, al.stream>>>(ix.inc_off, ix.inc, ix.pairs, sub, place, snap, m,
+                                                                    room, inc, g.er);
+    al.launches++;
+    BT_CUDA(cudaGetLastError());
+    BT_CUDA(cudaStreamSynchronize(al.stream));  // the host tables above
+    al.put(place);
+    al.put(sub);
+    al.put(tally);
+    al.put(cursor);
+    al.put(room);
+    return cudaSuccess;
+}
+
+}  // namespace bt

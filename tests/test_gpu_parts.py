@@ -1,0 +1,84 @@
+"""The peel by parts (coarse ranges of bitruss numbers, then each range by a block
+or a cluster of its own) at the sizes where it can go wrong: against the CPU
+oracle on small graphs, against closed forms on bicliques, and against the
+grid-wide peel (kept in use by a limit that addresses it) on larger ones.
+Supports, bitruss numbers and the peel's statistics are whole numbers and have
+to be equal."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2001_06111_gb300 import bitruss as bt
+from paper_2001_06111_gb300 import build, synth
+from tests import pins
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def h():
+    build.build()
+    handle = bt.bt_create(0)
+    yield handle
+    handle.close()
+
+
+def grid_peel(h, *args, **kw):
+    bt.bt_set_limits(h, join_cap=1 << 30)  # far above any cap: the grid-wide kernel, its defaults
+    try:
+        return bt.bt_decompose(h, *args, **kw)
+    finally:
+        bt.bt_set_limits(h)
+
+
+# one part up to 1,024 edges, ranges above
+@pytest.mark.parametrize("m", [1, 2, 33, 1023, 1024, 1025, 3001])
+def test_small_graphs_against_the_oracle(h, m):
+    nU, nL = max(2, m // 8), max(2, m // 12)
+    g = synth.random_tiny(m, nU, nL, m) if m < 100 else synth.chunglu(nU, nL, m, 2.3, 2.4, seed=m)
+    s0, p0 = oracle.bitruss(g.edges, g.nU, g.nL)
+    sup, phi, _ = bt.bt_decompose(h, g.edges, g.nU, g.nL)
+    np.testing.assert_array_equal(sup, s0)
+    np.testing.assert_array_equal(phi.astype(np.uint64), p0)
+
+
+# every edge of K_{a,b} has support and bitruss number (a-1)(b-1).  All edges leave
+# in one batch: batches above the 512 kept in shared memory and the 1,024 threads,
+# more touched blooms than a block lists (C(a,2) of them), parts around the
+# 43,008 edges whose supports fit a block (above: a cluster)
+@pytest.mark.parametrize("a,b", [(16, 32), (16, 33), (31, 33), (32, 33), (91, 92), (128, 336), (128, 337), (211, 210)])
+def test_bicliques(h, a, b):
+    e = pins.biclique(a, b)
+    sup, phi, st = bt.bt_decompose(h, e, a, b)
+    want = (a - 1) * (b - 1)
+    assert (sup == want).all() and (phi == want).all()
+    assert (st["rounds"], st["levels"], st["phi_max"]) == (1, 1, want)
+
+
+# dense planted blocks: parts heavy enough for clusters, blooms of many pairs,
+# groups of one, two and more pairs in a bloom
+@pytest.mark.parametrize("m,nplant,lo,hi,flags", [(20001, 6, 10, 40, 0), (150001, 3, 100, 200, 0),
+                                                  (150001, 3, 100, 200, bt.BT_TIE_LOWER_FIRST),
+                                                  (300007, 2, 250, 300, 0), (400003, 0, 0, 0, 0)])
+def test_same_as_the_grid_peel(h, m, nplant, lo, hi, flags):
+    g = synth.chunglu(m // 12, m // 30, m, 2.1, 2.4, seed=m, nplant=nplant, plant_lo=lo, plant_hi=hi, plant_p=0.9)
+    ref = grid_peel(h, g.edges, g.nU, g.nL, flags=flags)
+    for _ in range(2):
+        out = bt.bt_decompose(h, g.edges, g.nU, g.nL, flags=flags)
+        np.testing.assert_array_equal(out[0], ref[0])
+        np.testing.assert_array_equal(out[1], ref[1])
+        assert out[2] == ref[2]
+
+
+@pytest.mark.parametrize("n,hi", [(3, 300), (5, 600), (40, 20000)])
+def test_batches_same_as_the_grid_peel(h, n, hi):
+    gs = [synth.batch_graph(900 + i, hi=hi) for i in range(n)]
+    gs = [(g.edges, g.nU, g.nL) for g in gs] + [(np.empty((0, 2), np.int32), 3, 2), (pins.biclique(40, 50), 40, 50)]
+    bt.bt_set_limits(h, join_cap=1 << 30)
+    ref, st0 = bt.bt_decompose_batch(h, gs, count_threads=512, peel_item=32)
+    bt.bt_set_limits(h)
+    out, st1 = bt.bt_decompose_batch(h, gs, count_threads=512, peel_item=32)
+    assert st0 == st1
+    for (s0, p0), (s1, p1) in zip(ref, out):
+        np.testing.assert_array_equal(s0, s1)
+        np.testing.assert_array_equal(p0, p1)
