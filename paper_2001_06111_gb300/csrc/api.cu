@@ -200,13 +200,14 @@ int count_and_index(bt_handle *h, Prepared &P, uint64_t *d_support, bool want_in
         co.nbv = al.get<uint64_t>(P.g.n);
         if (al.err != cudaSuccess) return cuda_fail(h, al.err, "allocating count buffers");
     }
-    cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al, h->count_nt);
+    cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al);
     if (e != cudaSuccess) return cuda_fail(h, e, "counting wedges");
     unsigned long long bf = 0;
     e = cudaMemcpyAsync(&bf, co.butterflies_dev, sizeof(bf), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     al.put(co.butterflies_dev);
     if (e != cudaSuccess) return cuda_fail(h, e, "counting wedges");
+    bf /= 2;  // every butterfly gives each of its two wedges in a bloom one
     butterflies = bf;
     if (want_index) {
         // W for the statistics: sum of wedges per start vertex
@@ -385,7 +386,7 @@ int bt_count_support_part(bt_handle *h, const int32_t *edges, uint64_t m, uint32
     if (rc == BT_OK) {
         bt::CountOut co;
         co.support = d_int;
-        cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al, h->count_nt, hb[0], hb[1]);
+        cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al, hb[0], hb[1]);
         if (e == cudaSuccess) {
             al.put(co.butterflies_dev);
             e = bt::gather_u64(d_int, P.g.newid, d_sup, m, al);  // back to input order

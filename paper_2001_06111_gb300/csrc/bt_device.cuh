@@ -82,5 +82,36 @@ __device__ __forceinline__ uint32_t last_le_u32(const uint32_t *a, uint32_t len,
     return lo;
 }
 
+// Items of different lengths laid side by side: off[0 .. n] (shared memory) are
+// their first entries, strictly ascending, off[n] the number of entries.  A warp
+// takes neighbouring entries, 32 at a turn, and finds the items of all of them
+// from 32 neighbouring offsets read once; a binary search an entry (ten
+// conflicting reads of shared memory) was what bound such loops.
+
+// The item that holds entry x (the same for the whole warp).
+__device__ __forceinline__ uint32_t item_of(const uint32_t *off, uint32_t n, uint32_t x) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t b = 0;  // n <= 1024: first the 32 items it lies among
+    if (n > 32u)
+        b = 32u * (uint32_t)(__popc(__ballot_sync(0xffffffffu, 32u * lane < n && off[32u * lane] <= x)) - 1);
+    return b + (uint32_t)__popc(__ballot_sync(0xffffffffu, b + lane < n && off[b + lane] <= x)) - 1u;
+}
+// The items of entries [w, w + 32), one a lane; j0: the item of entry w, which
+// becomes that of w + 32.
+__device__ __forceinline__ uint32_t items_of(const uint32_t *off, uint32_t n, uint32_t w, uint32_t &j0) {
+    const uint32_t lane = threadIdx.x & 31, i = j0 + 1u + lane;
+    const uint32_t rel = i <= n ? off[i] - w : 64u;
+    const unsigned starts = __reduce_or_sync(0xffffffffu, rel < 32u ? 1u << rel : 0u);
+    const uint32_t j = j0 + __popc(starts & (0xffffffffu >> (31u - lane)));
+    j0 += __popc(__ballot_sync(0xffffffffu, rel <= 32u));
+    return j;
+}
+// Entries [lo, hi) of `total` that warp `w` of `nw` takes.
+__device__ __forceinline__ void share_of(uint32_t total, uint32_t w, uint32_t nw, uint32_t &lo, uint32_t &hi) {
+    const uint32_t per = ((total + nw * 32u - 1u) / (nw * 32u)) * 32u;
+    lo = w * per < total ? w * per : total;
+    hi = total - lo < per ? total : lo + per;
+}
+
 }  // namespace dev
 }  // namespace bt

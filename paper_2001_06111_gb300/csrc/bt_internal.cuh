@@ -156,6 +156,9 @@ struct Csr {
     uint32_t *hv = nullptr;   // [n] #neighbours of lower rank (a prefix of the list)
     uint32_t *pl = nullptr;   // [2m] for arc (u->v), v<u: #w in N(v) with w<u; else 0
     uint64_t *wv = nullptr;   // [n] priority-obeyed wedges started at each vertex
+    // start vertices that the counting kernel gives a block each (the others get a
+    // warp): n_heavy[0] ranks, roughly ascending
+    uint32_t *heavy = nullptr, *n_heavy = nullptr;
     // Internal edge ids: an edge is numbered by its position in the lower-rank
     // prefix of its higher-ranked endpoint, so the edges of one vertex are
     // contiguous (blooms anchored there touch neighbouring words).  eid holds
@@ -178,6 +181,11 @@ struct GraphSplit {
     const uint32_t *offU = nullptr, *offL = nullptr;
     uint32_t max_n = 0;
 };
+
+// A start vertex of up to kLightW wedges over up to kLightH middle vertices is
+// counted by a warp.
+constexpr uint32_t kLightW = 256, kLightH = 32;
+__host__ __device__ inline bool is_light(uint64_t W, uint32_t h) { return W <= kLightW && h <= kLightH; }
 
 // Builds the CSR (and wedge prefix lengths) from a device edge list.
 // err_word: device u32 receiving kErr* bits.  Returns a CUDA error.
@@ -202,16 +210,14 @@ struct CountOut {
     uint32_t *inc_cnt = nullptr;  // [m] links per edge (index mode) or nullptr
     uint64_t *w2v = nullptr;      // [n] bloom wedges per start vertex (index mode)
     uint64_t *nbv = nullptr;      // [n] blooms per start vertex (index mode)
-    unsigned long long *butterflies_dev = nullptr;  // [1] set by count_wedges; caller frees
+    unsigned long long *butterflies_dev = nullptr;  // [1] twice the butterflies, set by count_wedges; caller frees
     // [m] or nullptr: edges whose bitruss number is already known (progressive
     // compression); they get no links and are flagged in bit 31 inside pairs
     const uint8_t *assigned = nullptr;
 };
-// nt: count block size (256, 512 or 1024; anything else means 512).  Only
-// start vertices of rank in [lo, hi) are enumerated: the supports are then
+// Only start vertices of rank in [lo, hi) are enumerated: the supports are then
 // those of the blooms started there (a counting shard).
-cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, int nt = 512, uint32_t lo = 0,
-                         uint32_t hi = 0xFFFFFFFFu);
+cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint32_t lo = 0, uint32_t hi = 0xFFFFFFFFu);
 // out[0], out[1]: the first rank r with pre[r] >= t0, resp. >= t1 (pre is a
 // non-decreasing array of n values; n when no such rank).
 cudaError_t rank_bounds(const uint64_t *pre, uint32_t n, uint64_t t0, uint64_t t1, uint32_t *out, Alloc &al);

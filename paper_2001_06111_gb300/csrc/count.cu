@@ -12,17 +12,18 @@
 //   emit    the bloom gets bloom number c, and the wedge becomes one twin
 //           pair ((u,v),(v,w)) linked to it (Alg. 3, the second wedge loop).
 //
-// Work layout: persistent blocks pull start vertices from a global queue in
-// decreasing rank (heaviest first).  A block enumerates the wedges of its
-// vertex in chunks of NT middle vertices (NT = block size, picked by the
-// batch autotuner from 256, 512, 1024): a block scan of the per-arc
-// prefix lengths flattens the chunk's wedges, so every thread handles whole
-// wedges regardless of the degree skew.  Counters are a dense per-block
-// array indexed by rank, kept at zero between vertices: when u has fewer
-// than 2^16 lower-ranked neighbours and the arrays are small, a counter's
-// word also counts its readers in pass B and the last reader clears it;
-// otherwise a third walk (pass C) clears the counters.  Emit keeps one 64-bit word per counter (count and
-// claimed bloom) so each wedge touches one memory sector per walk.
+// Counting (k_count, k_count_light).  Start vertices with few wedges are counted
+// by a warp with a hash table in shared memory; the others by a block, heaviest
+// first.  A block lays the wedges over up to 1,024 middle vertices side by side
+// (dev::items_of), so every lane has four wedges in flight whatever the degrees.
+// What bounded the dense counters of a block in global memory was the rate of
+// scattered accesses (3 GB of them on the 30M-edge graph): now the counters of the
+// ranks just below the start vertex, the ones most wedges end at, are in shared
+// memory, and only those of lower ranks are in global memory.
+// Emit: persistent blocks pull start vertices from a queue, walk their wedges in
+// chunks of NT middle vertices (NT = block size, picked by the batch autotuner
+// from 256, 512, 1024), with a dense array of 64-bit words a block (count and
+// claimed bloom) indexed by rank, kept at zero between vertices.
 #include "bt_device.cuh"
 #include "bt_internal.cuh"
 
@@ -78,22 +79,6 @@ __device__ __forceinline__ uint32_t next_vertex(uint32_t *queue, uint32_t lo, ui
 
 __device__ __forceinline__ uint32_t ld_cg(const uint32_t *p) { return __ldcg(p); }
 
-// Pass A over all chunks of u.
-template <int NT>
-__device__ void pass_count(Chunk<NT> &ch, const uint64_t *off, const uint32_t *adj,
-                           const uint32_t *eid, const uint32_t *pl, uint64_t a, uint32_t h,
-                           uint32_t *cnt, uint32_t vb) {
-    for (uint32_t c0 = 0; c0 < h; c0 += NT) {
-        uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-        for (uint32_t t = threadIdx.x; t < T; t += NT) {
-            uint32_t vi;
-            uint64_t arc = wedge_arc(ch, off, t, vi);
-            atomicAdd(&cnt[adj[arc] - vb], 1u);
-        }
-        __syncthreads();
-    }
-}
-
 // Pass A on emit's packed words (count in the low 32 bits).
 template <int NT>
 __device__ void pass_count64(Chunk<NT> &ch, const uint64_t *off, const uint32_t *adj,
@@ -110,117 +95,363 @@ __device__ void pass_count64(Chunk<NT> &ch, const uint64_t *off, const uint32_t 
     }
 }
 
-template <bool kIndex, int NT>
-__global__ void __launch_bounds__(NT) k_count(
-    const uint64_t *__restrict__ off, const uint32_t *__restrict__ adj,
-    const uint32_t *__restrict__ eid, const uint32_t *__restrict__ hv,
-    const uint32_t *__restrict__ pl, const uint64_t *__restrict__ wv, uint32_t lo, uint32_t hi,
-    const uint32_t *__restrict__ vbase, uint32_t cn,
-    uint32_t *cnt_all, unsigned long long *support, uint32_t *inc_cnt, uint64_t *w2v,
-    uint64_t *nbv, unsigned long long *totals, uint32_t *queue, const uint8_t *__restrict__ assigned,
-    bool pack) {
-    __shared__ Chunk<NT> ch;
-    __shared__ unsigned long long s_acc[NT];
-    __shared__ uint32_t s_inc[NT];
-    __shared__ uint32_t s_q;
-    // this block's counters: the w of a start vertex u lie in u's graph, at
-    // w - vbase[u] (vbase null: one graph)
-    uint32_t *cnt = cnt_all + (size_t)blockIdx.x * cn;
-    s_acc[threadIdx.x] = 0;
-    s_inc[threadIdx.x] = 0;
-    unsigned long long bf_total = 0;
-    for (;;) {
-        uint32_t u = next_vertex(queue, lo, hi, &s_q);
-        if (u == 0xFFFFFFFFu) break;
-        if (wv[u] == 0) {
-            if (kIndex && threadIdx.x == 0) {
-                w2v[u] = 0;
-                nbv[u] = 0;
-            }
-            continue;
-        }
-        const uint64_t a = off[u];
-        const uint32_t h = hv[u];
-        const uint32_t vb = vbase ? vbase[u] : 0u;
-        pass_count(ch, off, adj, eid, pl, a, h, cnt, vb);
-        // a counter never exceeds h (one per middle vertex): when h < 2^16 the
-        // count keeps the low half of its word and pass B counts its readers
-        // in the high half, so the last reader clears the word (no pass C).
-        // Only while the counter arrays are small (pack): when they live in
-        // DRAM the returning atomic lengthens pass B more than pass C costs.
-        const bool packed = pack && h < 0x10000u;
-        unsigned long long nb_local = 0;
-        // pass B: attribute c-1 to both edges of every wedge in a bloom
-        unsigned long long w2_local = 0;
-        for (uint32_t c0 = 0; c0 < h; c0 += NT) {
-            uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-            for (uint32_t t = threadIdx.x; t < T; t += NT) {
-                uint32_t vi;
-                uint64_t arc = wedge_arc(ch, off, t, vi);
-                uint32_t *cp = &cnt[adj[arc] - vb];
-                uint32_t c;
-                if (packed) {
-                    const uint32_t old = atomicAdd(cp, 1u << 16);
-                    c = old & 0xFFFFu;
-                    if ((old >> 16) + 1u == c) {
-                        // the last of the c wedges: the bloom is counted once
-                        *cp = 0u;
-                        if (c >= 2) {
-                            ++nb_local;
-                            bf_total += (unsigned long long)c * (c - 1) / 2;
-                        }
-                    }
-                } else {
-                    c = ld_cg(cp);
-                }
-                if (c >= 2) {
-                    uint32_t evw = eid[arc];
-                    atomicAdd(&support[evw], (unsigned long long)(c - 1));
-                    atomicAdd(&s_acc[vi], (unsigned long long)(c - 1));
-                    if (kIndex) {
-                        // edges already assigned (progressive compression) get no links
-                        if (!assigned || !assigned[evw]) atomicAdd(&inc_cnt[evw], 1u);
-                        if (!assigned || !assigned[ch.e[vi]]) atomicAdd(&s_inc[vi], 1u);
-                        ++w2_local;
-                    }
-                }
-            }
-            __syncthreads();
-            if (s_acc[threadIdx.x]) {
-                atomicAdd(&support[ch.e[threadIdx.x]], s_acc[threadIdx.x]);
-                s_acc[threadIdx.x] = 0;
-            }
-            if (kIndex && s_inc[threadIdx.x]) {
-                atomicAdd(&inc_cnt[ch.e[threadIdx.x]], s_inc[threadIdx.x]);
-                s_inc[threadIdx.x] = 0;
-            }
-            __syncthreads();
-        }
-        // pass C: reset counters; the first thread to clear a bloom counts it
-        for (uint32_t c0 = 0; c0 < (packed ? 0u : h); c0 += NT) {
-            uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-            for (uint32_t t = threadIdx.x; t < T; t += NT) {
-                uint32_t vi;
-                uint64_t arc = wedge_arc(ch, off, t, vi);
-                uint32_t old = atomicExch(&cnt[adj[arc] - vb], 0u);
-                if (old >= 2) {
-                    ++nb_local;
-                    bf_total += (unsigned long long)old * (old - 1) / 2;
-                }
-            }
-            __syncthreads();
-        }
-        if (kIndex) {
-            unsigned long long w2s = dev::block_sum(w2_local);
-            unsigned long long nbs = dev::block_sum(nb_local);
-            if (threadIdx.x == 0) {
-                w2v[u] = w2s;
-                nbv[u] = nbs;
-            }
+// ------------------------------------------------------------------- count
+constexpr int kCT = 1024;                // threads of a count block (one an SM)
+constexpr uint32_t kCU = 4;              // wedges a lane has in flight
+constexpr uint32_t kHot = 88 * 1024;     // 16-bit counters in shared memory
+
+struct CountArgs {
+    const uint64_t *off;
+    const uint32_t *adj, *eid, *hv, *pl;
+    const uint64_t *wv;
+    uint32_t lo, hi;
+    const uint32_t *heavy, *n_heavy;
+    const uint32_t *vbase;
+    uint32_t cold_n;  // 32-bit counters of a block in global memory
+    uint32_t *cold;
+    unsigned long long *support;
+    uint32_t *inc_cnt;
+    uint64_t *w2v, *nbv;
+    unsigned long long *totals;  // sum of c - 1 over bloom wedges: twice the butterflies
+    uint32_t *queue;
+    const uint8_t *assigned;
+};
+
+struct CountShared {
+    uint32_t n;
+    uint32_t off[kCT + 1];           // first wedge of each middle vertex
+    uint32_t e[kCT + 1];             // its edge (u, v)
+    unsigned long long at[kCT + 1];  // wedge x of item j is arc at[j] + x
+    uint32_t acc[kCT], inc[kCT];     // support and links of (u, v) from these (supports are below m < 2^31)
+    uint32_t u;
+};
+
+// Lays the wedges over middle vertices [c0, c0 + kCT) of u side by side, empty
+// ones left out.  Returns their number.
+__device__ __forceinline__ uint32_t lay_wedges(CountShared &s, const CountArgs &a, uint64_t arc, uint32_t h, uint32_t c0) {
+    const uint32_t tid = threadIdx.x, i = c0 + tid;
+    uint32_t len = 0, e = 0;
+    uint64_t at = 0;
+    if (i < h) {
+        len = a.pl[arc + i];
+        if (len) {
+            e = a.eid[arc + i];
+            at = a.off[a.adj[arc + i]];
         }
     }
-    bf_total = dev::block_sum(bf_total);
-    if (threadIdx.x == 0 && bf_total) atomicAdd(&totals[0], bf_total);
+    unsigned long long all;
+    const unsigned long long ex =
+        dev::block_excl_scan<unsigned long long>((unsigned long long)(len > 0u) << 48 | len, &all);
+    const uint32_t j = (uint32_t)(ex >> 48), x = (uint32_t)ex;
+    if (len) {
+        s.off[j] = x;
+        s.e[j] = e;
+        s.at[j] = at - x;
+    }
+    if (tid == kCT - 1) {
+        s.n = j + (len > 0u);
+        s.off[j + (len > 0u)] = (uint32_t)all;
+    }
+    __syncthreads();
+    return (uint32_t)all;
+}
+
+// Start vertices with many wedges, one block each, heaviest first.  The counters
+// of the kHot ranks below u are in shared memory (ranks ascend with degree, so
+// they are met by most wedges of a skewed graph), 16 bits each; a start vertex of
+// 2^16 or more middle vertices uses half the ranks with 32 bits.  Those of lower
+// ranks are 32-bit words of this block in global memory: when a count fits 16
+// bits its readers in pass B are counted in the high half and the last one
+// clears the word, else a third walk clears them.
+template <bool kIndex>
+__global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs a) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    CountShared &s = *reinterpret_cast<CountShared *>(s_dyn);
+    uint32_t *hot = reinterpret_cast<uint32_t *>(s_dyn + sizeof(CountShared));
+    uint32_t *cold = a.cold + (size_t)blockIdx.x * a.cold_n;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t i = tid; i < kHot / 2; i += kCT) hot[i] = 0;
+    s.acc[tid] = 0;
+    s.inc[tid] = 0;
+    unsigned long long twice = 0;
+    const uint32_t n_heavy = *a.n_heavy;
+    if (tid == 0) s.u = atomicAdd(a.queue, 1u);
+    __syncthreads();
+    for (;;) {
+        const uint32_t q = s.u;
+        if (q >= n_heavy) break;
+        __syncthreads();
+        uint32_t next = 0;  // the following turn, asked for ahead
+        if (tid == 0) next = atomicAdd(a.queue, 1u);
+        const uint32_t u = a.heavy[n_heavy - 1u - q];
+        if (u >= a.lo && u < a.hi) {
+            const uint64_t arc = a.off[u];
+            const uint32_t h = a.hv[u];
+            const uint32_t vb = a.vbase ? a.vbase[u] : 0u;
+            const bool narrow = h < 0x10000u;  // a count never exceeds h
+            const uint32_t width = narrow ? kHot : kHot / 2;
+            const uint32_t ru = u - vb;
+            const uint32_t base = ru > width ? ru - width : 0u;  // hot counters are those of ranks [base, ru)
+            unsigned long long w2 = 0, nb = 0;
+            // pass A: cnt[w] += 1; the second wedge of an end vertex makes its bloom
+            for (uint32_t c0 = 0; c0 < h; c0 += kCT) {
+                const uint32_t total = lay_wedges(s, a, arc, h, c0);
+                uint32_t lo, hi;
+                dev::share_of(total, warp, kCT / 32, lo, hi);
+                uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
+                for (uint32_t x0 = lo; x0 < hi; x0 += 32u * kCU) {
+                    uint32_t w[kCU], old[kCU];
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        const uint32_t x = x0 + 32u * r + lane, j = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
+                        w[r] = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        old[r] = 0;
+                        if (w[r] == 0xFFFFFFFFu) continue;
+                        if (w[r] >= base) {
+                            const uint32_t i = w[r] - base;
+                            if (narrow) old[r] = atomicAdd(&hot[i >> 1], 1u << (16u * (i & 1u))) >> (16u * (i & 1u)) & 0xFFFFu;
+                            else old[r] = atomicAdd(&hot[i], 1u);
+                        } else if (kIndex) {
+                            old[r] = atomicAdd(&cold[w[r]], 1u);
+                        } else {
+                            atomicAdd(&cold[w[r]], 1u);
+                        }
+                    }
+                    if (kIndex) {
+#pragma unroll
+                        for (uint32_t r = 0; r < kCU; ++r) nb += old[r] == 1u;
+                    }
+                }
+                __syncthreads();
+            }
+            // pass B: attribute c - 1 to both edges of every wedge in a bloom
+            for (uint32_t c0 = 0; c0 < h; c0 += kCT) {
+                const uint32_t total = lay_wedges(s, a, arc, h, c0);
+                uint32_t lo, hi;
+                dev::share_of(total, warp, kCT / 32, lo, hi);
+                uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
+                for (uint32_t x0 = lo; x0 < hi; x0 += 32u * kCU) {
+                    uint32_t w[kCU], c[kCU], jj[kCU], e[kCU];
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        const uint32_t x = x0 + 32u * r + lane;
+                        jj[r] = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
+                        w[r] = x < hi ? a.adj[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        c[r] = 0;
+                        if (w[r] == 0xFFFFFFFFu) continue;
+                        if (w[r] >= base) {
+                            const uint32_t i = w[r] - base;
+                            c[r] = narrow ? hot[i >> 1] >> (16u * (i & 1u)) & 0xFFFFu : hot[i];
+                        } else if (narrow) {
+                            const uint32_t old = atomicAdd(&cold[w[r]], 1u << 16);
+                            c[r] = old & 0xFFFFu;
+                            if ((old >> 16) + 1u == c[r]) cold[w[r]] = 0u;  // every wedge has read it
+                        } else {
+                            c[r] = ld_cg(&cold[w[r]]);
+                        }
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        const uint32_t x = x0 + 32u * r + lane;
+                        e[r] = c[r] >= 2u ? a.eid[s.at[jj[r]] + x] : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t r = 0; r < kCU; ++r) {
+                        if (c[r] < 2u) continue;
+                        atomicAdd(&a.support[e[r]], (unsigned long long)(c[r] - 1u));
+                        atomicAdd(&s.acc[jj[r]], c[r] - 1u);
+                        twice += c[r] - 1u;
+                        if (kIndex) {
+                            // edges already assigned (progressive compression) get no links
+                            if (!a.assigned || !a.assigned[e[r]]) atomicAdd(&a.inc_cnt[e[r]], 1u);
+                            atomicAdd(&s.inc[jj[r]], 1u);
+                            ++w2;
+                        }
+                    }
+                }
+                __syncthreads();
+                if (tid < s.n) {
+                    const uint32_t e = s.e[tid];
+                    if (s.acc[tid]) atomicAdd(&a.support[e], (unsigned long long)s.acc[tid]);
+                    s.acc[tid] = 0;
+                    if (kIndex && s.inc[tid]) {
+                        if (!a.assigned || !a.assigned[e]) atomicAdd(&a.inc_cnt[e], s.inc[tid]);
+                        s.inc[tid] = 0;
+                    }
+                }
+                __syncthreads();
+            }
+            if (!narrow && base) {
+                for (uint32_t c0 = 0; c0 < h; c0 += kCT) {
+                    const uint32_t total = lay_wedges(s, a, arc, h, c0);
+                    uint32_t lo, hi;
+                    dev::share_of(total, warp, kCT / 32, lo, hi);
+                    uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
+                    for (uint32_t x0 = lo; x0 < hi; x0 += 32u) {
+                        const uint32_t x = x0 + lane, j = dev::items_of(s.off, s.n, x0, j0);
+                        const uint32_t w = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
+                        if (w < base) cold[w] = 0u;
+                    }
+                    __syncthreads();
+                }
+            }
+            const uint32_t used = narrow ? (ru - base + 1u) / 2u : ru - base;
+            for (uint32_t i = tid; i < used; i += kCT) hot[i] = 0;
+            if (kIndex) {
+                const unsigned long long w2s = dev::block_sum(w2);
+                const unsigned long long nbs = dev::block_sum(nb);
+                if (tid == 0) {
+                    a.w2v[u] = w2s;
+                    a.nbv[u] = nbs;
+                }
+            }
+        }
+        if (tid == 0) s.u = next;
+        __syncthreads();
+    }
+    twice = dev::block_sum(twice);
+    if (tid == 0 && twice) atomicAdd(&a.totals[0], twice);
+}
+
+// Start vertices with few wedges, a warp each: the end vertices go to a hash
+// table of the warp in shared memory.  Most start vertices of a skewed graph are
+// of this kind; a block's barriers and its turn at the queue cost more than
+// their wedges.
+template <bool kIndex>
+__global__ void __launch_bounds__(256) k_count_light(const __grid_constant__ CountArgs a) {
+    constexpr uint32_t kSlots = 2 * kLightW, kWin = kLightW / 32, kWarps = 8;
+    constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+    __shared__ uint32_t s_key[kWarps][kSlots], s_cnt[kWarps][kSlots];
+    __shared__ uint32_t s_off[kWarps][33], s_acc[kWarps][32], s_inc[kWarps][32];
+    __shared__ unsigned long long s_at[kWarps][33];
+    const uint32_t lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    uint32_t *key = s_key[wi], *cnt = s_cnt[wi], *off = s_off[wi];
+    for (uint32_t i = lane; i < kSlots; i += 32) {
+        key[i] = kEmpty;
+        cnt[i] = 0;
+    }
+    s_acc[wi][lane] = s_inc[wi][lane] = 0;
+    __syncwarp();
+    unsigned long long twice = 0;
+    const uint32_t nw = gridDim.x * kWarps;
+    // warp x takes ranks x, x + nw, ...: 32 looked up at a turn, so that a small
+    // graph still gives every vertex its own warp
+    const uint32_t ranks = a.hi - a.lo;
+    for (uint64_t g = blockIdx.x * kWarps + wi; g < ranks; g += 32ull * nw) {
+        bool light = false;
+        uint32_t my_h = 0, my_u = 0;
+        uint64_t my_arc = 0;
+        if (g + (uint64_t)lane * nw < ranks) {
+            const uint32_t u = my_u = a.lo + (uint32_t)(g + (uint64_t)lane * nw);
+            const uint64_t W = a.wv[u];
+            if (kIndex && W == 0) a.w2v[u] = a.nbv[u] = 0;
+            if (W > 0) {
+                my_h = a.hv[u];
+                my_arc = a.off[u];
+                light = is_light(W, my_h);
+            }
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, light);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const uint32_t u = __shfl_sync(0xffffffffu, my_u, src), h = __shfl_sync(0xffffffffu, my_h, src);
+            const uint64_t arc = __shfl_sync(0xffffffffu, my_arc, src);
+            uint32_t len = 0, e = 0;
+            uint64_t at = 0;
+            if (lane < h) {
+                len = a.pl[arc + lane];
+                if (len) {
+                    e = a.eid[arc + lane];
+                    at = a.off[a.adj[arc + lane]];
+                }
+            }
+            const unsigned has = __ballot_sync(0xffffffffu, len > 0u);
+            const uint32_t incl = dev::warp_incl_scan(len), total = __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t j = __popc(has & ((1u << lane) - 1u)), n = __popc(has);
+            if (len) {
+                off[j] = incl - len;
+                s_at[wi][j] = at - (incl - len);
+            }
+            if (lane == 31) off[n] = total;
+            __syncwarp();
+            uint32_t slot[kWin], jj[kWin], j0 = 0, nb = 0;
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                slot[r] = kEmpty;
+                jj[r] = 0;
+                if (32u * r < total) {
+                    jj[r] = dev::items_of(off, n, 32u * r, j0);
+                    const uint32_t x = 32u * r + lane;
+                    if (x < total) slot[r] = a.adj[s_at[wi][jj[r]] + x];
+                }
+            }
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                if (slot[r] == kEmpty) continue;
+                const uint32_t w = slot[r];
+                uint32_t i = (w * 0x9E3779B1u) >> 23;  // 2^9 slots
+                for (;;) {
+                    const uint32_t k = atomicCAS(&key[i], kEmpty, w);
+                    if (k == kEmpty || k == w) break;
+                    i = (i + 1u) & (kSlots - 1u);
+                }
+                slot[r] = i;
+                if (atomicAdd(&cnt[i], 1u) == 1u) ++nb;
+            }
+            __syncwarp();
+            uint32_t w2 = 0;
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                if (slot[r] == kEmpty) continue;
+                const uint32_t c = cnt[slot[r]];
+                if (c < 2u) continue;
+                const uint32_t ev = a.eid[s_at[wi][jj[r]] + 32u * r + lane];
+                atomicAdd(&a.support[ev], (unsigned long long)(c - 1u));
+                atomicAdd(&s_acc[wi][jj[r]], c - 1u);
+                twice += c - 1u;
+                if (kIndex) {
+                    if (!a.assigned || !a.assigned[ev]) atomicAdd(&a.inc_cnt[ev], 1u);
+                    atomicAdd(&s_inc[wi][jj[r]], 1u);
+                    ++w2;
+                }
+            }
+            __syncwarp();
+            // the lane that read item j's record adds what the item gathered
+            if (len) {
+                const uint32_t acc = s_acc[wi][j];
+                if (acc) atomicAdd(&a.support[e], (unsigned long long)acc);
+                s_acc[wi][j] = 0;
+                if (kIndex && s_inc[wi][j]) {
+                    if (!a.assigned || !a.assigned[e]) atomicAdd(&a.inc_cnt[e], s_inc[wi][j]);
+                    s_inc[wi][j] = 0;
+                }
+            }
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r)
+                if (slot[r] != kEmpty) {
+                    key[slot[r]] = kEmpty;
+                    cnt[slot[r]] = 0;
+                }
+            if (kIndex) {
+                w2 = dev::warp_sum(w2);
+                nb = dev::warp_sum(nb);
+                if (lane == 0) {
+                    a.w2v[u] = w2;
+                    a.nbv[u] = nb;
+                }
+            }
+            __syncwarp();
+        }
+    }
+    twice = dev::warp_sum(twice);
+    if (lane == 0 && twice) atomicAdd(&a.totals[0], twice);
 }
 
 // Emit the index: blooms (bloom number, first pair), twin pairs and the
@@ -315,63 +546,62 @@ __global__ void __launch_bounds__(NT) k_emit(
     }
 }
 
-template <int NT>
-int blocks_per_sm_count() {
-    int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_count<true, NT>, NT, 0);
-    return b > 0 ? b : 1;
-}
-
-int blocks_per_sm_for(int nt) {
-    return nt == 256 ? blocks_per_sm_count<256>()
-                     : nt == 1024 ? blocks_per_sm_count<1024>() : blocks_per_sm_count<512>();
-}
-
-template <int NT>
-void launch_count(bool index, unsigned blocks, const Csr &g, uint32_t lo, uint32_t hi, uint32_t *cnt,
-                  unsigned long long *sup, CountOut &o, unsigned long long *totals, uint32_t *queue,
-                  cudaStream_t st) {
-    // two walks per vertex while all blocks' counter arrays total at most
-    // 1 GiB (2M-edge graph, 0.34 GB: 6.98 -> 6.47 ms); three above it
-    // (30M-edge graph, 3 GB: 267-274 against 305-318 ms with two)
-    const bool pack = (uint64_t)blocks * g.cnt_n * sizeof(uint32_t) <= (1ull << 30);
-    if (index)
-        k_count<true, NT><<<blocks, NT, 0, st>>>(g.off, g.adj, g.eid, g.hv, g.pl, g.wv, lo, hi, g.vbase, g.cnt_n, cnt,
-                                                  sup, o.inc_cnt, o.w2v, o.nbv, totals, queue, o.assigned, pack);
-    else
-        k_count<false, NT><<<blocks, NT, 0, st>>>(g.off, g.adj, g.eid, g.hv, g.pl, g.wv, lo, hi, g.vbase, g.cnt_n, cnt,
-                                                   sup, nullptr, nullptr, nullptr, totals, queue, nullptr, pack);
-}
-
 }  // namespace
 
-cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, int nt, uint32_t lo, uint32_t hi) {
+cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint32_t lo, uint32_t hi) {
     const bool index = o.inc_cnt != nullptr;
     if (hi > g.n) hi = g.n;
     if (lo > hi) lo = hi;
-    if (nt != 256 && nt != 1024) nt = 512;
-    int bps = blocks_per_sm_for(nt);
-    unsigned blocks = (unsigned)(num_sms * bps);
-    uint32_t *cnt = al.get<uint32_t>((size_t)blocks * g.cnt_n);
-    uint32_t *queue = al.get<uint32_t>(1);
-    unsigned long long *totals = al.get<unsigned long long>(1);
+    const unsigned blocks = (unsigned)num_sms;
+    // ranks below the counters in shared memory (half as many where they have 32
+    // bits, for a start vertex of 2^16 middle vertices: its graph has those and more)
+    const uint32_t width = g.cnt_n < 0x10000u ? kHot : kHot / 2;
+    CountArgs a{};
+    a.off = g.off;
+    a.adj = g.adj;
+    a.eid = g.eid;
+    a.hv = g.hv;
+    a.pl = g.pl;
+    a.wv = g.wv;
+    a.heavy = g.heavy;
+    a.n_heavy = g.n_heavy;
+    a.lo = lo;
+    a.hi = hi;
+    a.vbase = g.vbase;
+    a.cold_n = g.cnt_n > width ? g.cnt_n - width : 0u;
+    a.cold = al.get<uint32_t>((size_t)blocks * a.cold_n);
+    a.queue = al.get<uint32_t>(1);
+    a.totals = al.get<unsigned long long>(1);
     if (al.err != cudaSuccess) return al.err;
-    BT_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)blocks * g.cnt_n, al.stream));
-    BT_CUDA(cudaMemsetAsync(queue, 0, sizeof(uint32_t), al.stream));
-    BT_CUDA(cudaMemsetAsync(totals, 0, sizeof(unsigned long long), al.stream));
+    a.support = reinterpret_cast<unsigned long long *>(o.support);
+    a.inc_cnt = o.inc_cnt;
+    a.w2v = o.w2v;
+    a.nbv = o.nbv;
+    a.assigned = index ? o.assigned : nullptr;
+    if (a.cold_n) BT_CUDA(cudaMemsetAsync(a.cold, 0, sizeof(uint32_t) * (size_t)blocks * a.cold_n, al.stream));
+    BT_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), al.stream));
+    BT_CUDA(cudaMemsetAsync(a.totals, 0, sizeof(unsigned long long), al.stream));
     BT_CUDA(cudaMemsetAsync(o.support, 0, sizeof(uint64_t) * g.m, al.stream));
     if (index) BT_CUDA(cudaMemsetAsync(o.inc_cnt, 0, sizeof(uint32_t) * g.m, al.stream));
-    auto *sup = reinterpret_cast<unsigned long long *>(o.support);
+    const size_t smem = sizeof(CountShared) + kHot * sizeof(uint16_t);
+    const unsigned groups = (hi - lo + 7u) / 8u, room = (unsigned)num_sms * 5u;
+    const unsigned light = groups < room ? (groups ? groups : 1u) : room;
     al.mark(kPhCount, false);
-    if (nt == 256) launch_count<256>(index, blocks, g, lo, hi, cnt, sup, o, totals, queue, al.stream);
-    else if (nt == 1024) launch_count<1024>(index, blocks, g, lo, hi, cnt, sup, o, totals, queue, al.stream);
-    else launch_count<512>(index, blocks, g, lo, hi, cnt, sup, o, totals, queue, al.stream);
-    al.launches++;
+    if (index) {
+        BT_CUDA(cudaFuncSetAttribute(k_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_count<true><<<blocks, kCT, smem, al.stream>>>(a);
+        k_count_light<true><<<light, 256, 0, al.stream>>>(a);
+    } else {
+        BT_CUDA(cudaFuncSetAttribute(k_count<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_count<false><<<blocks, kCT, smem, al.stream>>>(a);
+        k_count_light<false><<<light, 256, 0, al.stream>>>(a);
+    }
+    al.launches += 2;
     al.mark(kPhCount, true);
     BT_CUDA(cudaGetLastError());
-    o.butterflies_dev = totals;
-    al.put(cnt);
-    al.put(queue);
+    o.butterflies_dev = a.totals;
+    al.put(a.cold);
+    al.put(a.queue);
     return cudaSuccess;
 }
 
@@ -412,10 +642,10 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     ix.pairs = al.get<uint2>(ix.w2);
     ix.inc = al.get<uint2>(ix.links);
     uint32_t *inc_fill = al.get<uint32_t>(m);
-    // 1024-thread emit blocks: one per SM, so that half as many pairs of
-    // dense per-block arrays compete for L2 (measured 5-20 % faster than two
-    // per SM; the count kernel keeps two per SM, where one measured slower)
-    int bps = nt == 1024 ? 1 : blocks_per_sm_for(nt);
+    // as few resident blocks as keep the SMs busy, so that few of their dense
+    // arrays compete for L2 (1024 threads: one block an SM measured 5-20 % faster
+    // than two; a batch of 384 graphs with 256 threads: 8.7 ms with six, 10.0 with eight)
+    const int bps = nt == 1024 ? 1 : nt == 512 ? 3 : 6;
     unsigned blocks = (unsigned)(num_sms * bps);
     unsigned long long *cw = al.get<unsigned long long>((size_t)blocks * g.cnt_n);
     uint32_t *queue = al.get<uint32_t>(1);

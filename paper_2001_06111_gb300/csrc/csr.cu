@@ -131,7 +131,7 @@ __device__ __forceinline__ uint32_t lower_bound(const uint32_t *a, uint32_t len,
 // Warp per vertex u: hv[u] = |{v in N(u): v < u}|; for those arcs
 // pl = |{w in N(v): w < u}|; wv[u] = sum of pl (wedges started at u).
 __global__ void k_wedge_prefix(const uint64_t *off, const uint32_t *adj, uint32_t n, uint32_t *hv,
-                               uint32_t *pl, uint64_t *wv) {
+                               uint32_t *pl, uint64_t *wv, uint32_t *heavy, uint32_t *n_heavy) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -154,6 +154,7 @@ __global__ void k_wedge_prefix(const uint64_t *off, const uint32_t *adj, uint32_
         if (lane == 0) {
             hv[u] = h;
             wv[u] = acc;
+            if (acc && !is_light(acc, h)) heavy[atomicAdd(n_heavy, 1u)] = u;
         }
     }
 }
@@ -303,13 +304,16 @@ cudaError_t build_csr(const int32_t *d_edges, uint64_t m, uint32_t nU, uint32_t 
     g.pl = al.get<uint32_t>(na);
     g.hv = al.get<uint32_t>(n);
     g.wv = al.get<uint64_t>(n);
+    g.heavy = al.get<uint32_t>(n);
+    g.n_heavy = al.get<uint32_t>(1);
     if (al.err != cudaSuccess) return al.err;
     k_csr_fill<<<grid_for(na, 256), 256, 0, al.stream>>>(keys, vals, na, n, g.adj, g.eid, err_word);
     al.launches++;
     al.put(keys);
     al.put(vals);
+    BT_CUDA(cudaMemsetAsync(g.n_heavy, 0, sizeof(uint32_t), al.stream));
     k_wedge_prefix<<<grid_for((uint64_t)n * 32, 256), 256, 0, al.stream>>>(g.off, g.adj, n, g.hv,
-                                                                           g.pl, g.wv);
+                                                                           g.pl, g.wv, g.heavy, g.n_heavy);
     al.launches++;
     // internal edge ids grouped by the higher-ranked endpoint
     {
@@ -363,6 +367,8 @@ void free_csr(Csr &g, Alloc &al) {
     al.put(g.pl);
     al.put(g.hv);
     al.put(g.wv);
+    al.put(g.heavy);
+    al.put(g.n_heavy);
     g = Csr{};
 }
 

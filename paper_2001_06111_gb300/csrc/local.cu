@@ -264,31 +264,6 @@ struct Part {
     __device__ __forceinline__ const uint2 *entry(uint32_t j, uint32_t x) const {
         return reinterpret_cast<const uint2 *>(s.at[j] + 8ull * x);
     }
-    // The item that holds entry x (the same for the whole warp).
-    __device__ __forceinline__ uint32_t item_of(uint32_t x) const {
-        const uint32_t lane = threadIdx.x & 31, n = s.n;
-        uint32_t b = 0;
-        if (n > 32u) b = 32u * (uint32_t)(__popc(__ballot_sync(kAll, 32u * lane < n && s.off[32u * lane] <= x)) - 1);
-        return b + (uint32_t)__popc(__ballot_sync(kAll, b + lane < n && s.off[b + lane] <= x)) - 1u;
-    }
-    // The items of entries [w, w + 32), one a lane; j0: the item of entry w,
-    // which becomes that of w + 32.  32 neighbouring offsets are read once and
-    // the lanes count the items that start up to them.
-    __device__ __forceinline__ uint32_t items_of(uint32_t w, uint32_t &j0) const {
-        const uint32_t lane = threadIdx.x & 31, i = j0 + 1u + lane;
-        const uint32_t rel = i <= s.n ? s.off[i] - w : 64u;
-        const unsigned starts = __reduce_or_sync(kAll, rel < 32u ? 1u << rel : 0u);
-        const uint32_t j = j0 + __popc(starts & (0xffffffffu >> (31u - lane)));
-        j0 += __popc(__ballot_sync(kAll, rel <= 32u));
-        return j;
-    }
-    // Entries [lo, hi) of `total` that warp `w` of `nw` takes.
-    __device__ __forceinline__ static void share(uint32_t total, uint32_t w, uint32_t nw, uint32_t &lo, uint32_t &hi) {
-        const uint32_t per = ((total + nw * 32u - 1u) / (nw * 32u)) * 32u;
-        lo = w * per < total ? w * per : total;
-        hi = total - lo < per ? total : lo + per;
-    }
-
     // The batch's edges in shared memory receive state v.
     __device__ __forceinline__ void mark(uint32_t head, uint32_t F, int v) {
         for (uint32_t i = threadIdx.x; i < F; i += kNT)
@@ -303,7 +278,7 @@ struct Part {
         uint2 l[U];
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) {
-            const uint32_t x = w + 32u * u + lane, j = items_of(w + 32u * u, j0);
+            const uint32_t x = w + 32u * u + lane, j = dev::items_of(s.off, s.n, w + 32u * u, j0);
             ed[u] = s.id[j];
             l[u] = x < hi ? *entry(j, x) : make_uint2(0u, 0u);
         }
@@ -396,8 +371,8 @@ struct Part {
             }
             c0 += n;
             uint32_t lo, hi;
-            share((uint32_t)total, warp, nranks * (kNT / 32), lo, hi);
-            uint32_t j0 = lo < hi ? item_of(lo) : 0u;
+            dev::share_of((uint32_t)total, warp, nranks * (kNT / 32), lo, hi);
+            uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
             if (hi - lo > 32u) {
                 for (uint32_t w = lo; w < hi; w += 32u * kU) kill_window<kU>(w, hi, j0);
             } else if (lo < hi) {
@@ -415,7 +390,7 @@ struct Part {
         uint32_t c[U];
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) {
-            const uint32_t x = w + 32u * u + lane, j = items_of(w + 32u * u, j0);
+            const uint32_t x = w + 32u * u + lane, j = dev::items_of(s.off, s.n, w + 32u * u, j0);
             c[u] = s.c[j];
             pr[u] = x < hi ? *entry(j, x) : make_uint2(0u, 0u);
         }
@@ -443,8 +418,8 @@ struct Part {
         const uint32_t total =
             (uint32_t)lay(n, r.z != r.w ? r.y : 0u, B, r.w, r.y <= 2u ? a.bl[B].pair : a.pairs + r.x);
         uint32_t lo, hi;
-        share(total, tid >> 5, kNT / 32, lo, hi);
-        uint32_t j0 = lo < hi ? item_of(lo) : 0u;
+        dev::share_of(total, tid >> 5, kNT / 32, lo, hi);
+        uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
         if (hi - lo > 32u) {
             for (uint32_t w = lo; w < hi; w += 32u * kU) apply_window<kU>(w, hi, j0);
         } else if (lo < hi) {

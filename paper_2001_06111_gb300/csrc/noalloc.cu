@@ -32,7 +32,7 @@ namespace {
 constexpr size_t kStaticBytes = 48ull << 20;   // 48 MiB per device
 constexpr uint64_t kMaxEdges = 1ull << 18;      // 262,144 edges
 constexpr uint64_t kMaxVertices = 1ull << 17;   // nU + nL <= 131,072
-constexpr int kStaticSms = 8;                   // count kernel: 8 x (blocks per SM) blocks
+constexpr int kStaticSms = 40;                  // count blocks with counters in the array: 344 KB each at most
 constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
@@ -92,7 +92,9 @@ extern "C" int bt_count_support_static(const int32_t *d_edges, uint64_t m, uint3
     bt::CountOut co;
     co.support = al.get<uint64_t>(m);  // internal edge order, gathered below
     if (!co.support) return BT_ERR_TOO_LARGE;
-    e = bt::count_wedges(g, co, kStaticSms < num_sms ? kStaticSms : num_sms, al);
+    // graphs of fewer than 2^16 vertices need no counters outside shared memory
+    const int sms = g.n < 0x10000u || kStaticSms > num_sms ? num_sms : kStaticSms;
+    e = bt::count_wedges(g, co, sms, al);
     if (e == cudaErrorMemoryAllocation) return BT_ERR_TOO_LARGE;
     if (e == cudaSuccess) e = bt::gather_u64(co.support, g.newid, d_support_out, m, al);
     if (e == cudaSuccess) e = cudaStreamSynchronize(al.stream);

@@ -1,0 +1,71 @@
+"""The counting kernels at the edges of their tiers: start vertices counted by a
+warp (up to 256 wedges over up to 32 middle vertices) and by a block, chunks of
+1,024 middle vertices, and counters inside and below the 90,112 ranks (16 bits)
+or 45,056 (32 bits) kept in shared memory."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2001_06111_gb300 import bitruss as bt
+from paper_2001_06111_gb300 import build, synth
+from tests import pins
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def h():
+    build.build()
+    handle = bt.bt_create(0)
+    yield handle
+    handle.close()
+
+
+def check(h, e, nU, nL):
+    np.testing.assert_array_equal(bt.bt_count_support(h, e, nU, nL), oracle.support(e, nU, nL))
+    st = bt.bt_build_index(h, e, nU, nL)
+    assert 4 * st["n_butterflies"] == int(oracle.support(e, nU, nL).sum())
+
+
+# K_{a,b}: support (a-1)(b-1); wedges and middle vertices around 256 and 32 and around 1,024
+@pytest.mark.parametrize("a,b", [(2, 2), (8, 32), (8, 33), (9, 31), (16, 16), (17, 16), (32, 32), (33, 32), (2, 1023),
+                                 (2, 1024), (2, 1025), (3, 2049)])
+def test_bicliques(h, a, b):
+    sup = bt.bt_count_support(h, pins.biclique(a, b), a, b)
+    assert (sup == (a - 1) * (b - 1)).all()
+    st = bt.bt_build_index(h, pins.biclique(a, b), a, b)
+    assert st["n_butterflies"] == a * (a - 1) * b * (b - 1) // 4
+
+
+# a hub pair over all lower vertices beside many vertices of low degree: end vertices
+# far below the hub, in and out of the counters in shared memory
+@pytest.mark.parametrize("nU,nL", [(90110, 700), (90112, 700), (140000, 3000)])
+def test_counters_below_the_window(h, nU, nL):
+    rng = np.random.default_rng(nU)
+    hubs = np.stack(np.meshgrid([0, 1], np.arange(nL), indexing="ij"), -1).reshape(-1, 2)
+    u = np.repeat(np.arange(2, nU), 2)
+    v = rng.integers(0, nL // 2, u.size // 2)
+    rest = np.stack([u, np.stack([v, v + 1 + rng.integers(0, nL // 2 - 1, v.size)], 1).reshape(-1)], 1)
+    e = np.concatenate([hubs, rest]).astype(np.int32)
+    check(h, e, nU, nL)
+
+
+# 2^16 and more middle vertices: 32-bit counters.  Four upper vertices have edges,
+# so the supports follow from their common neighbours (paths of three edges from u
+# to v, less those over (u, v)).
+@pytest.mark.parametrize("nL", [65535, 65536, 70001])
+def test_start_vertex_of_many_middles(h, nL):
+    lower = np.arange(nL)
+    e = np.concatenate([np.stack([np.full(nL, i), lower], 1) for i in range(3)]
+                       + [np.stack([np.full(50, 3), lower[:50]], 1)]).astype(np.int32)
+    adj = np.zeros((4, nL), dtype=np.int64)
+    adj[e[:, 0], e[:, 1]] = 1
+    paths = (adj @ adj.T) @ adj
+    want = paths[e[:, 0], e[:, 1]] - adj.sum(1)[e[:, 0]] - adj.sum(0)[e[:, 1]] + 1
+    np.testing.assert_array_equal(bt.bt_count_support(h, e, 60000, nL).astype(np.int64), want)
+    assert 4 * bt.bt_build_index(h, e, 60000, nL)["n_butterflies"] == int(want.sum())
+
+
+def test_skewed_graph(h):
+    g = synth.chunglu(9000, 4000, 60000, 2.0, 2.2, seed=5)
+    check(h, g.edges, g.nU, g.nL)
