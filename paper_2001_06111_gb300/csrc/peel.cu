@@ -143,7 +143,7 @@ struct PeelArgs {
     const uint2 *pairs;
     const uint32_t *bloom_off;
     BloomWord *blooms;
-    long long *sup;
+    int *sup;  // below m < 2^31: k butterflies on an edge need k other edges opposite it
     uint32_t *state;
     uint32_t *phi;
     uint32_t *died;           // death stamp of a twin pair (kAlive while alive)
@@ -188,7 +188,7 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 
 __device__ __forceinline__ uint32_t ldcg_u32(const uint32_t *p) { return __ldcg(p); }
-__device__ __forceinline__ long long ldcg_ll(const long long *p) { return __ldcg(p); }
+__device__ __forceinline__ long long ldcg_ll(const int *p) { return __ldcg(p); }
 
 // Grid-wide barrier over all blocks of a cooperative launch.  Arrivals go
 // to one monotonic counter (release); barrier number b completes when the
@@ -416,7 +416,7 @@ __device__ __forceinline__ void apply_slots(const PeelArgs &a, const uint32_t (&
                                             uint32_t round, unsigned long long &upd, uint32_t *s_je, uint32_t *s_jn) {
     const uint32_t q = round + 1u;
     uint32_t e[2 * N];
-    long long dec[2 * N];
+    int dec[2 * N];
 #pragma unroll
     for (uint32_t r = 0; r < N; ++r) {
         // bit 31 flags an edge whose bitruss number is already known: it is
@@ -435,21 +435,18 @@ __device__ __forceinline__ void apply_slots(const PeelArgs &a, const uint32_t (&
         } else if (dr == round && kB[r] > 1u) {
             // died now: a member outside S (its bit not stamped) loses its
             // k_B - 1 butterflies
-            if (!(fx || (d[r] & 1u))) dec[2 * r] = (long long)kB[r] - 1;
-            if (!(fy || (d[r] & 2u))) dec[2 * r + 1] = (long long)kB[r] - 1;
+            if (!(fx || (d[r] & 1u))) dec[2 * r] = (int)kB[r] - 1;
+            if (!(fy || (d[r] & 2u))) dec[2 * r + 1] = (int)kB[r] - 1;
         }
     }
-    long long old[2 * N];
+    int old[2 * N];
 #pragma unroll
-    for (uint32_t i = 0; i < 2 * N; ++i)
-        old[i] = dec[i] ? (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&a.sup[e[i]]),
-                                               (unsigned long long)(-dec[i]))
-                        : 0;
+    for (uint32_t i = 0; i < 2 * N; ++i) old[i] = dec[i] ? atomicSub(&a.sup[e[i]], dec[i]) : 0;
 #pragma unroll
     for (uint32_t i = 0; i < 2 * N; ++i) {
         if (!dec[i]) continue;
         ++upd;
-        const long long now = old[i] - dec[i];
+        const int now = old[i] - dec[i];
         if (old[i] >= L.khi && now < L.khi) push_near(a, e[i], L.nq);
         // exactly one decrement takes the edge from > k to <= k: it joins the
         // next batch
@@ -1044,11 +1041,11 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
 // Edges already assigned (mask set) start in the permanent state: never alive,
 // never queued.
 constexpr uint32_t kPerm = 0xFFFFFFFEu;
-__global__ void k_peel_init(const uint64_t *support, uint64_t m, long long *sup, uint32_t *state,
+__global__ void k_peel_init(const uint64_t *support, uint64_t m, int *sup, uint32_t *state,
                             const uint8_t *assigned, uint32_t *alive) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        sup[i] = (long long)support[i];
+        sup[i] = (int)support[i];
         state[i] = (assigned && assigned[i]) ? kPerm : kAlive;
         alive[i] = (uint32_t)i;
     }
@@ -1091,7 +1088,7 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     a.inc = ix.inc;
     a.pairs = ix.pairs;
     a.phi = phi_out;
-    a.sup = al.get<long long>(m);
+    a.sup = al.get<int>(m);
     a.state = al.get<uint32_t>(m);
     a.died = al.get<uint32_t>(ix.w2);
     a.bloom_off = ix.bloom_off;
