@@ -221,7 +221,7 @@ int count_and_index(bt_handle *h, Prepared &P, uint64_t *d_support, bool want_in
         al.put(tot);
         al.put(scratch);
         if (e != cudaSuccess) return cuda_fail(h, e, "summing wedges");
-        e = bt::emit_index(P.g, co, ix, h->num_sms, al, h->stream, h->count_nt);
+        e = bt::emit_index(P.g, co, ix, h->num_sms, al, h->stream);
         al.put(co.inc_cnt);
         al.put(co.w2v);
         al.put(co.nbv);
@@ -996,6 +996,13 @@ static int autotune(bt_handle *h, const bt_graph *graphs, uint32_t n, uint32_t f
         return BT_OK;
     }
     if (total == 0) return BT_OK;
+    if (!grid_peel_only(h)) {
+        // counting and emit pick their own tiers and the coarse peel its items:
+        // the schedule has nothing left that a sample would tell apart
+        h->tuned[sig] = {h->count_nt, h->peel_seg};
+        *tuned = 1;
+        return BT_OK;
+    }
     // sample: every stride-th graph, about 8M edges
     const uint64_t target = 8ull << 20;
     const uint32_t stride = (uint32_t)std::max<uint64_t>(1, (total + target - 1) / target);

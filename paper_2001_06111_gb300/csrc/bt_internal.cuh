@@ -140,6 +140,9 @@ cudaError_t widen_u32(const uint32_t *in, uint64_t *out, size_t n, Alloc &al);
 // keys.  Result ends in (keys, vals); (tk, tv) are scratch of the same size.
 cudaError_t radix_sort_u32(uint32_t *keys, uint32_t *vals, uint32_t *tk, uint32_t *tv, size_t n,
                            int bits, Alloc &al);
+// order: the places of the keys, largest key first, equal keys in input order;
+// sorted (nullable) receives the keys in that order.
+cudaError_t radix_order_desc_u32(const uint32_t *keys, size_t n, uint32_t *order, uint32_t *sorted, Alloc &al);
 cudaError_t radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t *tk, uint32_t *tv, size_t n,
                            int bits, Alloc &al);
 
@@ -157,7 +160,7 @@ struct Csr {
     uint32_t *pl = nullptr;   // [2m] for arc (u->v), v<u: #w in N(v) with w<u; else 0
     uint64_t *wv = nullptr;   // [n] priority-obeyed wedges started at each vertex
     // start vertices that the counting kernel gives a block each (the others get a
-    // warp): n_heavy[0] ranks, roughly ascending
+    // warp): n_heavy[64] ranks, by the power of two of their wedges, most first
     uint32_t *heavy = nullptr, *n_heavy = nullptr;
     // Internal edge ids: an edge is numbered by its position in the lower-rank
     // prefix of its higher-ranked endpoint, so the edges of one vertex are
@@ -245,8 +248,7 @@ struct Index {
         return nb * 8 + 4 + w2 * 8 + (m + 1) * 8 + links * 8;
     }
 };
-cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, Alloc &al,
-                       cudaStream_t stream, int nt = 512);
+cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, Alloc &al, cudaStream_t stream);
 void free_index(Index &ix, Alloc &al);
 
 // ---------------------------------------------------------------- peeling

@@ -20,80 +20,13 @@
 // scattered accesses (3 GB of them on the 30M-edge graph): now the counters of the
 // ranks just below the start vertex, the ones most wedges end at, are in shared
 // memory, and only those of lower ranks are in global memory.
-// Emit: persistent blocks pull start vertices from a queue, walk their wedges in
-// chunks of NT middle vertices (NT = block size, picked by the batch autotuner
-// from 256, 512, 1024), with a dense array of 64-bit words a block (count and
-// claimed bloom) indexed by rank, kept at zero between vertices.
 #include "bt_device.cuh"
 #include "bt_internal.cuh"
 
 namespace bt {
 namespace {
 
-template <int NT>
-struct Chunk {
-    uint32_t off[NT + 1];  // exclusive prefix of wedge counts; off[NT] = total
-    uint32_t v[NT];        // middle vertex (rank)
-    uint32_t e[NT];        // edge id of (u, v)
-};
-
-// Loads middle vertices [c0, c0 + NT) of start vertex u.  Returns the
-// number of wedges in the chunk.  Contains __syncthreads().
-template <int NT>
-__device__ __forceinline__ uint32_t load_chunk(Chunk<NT> &ch, const uint32_t *adj, const uint32_t *eid,
-                                               const uint32_t *pl, uint64_t a, uint32_t h,
-                                               uint32_t c0) {
-    uint32_t i = c0 + threadIdx.x;
-    uint32_t p = 0, v = 0, e = 0;
-    if (i < h) {
-        p = pl[a + i];
-        v = adj[a + i];
-        e = eid[a + i];
-    }
-    uint32_t tot;
-    uint32_t ex = dev::block_excl_scan<uint32_t>(p, &tot);
-    ch.off[threadIdx.x] = ex;
-    ch.v[threadIdx.x] = v;
-    ch.e[threadIdx.x] = e;
-    if (threadIdx.x == 0) ch.off[NT] = tot;
-    __syncthreads();
-    return tot;
-}
-
-// Wedge t of the chunk -> (chunk slot vi, arc index of (v, w) in the CSR).
-template <int NT>
-__device__ __forceinline__ uint64_t wedge_arc(const Chunk<NT> &ch, const uint64_t *off, uint32_t t,
-                                              uint32_t &vi) {
-    vi = dev::last_le_u32(ch.off, NT, t);
-    return off[ch.v[vi]] + (t - ch.off[vi]);
-}
-
-// Next start vertex of the rank range [lo, hi), highest rank first.
-__device__ __forceinline__ uint32_t next_vertex(uint32_t *queue, uint32_t lo, uint32_t hi, uint32_t *s_q) {
-    if (threadIdx.x == 0) *s_q = atomicAdd(queue, 1u);
-    __syncthreads();
-    uint32_t qi = *s_q;
-    __syncthreads();
-    return qi < hi - lo ? hi - 1 - qi : 0xFFFFFFFFu;
-}
-
 __device__ __forceinline__ uint32_t ld_cg(const uint32_t *p) { return __ldcg(p); }
-
-// Pass A on emit's packed words (count in the low 32 bits).
-template <int NT>
-__device__ void pass_count64(Chunk<NT> &ch, const uint64_t *off, const uint32_t *adj,
-                             const uint32_t *eid, const uint32_t *pl, uint64_t a, uint32_t h,
-                             unsigned long long *cw, uint32_t vb) {
-    for (uint32_t c0 = 0; c0 < h; c0 += NT) {
-        uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-        for (uint32_t t = threadIdx.x; t < T; t += NT) {
-            uint32_t vi;
-            uint64_t arc = wedge_arc(ch, off, t, vi);
-            atomicAdd(&cw[adj[arc] - vb], 1ull);
-        }
-        __syncthreads();
-    }
-}
 
 // ------------------------------------------------------------------- count
 constexpr int kCT = 1024;                // threads of a count block (one an SM)
@@ -174,7 +107,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
     s.acc[tid] = 0;
     s.inc[tid] = 0;
     unsigned long long twice = 0;
-    const uint32_t n_heavy = *a.n_heavy;
+    const uint32_t n_heavy = a.n_heavy[64];
     if (tid == 0) s.u = atomicAdd(a.queue, 1u);
     __syncthreads();
     for (;;) {
@@ -183,7 +116,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
         __syncthreads();
         uint32_t next = 0;  // the following turn, asked for ahead
         if (tid == 0) next = atomicAdd(a.queue, 1u);
-        const uint32_t u = a.heavy[n_heavy - 1u - q];
+        const uint32_t u = a.heavy[q];
         if (u >= a.lo && u < a.hi) {
             const uint64_t arc = a.off[u];
             const uint32_t h = a.hv[u];
@@ -454,94 +387,332 @@ __global__ void __launch_bounds__(256) k_count_light(const __grid_constant__ Cou
     if (lane == 0 && twice) atomicAdd(&a.totals[0], twice);
 }
 
-// Emit the index: blooms (bloom number, first pair), twin pairs and the
-// per-edge link lists.  The dense per-block array holds one 64-bit word per
-// end vertex: the wedge count in the low half and, once the bloom is claimed,
-// 2 + its index among the vertex's blooms in the high half, so a wedge reads
-// and updates one word (one memory sector) in every pass.
-template <int NT>
-__global__ void __launch_bounds__(NT) k_emit(
-    const uint64_t *__restrict__ off, const uint32_t *__restrict__ adj,
-    const uint32_t *__restrict__ eid, const uint32_t *__restrict__ hv,
-    const uint32_t *__restrict__ pl, const uint64_t *__restrict__ wv, uint32_t n,
-    const uint32_t *__restrict__ vbase, uint32_t cn,
-    unsigned long long *cw_all, const uint64_t *__restrict__ bloom_base,
-    const uint64_t *__restrict__ pair_base, const uint64_t *__restrict__ inc_off,
-    uint32_t *inc_fill, uint32_t *bloom_k, uint32_t *bloom_off, uint2 *pairs,
-    uint2 *inc, uint32_t *queue, const uint8_t *__restrict__ assigned, bool twin) {
-    __shared__ Chunk<NT> ch;
-    __shared__ uint32_t s_q;
-    // bloom count (high 32 bits) and pair count (low 32 bits) of the vertex,
-    // advanced by one atomic so that pair ranges follow bloom ids
-    __shared__ unsigned long long s_alloc;
-    unsigned long long *cw = cw_all + (size_t)blockIdx.x * cn;
+// -------------------------------------------------------------------- emit
+// Emit the index: blooms (bloom number, first pair), twin pairs and the per-edge
+// link lists, by the tiers and with the counters of the count kernels.  Once the
+// counts of a start vertex are final, every end vertex w with two wedges or more
+// gets a bloom: its id and the end of its pair range go to one 64-bit word, from
+// whose low half each wedge takes its pair by an atomic.
+//
+// An edge is the first member of pairs of one start vertex only, its own higher
+// endpoint: those links fill its list from the front, counted in shared memory.
+// Links as second member come from many start vertices and fill it from the
+// back, by one atomic on a 64-bit cursor an edge that starts at the list's end.
+// What is left to bound it are the scattered 8-byte link stores and those cursors.
+struct EmitArgs {
+    CountArgs c;            // counters and graph (support, w2v, nbv unused)
+    unsigned long long *word;  // [blocks * cnt_n] (pair range end | bloom << 32) of an end vertex
+    uint32_t *found;        // [blocks * cold_n] end vertices below the hot ranks with a bloom
+    uint32_t cnt_n;
+    const uint64_t *bloom_base, *pair_base, *inc_off;
+    unsigned long long *cursor;  // [m] end of the free places of each edge's list
+    uint32_t *bloom_k, *bloom_off;
+    uint2 *pairs, *inc;
+    bool twin;
+};
+
+// A pair of bloom B in `slot`: euv is the first member, its link number `place`.
+__device__ __forceinline__ void put_pair(const EmitArgs &a, uint32_t slot, uint32_t B, uint32_t euv, uint32_t evw,
+                                         bool fu, bool fw, uint64_t at, unsigned long long back) {
+    // an assigned edge is flagged in bit 31 and gets no link
+    a.pairs[slot] = make_uint2(euv | (fu ? 0x80000000u : 0u), evw | (fw ? 0x80000000u : 0u));
+    // each link carries its bloom and which member of the pair the edge is, or
+    // the twin itself and the bloom
+    if (!fu) a.inc[at] = make_uint2(a.twin ? evw : slot, B);
+    if (!fw) a.inc[back - 1u] = make_uint2(a.twin ? euv : slot, B | (a.twin ? 0u : 0x80000000u));
+}
+
+struct EmitShared {
+    CountShared c;
+    unsigned long long front[kCT];  // first free place of (u, v)'s list
+    unsigned long long alloc;       // blooms (high) and pairs (low) of the start vertex handed out
+    uint32_t n_found;
+};
+// hot ranks of emit (its tables take more of the shared memory)
+constexpr uint32_t kHotE = 80 * 1024;
+
+// Blooms for the lanes whose end vertex w has c >= 2 wedges: id and pair range,
+// one shared atomic a warp.
+__device__ __forceinline__ void claim(const EmitArgs &a, unsigned long long *alloc, unsigned long long *word, uint32_t w,
+                                      uint32_t c, uint64_t bb, uint64_t pb) {
+    const uint32_t lane = threadIdx.x & 31;
+    const bool has = c >= 2u;
+    const unsigned m = __ballot_sync(0xffffffffu, has);
+    if (!m) return;
+    const uint32_t incl = dev::warp_incl_scan(has ? c : 0u), sum = __shfl_sync(0xffffffffu, incl, 31);
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(alloc, (unsigned long long)__popc(m) << 32 | sum);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (has) {
+        const uint32_t B = (uint32_t)bb + (uint32_t)(base >> 32) + __popc(m & ((1u << lane) - 1u));
+        const uint32_t end = (uint32_t)pb + (uint32_t)base + incl;
+        a.bloom_k[B] = c;
+        a.bloom_off[B] = end - c;
+        word[w] = (unsigned long long)B << 32 | end;
+    }
+}
+
+__global__ void __launch_bounds__(kCT) k_emit(const __grid_constant__ EmitArgs ea) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    EmitShared &es = *reinterpret_cast<EmitShared *>(s_dyn);
+    CountShared &s = es.c;
+    const CountArgs &a = ea.c;
+    uint32_t *hot = reinterpret_cast<uint32_t *>(s_dyn + sizeof(EmitShared));
+    uint32_t *cold = a.cold + (size_t)blockIdx.x * a.cold_n;
+    uint32_t *found = ea.found + (size_t)blockIdx.x * a.cold_n;
+    unsigned long long *word = ea.word + (size_t)blockIdx.x * ea.cnt_n;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t i = tid; i < kHotE / 2; i += kCT) hot[i] = 0;
+    const uint32_t n_heavy = a.n_heavy[64];
+    if (tid == 0) s.u = atomicAdd(a.queue, 1u);
+    __syncthreads();
     for (;;) {
-        uint32_t u = next_vertex(queue, 0u, n, &s_q);
-        if (u == 0xFFFFFFFFu) break;
-        if (wv[u] == 0) continue;
-        const uint64_t a = off[u];
-        const uint32_t h = hv[u];
-        const uint64_t bb = bloom_base[u];
-        const uint64_t pb = pair_base[u];
-        const uint32_t vb = vbase ? vbase[u] : 0u;
-        if (threadIdx.x == 0) s_alloc = 0;
-        pass_count64(ch, off, adj, eid, pl, a, h, cw, vb);
-        // claim: one thread per bloom allocates its id and pair range
-        for (uint32_t c0 = 0; c0 < h; c0 += NT) {
-            uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-            for (uint32_t t = threadIdx.x; t < T; t += NT) {
-                uint32_t vi;
-                uint64_t arc = wedge_arc(ch, off, t, vi);
-                const uint32_t w = adj[arc] - vb;  // counter index
-                const unsigned long long x = __ldcg(&cw[w]);
-                const uint32_t c = (uint32_t)x;
-                // a single wedge is the only reader of its word: clear it now
-                if (c == 1u) cw[w] = 0ull;
-                if (c >= 2 && atomicCAS(&cw[w], (unsigned long long)c, 1ull << 32 | c) == (unsigned long long)c) {
-                    unsigned long long old = atomicAdd(&s_alloc, (1ull << 32) | c);
-                    uint32_t j = (uint32_t)(old >> 32);
-                    uint32_t p = (uint32_t)old;
-                    uint64_t B = bb + j;
-                    bloom_k[B] = c;
-                    bloom_off[B] = (uint32_t)(pb + p);
-                    atomicExch(&cw[w], (unsigned long long)(j + 2u) << 32 | c);
+        const uint32_t q = s.u;
+        if (q >= n_heavy) break;
+        __syncthreads();
+        uint32_t next = 0;
+        if (tid == 0) {
+            next = atomicAdd(a.queue, 1u);
+            es.alloc = 0;
+            es.n_found = 0;
+        }
+        const uint32_t u = a.heavy[q];
+        const uint64_t arc = a.off[u], bb = ea.bloom_base[u], pb = ea.pair_base[u];
+        const uint32_t h = a.hv[u];
+        const uint32_t vb = a.vbase ? a.vbase[u] : 0u;
+        const bool narrow = h < 0x10000u;
+        const uint32_t width = narrow ? kHotE : kHotE / 2;
+        const uint32_t ru = u - vb;
+        const uint32_t base = ru > width ? ru - width : 0u;
+        __syncthreads();
+        // counts, as in k_count; end vertices of lower ranks with a bloom are listed
+        for (uint32_t c0 = 0; c0 < h; c0 += kCT) {
+            const uint32_t total = lay_wedges(s, a, arc, h, c0);
+            uint32_t lo, hi;
+            dev::share_of(total, warp, kCT / 32, lo, hi);
+            uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
+            for (uint32_t x0 = lo; x0 < hi; x0 += 32u * kCU) {
+                uint32_t w[kCU], old[kCU];
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    const uint32_t x = x0 + 32u * r + lane, j = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
+                    w[r] = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
                 }
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    old[r] = 0;
+                    if (w[r] == 0xFFFFFFFFu) continue;
+                    if (w[r] >= base) {
+                        const uint32_t i = w[r] - base;
+                        if (narrow) atomicAdd(&hot[i >> 1], 1u << (16u * (i & 1u)));
+                        else atomicAdd(&hot[i], 1u);
+                    } else {
+                        old[r] = atomicAdd(&cold[w[r]], 1u);
+                    }
+                }
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r)
+                    if (old[r] == 1u) found[atomicAdd(&es.n_found, 1u)] = w[r];
             }
             __syncthreads();
         }
-        // place each bloom wedge as a twin pair and link both edges to it
-        for (uint32_t c0 = 0; c0 < h; c0 += NT) {
-            uint32_t T = load_chunk(ch, adj, eid, pl, a, h, c0);
-            for (uint32_t t = threadIdx.x; t < T; t += NT) {
-                uint32_t vi;
-                uint64_t arc = wedge_arc(ch, off, t, vi);
-                const uint32_t w = adj[arc] - vb;  // counter index
-                const uint32_t x = (uint32_t)(__ldcg(&cw[w]) >> 32);
-                if (x >= 2) {
-                    uint64_t B = bb + (x - 2);
-                    // the low half counts down the bloom's wedges still to place
-                    uint32_t pos = (uint32_t)atomicAdd(&cw[w], ~0ull) - 1u;
-                    // the last wedge of the bloom comes after every read of the
-                    // word (each precedes its own decrement): clear it
-                    if (pos == 0u) cw[w] = 0ull;
-                    uint32_t slot = ld_cg(&bloom_off[B]) + pos;
-                    uint32_t euv = ch.e[vi], evw = eid[arc];
-                    const bool fu = assigned && assigned[euv], fw = assigned && assigned[evw];
-                    // an assigned edge is flagged in bit 31 and gets no link
-                    pairs[slot] = make_uint2(euv | (fu ? 0x80000000u : 0u), evw | (fw ? 0x80000000u : 0u));
-                    // each link carries its bloom and which member of the pair
-                    // the edge is, or the twin itself and the bloom
-                    if (!fu) {
-                        uint32_t q1 = atomicAdd(&inc_fill[euv], 1u);
-                        inc[inc_off[euv] + q1] = make_uint2(twin ? evw : slot, (uint32_t)B);
-                    }
-                    if (!fw) {
-                        uint32_t q2 = atomicAdd(&inc_fill[evw], 1u);
-                        inc[inc_off[evw] + q2] = make_uint2(twin ? euv : slot, (uint32_t)B | (twin ? 0u : 0x80000000u));
-                    }
-                }
+        // blooms
+        const uint32_t span = ru - base, n_found = es.n_found;
+        for (uint32_t i0 = 0; i0 < span; i0 += kCT) {
+            const uint32_t i = i0 + tid;
+            const uint32_t c = i >= span ? 0u : narrow ? hot[i >> 1] >> (16u * (i & 1u)) & 0xFFFFu : hot[i];
+            claim(ea, &es.alloc, word, base + i, c, bb, pb);
+        }
+        for (uint32_t i0 = 0; i0 < n_found; i0 += kCT) {
+            const uint32_t i = i0 + tid, w = i < n_found ? found[i] : 0u;
+            claim(ea, &es.alloc, word, w, i < n_found ? ld_cg(&cold[w]) : 0u, bb, pb);
+        }
+        __syncthreads();
+        // every bloom wedge becomes a twin pair linked to both edges
+        for (uint32_t c0 = 0; c0 < h; c0 += kCT) {
+            const uint32_t total = lay_wedges(s, a, arc, h, c0);
+            if (tid < s.n) {
+                es.front[tid] = ea.inc_off[s.e[tid]];
+                s.inc[tid] = a.assigned && a.assigned[s.e[tid]];
             }
             __syncthreads();
+            uint32_t lo, hi;
+            dev::share_of(total, warp, kCT / 32, lo, hi);
+            uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
+            for (uint32_t x0 = lo; x0 < hi; x0 += 32u * kCU) {
+                uint32_t w[kCU], jj[kCU], ev[kCU];
+                unsigned long long wd[kCU], back[kCU], at[kCU];
+                bool in[kCU];
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    const uint32_t x = x0 + 32u * r + lane;
+                    jj[r] = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
+                    w[r] = x < hi ? a.adj[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
+                }
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    uint32_t c = 0;
+                    if (w[r] != 0xFFFFFFFFu) {
+                        if (w[r] >= base) {
+                            const uint32_t i = w[r] - base;
+                            c = narrow ? hot[i >> 1] >> (16u * (i & 1u)) & 0xFFFFu : hot[i];
+                        } else {
+                            c = ld_cg(&cold[w[r]]);
+                            if (c == 1u) cold[w[r]] = 0u;  // its only reader
+                        }
+                    }
+                    in[r] = c >= 2u;
+                }
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    wd[r] = in[r] ? atomicAdd(&word[w[r]], ~0ull) : 0ull;  // the low half is never 0: no borrow
+                    ev[r] = in[r] ? a.eid[s.at[jj[r]] + x0 + 32u * r + lane] : 0u;
+                }
+                bool fu[kCU], fw[kCU];
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r) {
+                    fu[r] = s.inc[jj[r]] != 0u;
+                    fw[r] = in[r] && a.assigned && a.assigned[ev[r]];
+                    back[r] = in[r] && !fw[r] ? atomicAdd(&ea.cursor[ev[r]], ~0ull) : 0ull;
+                    at[r] = in[r] && !fu[r] ? atomicAdd(&es.front[jj[r]], 1ull) : 0ull;
+                }
+#pragma unroll
+                for (uint32_t r = 0; r < kCU; ++r)
+                    if (in[r])
+                        put_pair(ea, (uint32_t)wd[r] - 1u, (uint32_t)(wd[r] >> 32), s.e[jj[r]], ev[r], fu[r], fw[r],
+                                 at[r], back[r]);
+            }
+            __syncthreads();
+            if (tid < s.n) s.inc[tid] = 0;
+            __syncthreads();
+        }
+        // counters back to zero
+        for (uint32_t i = tid; i < n_found; i += kCT) cold[found[i]] = 0u;
+        const uint32_t used = narrow ? (span + 1u) / 2u : span;
+        for (uint32_t i = tid; i < used; i += kCT) hot[i] = 0;
+        if (tid == 0) s.u = next;
+        __syncthreads();
+    }
+}
+
+// Start vertices with few wedges, a warp each (as k_count_light).
+__global__ void __launch_bounds__(256) k_emit_light(const __grid_constant__ EmitArgs ea) {
+    constexpr uint32_t kSlots = 2 * kLightW, kWin = kLightW / 32, kWarps = 8;
+    constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+    __shared__ uint32_t s_key[kWarps][kSlots], s_cnt[kWarps][kSlots], s_bloom[kWarps][kSlots];
+    __shared__ uint32_t s_off[kWarps][33], s_e[kWarps][32];
+    __shared__ unsigned long long s_at[kWarps][33], s_front[kWarps][32];
+    const CountArgs &a = ea.c;
+    const uint32_t lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    uint32_t *key = s_key[wi], *cnt = s_cnt[wi], *bloom = s_bloom[wi], *off = s_off[wi];
+    for (uint32_t i = lane; i < kSlots; i += 32) {
+        key[i] = kEmpty;
+        cnt[i] = 0;
+    }
+    __syncwarp();
+    const uint32_t nw = gridDim.x * kWarps, ranks = a.hi - a.lo;
+    for (uint64_t g = blockIdx.x * kWarps + wi; g < ranks; g += 32ull * nw) {
+        bool light = false;
+        uint32_t my_h = 0, my_u = 0;
+        if (g + (uint64_t)lane * nw < ranks) {
+            my_u = a.lo + (uint32_t)(g + (uint64_t)lane * nw);
+            const uint64_t W = a.wv[my_u];
+            if (W > 1) {  // a bloom takes two wedges
+                my_h = a.hv[my_u];
+                light = is_light(W, my_h);
+            }
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, light);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const uint32_t u = __shfl_sync(0xffffffffu, my_u, src), h = __shfl_sync(0xffffffffu, my_h, src);
+            const uint64_t arc = a.off[u], bb = ea.bloom_base[u], pb = ea.pair_base[u];
+            uint32_t len = 0, e = 0;
+            uint64_t at = 0;
+            if (lane < h) {
+                len = a.pl[arc + lane];
+                if (len) {
+                    e = a.eid[arc + lane];
+                    at = a.off[a.adj[arc + lane]];
+                }
+            }
+            const unsigned has = __ballot_sync(0xffffffffu, len > 0u);
+            const uint32_t incl = dev::warp_incl_scan(len), total = __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t j = __popc(has & ((1u << lane) - 1u)), n = __popc(has);
+            if (len) {
+                off[j] = incl - len;
+                s_at[wi][j] = at - (incl - len);
+                s_e[wi][j] = e | (a.assigned && a.assigned[e] ? 0x80000000u : 0u);
+                s_front[wi][j] = ea.inc_off[e];
+            }
+            if (lane == 31) off[n] = total;
+            __syncwarp();
+            uint32_t slot[kWin], jj[kWin], j0 = 0;
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                slot[r] = kEmpty;
+                jj[r] = 0;
+                if (32u * r < total) {
+                    jj[r] = dev::items_of(off, n, 32u * r, j0);
+                    const uint32_t x = 32u * r + lane;
+                    if (x < total) slot[r] = a.adj[s_at[wi][jj[r]] + x];
+                }
+            }
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                if (slot[r] == kEmpty) continue;
+                const uint32_t w = slot[r];
+                uint32_t i = (w * 0x9E3779B1u) >> 23;
+                for (;;) {
+                    const uint32_t k = atomicCAS(&key[i], kEmpty, w);
+                    if (k == kEmpty || k == w) break;
+                    i = (i + 1u) & (kSlots - 1u);
+                }
+                slot[r] = i;
+                atomicAdd(&cnt[i], 1u);
+            }
+            __syncwarp();
+            // blooms: cnt becomes the end of the pair range (0: none)
+            uint32_t nb = 0, np = 0;
+            for (uint32_t i0 = 0; i0 < kSlots; i0 += 32) {
+                const uint32_t c = cnt[i0 + lane];
+                const bool b = c >= 2u;
+                const unsigned m = __ballot_sync(0xffffffffu, b);
+                const uint32_t pi = dev::warp_incl_scan(b ? c : 0u);
+                if (b) {
+                    const uint32_t B = (uint32_t)bb + nb + __popc(m & ((1u << lane) - 1u));
+                    const uint32_t end = (uint32_t)pb + np + pi;
+                    ea.bloom_k[B] = c;
+                    ea.bloom_off[B] = end - c;
+                    bloom[i0 + lane] = B;
+                    cnt[i0 + lane] = end;
+                } else if (c) {
+                    cnt[i0 + lane] = 0;
+                }
+                nb += __popc(m);
+                np += __shfl_sync(0xffffffffu, pi, 31);
+            }
+            __syncwarp();
+            // (the pair ranges of a bloom end above 0, and count down within them)
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r) {
+                if (slot[r] == kEmpty || cnt[slot[r]] == 0u) continue;
+                const uint32_t p = atomicSub(&cnt[slot[r]], 1u) - 1u, x = 32u * r + lane;
+                const uint32_t ev = a.eid[s_at[wi][jj[r]] + x], eu = s_e[wi][jj[r]];
+                const bool fu = eu >> 31, fw = a.assigned && a.assigned[ev];
+                const unsigned long long back = fw ? 0ull : atomicAdd(&ea.cursor[ev], ~0ull);
+                const unsigned long long front = fu ? 0ull : atomicAdd(&s_front[wi][jj[r]], 1ull);
+                put_pair(ea, p, bloom[slot[r]], eu & 0x7FFFFFFFu, ev, fu, fw, front, back);
+            }
+            __syncwarp();
+#pragma unroll
+            for (uint32_t r = 0; r < kWin; ++r)
+                if (slot[r] != kEmpty) {
+                    key[slot[r]] = kEmpty;
+                    cnt[slot[r]] = 0;
+                }
+            __syncwarp();
         }
     }
 }
@@ -605,9 +776,7 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     return cudaSuccess;
 }
 
-cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, Alloc &al,
-                       cudaStream_t stream, int nt) {
-    if (nt != 256 && nt != 1024) nt = 512;
+cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, Alloc &al, cudaStream_t stream) {
     const uint32_t n = g.n;
     const uint64_t m = g.m;
     ix.m = m;
@@ -623,7 +792,6 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     BT_CUDA(widen_u32(c.inc_cnt, incc64, m, al));
     BT_CUDA(cudaMemsetAsync(incc64 + m, 0, sizeof(uint64_t), al.stream));
     BT_CUDA(exclusive_scan_u64(incc64, ix.inc_off, m + 1, tot + 2, al));
-    al.put(incc64);
     uint64_t h_tot[3];
     BT_CUDA(cudaMemcpyAsync(h_tot, tot, sizeof(h_tot), cudaMemcpyDeviceToHost, stream));
     BT_CUDA(cudaStreamSynchronize(stream));
@@ -635,43 +803,66 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
         al.put(bloom_base);
         al.put(pair_base);
         al.put(tot);
+        al.put(incc64);
         return cudaErrorInvalidValue;  // reported as overflow by the caller
     }
     ix.bloom_k = al.get<uint32_t>(ix.nb);
     ix.bloom_off = al.get<uint32_t>(ix.nb + 1);
     ix.pairs = al.get<uint2>(ix.w2);
     ix.inc = al.get<uint2>(ix.links);
-    uint32_t *inc_fill = al.get<uint32_t>(m);
-    // as few resident blocks as keep the SMs busy, so that few of their dense
-    // arrays compete for L2 (1024 threads: one block an SM measured 5-20 % faster
-    // than two; a batch of 384 graphs with 256 threads: 8.7 ms with six, 10.0 with eight)
-    const int bps = nt == 1024 ? 1 : nt == 512 ? 3 : 6;
-    unsigned blocks = (unsigned)(num_sms * bps);
-    unsigned long long *cw = al.get<unsigned long long>((size_t)blocks * g.cnt_n);
-    uint32_t *queue = al.get<uint32_t>(1);
+    const unsigned blocks = (unsigned)num_sms;
+    EmitArgs a{};
+    a.c.off = g.off;
+    a.c.adj = g.adj;
+    a.c.eid = g.eid;
+    a.c.hv = g.hv;
+    a.c.pl = g.pl;
+    a.c.wv = g.wv;
+    a.c.hi = n;
+    a.c.heavy = g.heavy;
+    a.c.n_heavy = g.n_heavy;
+    a.c.vbase = g.vbase;
+    const uint32_t width = g.cnt_n < 0x10000u ? kHotE : kHotE / 2;  // as in count_wedges
+    a.c.cold_n = g.cnt_n > width ? g.cnt_n - width : 0u;
+    a.c.cold = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
+    a.c.queue = al.get<uint32_t>(1);
+    a.c.assigned = c.assigned;
+    a.word = al.get<unsigned long long>((size_t)blocks * g.cnt_n);
+    a.found = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
     if (al.err != cudaSuccess) return al.err;
+    a.cnt_n = g.cnt_n;
+    a.bloom_base = bloom_base;
+    a.pair_base = pair_base;
+    a.inc_off = ix.inc_off;
+    a.cursor = reinterpret_cast<unsigned long long *>(incc64);
+    a.bloom_k = ix.bloom_k;
+    a.bloom_off = ix.bloom_off;
+    a.pairs = ix.pairs;
+    a.inc = ix.inc;
+    a.twin = ix.twin_links;
     uint32_t w2_32 = (uint32_t)ix.w2;
     BT_CUDA(cudaMemcpyAsync(ix.bloom_off + ix.nb, &w2_32, sizeof(uint32_t), cudaMemcpyHostToDevice,
                             stream));
-    BT_CUDA(cudaMemsetAsync(inc_fill, 0, sizeof(uint32_t) * m, al.stream));
-    BT_CUDA(cudaMemsetAsync(cw, 0, sizeof(unsigned long long) * (size_t)blocks * g.cnt_n, al.stream));
-    BT_CUDA(cudaMemsetAsync(queue, 0, sizeof(uint32_t), al.stream));
+    // the lists are filled from their ends too
+    BT_CUDA(cudaMemcpyAsync(a.cursor, ix.inc_off + 1, sizeof(uint64_t) * m, cudaMemcpyDeviceToDevice, al.stream));
+    if (a.c.cold_n) BT_CUDA(cudaMemsetAsync(a.c.cold, 0, sizeof(uint32_t) * (size_t)blocks * a.c.cold_n, al.stream));
+    BT_CUDA(cudaMemsetAsync(a.c.queue, 0, sizeof(uint32_t), al.stream));
+    const size_t smem = sizeof(EmitShared) + kHotE * sizeof(uint16_t);
+    const unsigned groups = (n + 7u) / 8u, room = (unsigned)num_sms * 4u;
     al.mark(kPhEmit, false);
-#define BT_EMIT_ARGS                                                                         \
-    g.off, g.adj, g.eid, g.hv, g.pl, g.wv, n, g.vbase, g.cnt_n, cw, bloom_base, pair_base, ix.inc_off,  \
-        inc_fill, ix.bloom_k, ix.bloom_off, ix.pairs, ix.inc, queue, c.assigned, ix.twin_links
-    if (nt == 256) k_emit<256><<<blocks, 256, 0, al.stream>>>(BT_EMIT_ARGS);
-    else if (nt == 1024) k_emit<1024><<<blocks, 1024, 0, al.stream>>>(BT_EMIT_ARGS);
-    else k_emit<512><<<blocks, 512, 0, al.stream>>>(BT_EMIT_ARGS);
-#undef BT_EMIT_ARGS
-    al.launches++;
+    BT_CUDA(cudaFuncSetAttribute(k_emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_emit<<<blocks, kCT, smem, al.stream>>>(a);
+    k_emit_light<<<groups < room ? (groups ? groups : 1u) : room, 256, 0, al.stream>>>(a);
+    al.launches += 2;
     al.mark(kPhEmit, true);
     BT_CUDA(cudaGetLastError());
     // the host copy of w2_32 must outlive the async copy
     BT_CUDA(cudaStreamSynchronize(stream));
-    al.put(cw);
-    al.put(queue);
-    al.put(inc_fill);
+    al.put(a.c.cold);
+    al.put(a.c.queue);
+    al.put(a.word);
+    al.put(a.found);
+    al.put(incc64);
     al.put(bloom_base);
     al.put(pair_base);
     al.put(tot);

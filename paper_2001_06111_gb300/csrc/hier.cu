@@ -11,74 +11,64 @@
 namespace bt {
 namespace {
 
-// keys sort ascending, so the complement of phi puts the largest phi first;
-// the stable radix sort keeps equal phi in input order
-__global__ void k_hier_keys(const uint32_t *phi, uint64_t m, uint32_t *keys, uint32_t *vals) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        keys[i] = ~phi[i];
-        vals[i] = (uint32_t)i;
+constexpr int kHT = 256, kHR = 16, kHTile = kHT * kHR;
+
+// Entries >= k of each tile of kHTile.
+__global__ void __launch_bounds__(kHT) k_count_ge(const uint32_t *phi, uint64_t m, uint32_t k, uint32_t *count) {
+    const uint64_t base = (uint64_t)blockIdx.x * kHTile;
+    uint32_t n = 0;
+#pragma unroll
+    for (int r = 0; r < kHR; ++r) {
+        const uint64_t i = base + (uint64_t)r * kHT + threadIdx.x;
+        n += i < m && phi[i] >= k;
     }
+    n = dev::block_sum(n);
+    if (threadIdx.x == 0) count[blockIdx.x] = n;
 }
 
-__global__ void k_hier_phi(const uint32_t *keys, uint64_t m, uint32_t *phi_sorted) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        phi_sorted[i] = ~keys[i];
-}
-
-__global__ void k_flag_ge(const uint32_t *phi, uint64_t m, uint32_t k, uint32_t *flag) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        flag[i] = phi[i] >= k ? 1u : 0u;
-}
-
-__global__ void k_compact(const uint32_t *phi, const uint32_t *pos, uint64_t m, uint32_t k, uint32_t *out) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        if (phi[i] >= k) out[pos[i]] = (uint32_t)i;
-}
-
-inline unsigned grid_for(uint64_t items, int threads) {
-    uint64_t g = (items + threads - 1) / threads;
-    if (g == 0) g = 1;
-    return (unsigned)(g < 152 * 32 ? g : 152 * 32);
+// Their places, ascending: a warp takes 512 neighbouring entries.
+__global__ void __launch_bounds__(kHT) k_write_ge(const uint32_t *phi, uint64_t m, uint32_t k, const uint32_t *first,
+                                                  uint32_t *out) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t base = (uint64_t)blockIdx.x * kHTile + warp * (32 * kHR);
+    unsigned mask[kHR];
+    uint32_t n = 0;
+#pragma unroll
+    for (int r = 0; r < kHR; ++r) {
+        const uint64_t i = base + 32u * r + lane;
+        mask[r] = __ballot_sync(0xffffffffu, i < m && phi[i] >= k);
+        n += __popc(mask[r]);
+    }
+    __shared__ uint32_t s_n[kHT / 32];
+    if (lane == 0) s_n[warp] = n;
+    __syncthreads();
+    uint32_t at = first[blockIdx.x];
+    for (uint32_t w = 0; w < warp; ++w) at += s_n[w];
+#pragma unroll
+    for (int r = 0; r < kHR; ++r) {
+        if (mask[r] >> lane & 1u) out[at + __popc(mask[r] & ((1u << lane) - 1u))] = (uint32_t)(base + 32u * r + lane);
+        at += __popc(mask[r]);
+    }
 }
 
 }  // namespace
 
 cudaError_t hierarchy_order(const uint32_t *phi, uint64_t m, uint32_t *order, uint32_t *phi_sorted, Alloc &al) {
-    if (m == 0) return cudaSuccess;
-    uint32_t *keys = al.get<uint32_t>(m);
-    uint32_t *tk = al.get<uint32_t>(m);
-    uint32_t *tv = al.get<uint32_t>(m);
-    if (al.err != cudaSuccess) return al.err;
-    k_hier_keys<<<grid_for(m, 256), 256, 0, al.stream>>>(phi, m, keys, order);
-    al.launches++;
-    BT_CUDA(radix_sort_u32(keys, order, tk, tv, m, 32, al));
-    if (phi_sorted) {
-        k_hier_phi<<<grid_for(m, 256), 256, 0, al.stream>>>(keys, m, phi_sorted);
-        al.launches++;
-    }
-    al.put(keys);
-    al.put(tk);
-    al.put(tv);
-    return cudaGetLastError();
+    return radix_order_desc_u32(phi, m, order, phi_sorted, al);
 }
 
 cudaError_t select_ge(const uint32_t *phi, uint64_t m, uint32_t k, uint32_t *out, uint32_t *d_count,
                       Alloc &al) {
     if (m == 0) return cudaMemsetAsync(d_count, 0, sizeof(uint32_t), al.stream);
-    uint32_t *flag = al.get<uint32_t>(m);
-    uint32_t *pos = al.get<uint32_t>(m);
+    const uint32_t tiles = (uint32_t)((m + kHTile - 1) / kHTile);
+    uint32_t *count = al.get<uint32_t>(tiles);
     if (al.err != cudaSuccess) return al.err;
-    k_flag_ge<<<grid_for(m, 256), 256, 0, al.stream>>>(phi, m, k, flag);
+    k_count_ge<<<tiles, kHT, 0, al.stream>>>(phi, m, k, count);
     al.launches++;
-    BT_CUDA(exclusive_scan_u32(flag, pos, m, d_count, al));
-    k_compact<<<grid_for(m, 256), 256, 0, al.stream>>>(phi, pos, m, k, out);
+    BT_CUDA(exclusive_scan_u32(count, count, tiles, d_count, al));
+    k_write_ge<<<tiles, kHT, 0, al.stream>>>(phi, m, k, count, out);
     al.launches++;
-    al.put(flag);
-    al.put(pos);
+    al.put(count);
     return cudaGetLastError();
 }
 

@@ -104,57 +104,103 @@ constexpr int kSortRounds = 16;
 constexpr int kSortTile = kSortThreads * kSortRounds;
 
 template <typename K>
-__global__ void k_radix_hist(const K *keys, size_t n, int shift, uint32_t *hist, uint32_t ntiles) {
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K *keys, K xin, size_t n, int shift,
+                                                             uint32_t *hist, uint32_t ntiles) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    size_t base = (size_t)blockIdx.x * kSortTile;
+    const size_t base = (size_t)blockIdx.x * kSortTile;
+    K k[kSortRounds];
+#pragma unroll
     for (int r = 0; r < kSortRounds; ++r) {
-        size_t idx = base + (size_t)r * kSortThreads + threadIdx.x;
-        if (idx < n) atomicAdd(&h[(uint32_t)(keys[idx] >> shift) & 255u], 1u);
+        const size_t idx = base + (size_t)r * kSortThreads + threadIdx.x;
+        k[r] = idx < n ? keys[idx] ^ xin : K(0);
     }
+#pragma unroll
+    for (int r = 0; r < kSortRounds; ++r)
+        if (base + (size_t)r * kSortThreads + threadIdx.x < n) atomicAdd(&h[(uint32_t)(k[r] >> shift) & 255u], 1u);
     __syncthreads();
     hist[(size_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-// Stable scatter: items of a tile keep their input order within a digit.
+// Stable scatter: items of a tile keep their input order within a digit.  A warp
+// ranks its 512 neighbouring items by itself (16 turns, counters of its own, no
+// block barrier), the tile is put in digit order in shared memory, and every
+// digit's run goes out in one piece: bound by the bytes in and out.  Ranking the
+// tile in turns of the whole block with four barriers each, and writing from
+// there, took 1.1 ms a pass for 60M 64-bit keys, which now take 0.9.
 template <typename K>
-__global__ void k_radix_scatter(const K *kin, const uint32_t *vin, K *kout, uint32_t *vout,
-                                size_t n, int shift, const uint32_t *offs, uint32_t ntiles) {
-    __shared__ uint32_t s_base[256];
-    __shared__ uint32_t s_wcnt[kSortThreads / 32][256];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    s_base[tid] = offs[(size_t)tid * ntiles + blockIdx.x];
-    for (int w = 0; w < kSortThreads / 32; ++w) s_wcnt[w][tid] = 0;
+struct SortShared {
+    K key[kSortTile];
+    uint32_t val[kSortTile];
+    uint32_t cnt[kSortThreads / 32][256];  // a warp's counts, then its first place, by digit
+    uint32_t start[256], to[256];          // a digit's first place in the tile, and in the output less that
+};
+
+// Keys are read xor xin and written xor xout (kout null: not at all); vin null:
+// the values are the places.
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K *kin, K xin, const uint32_t *vin, K *kout,
+                                                                K xout, uint32_t *vout, size_t n, int shift,
+                                                                const uint32_t *offs, uint32_t ntiles) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    SortShared<K> &s = *reinterpret_cast<SortShared<K> *>(s_dyn);
+    constexpr int kWarps = kSortThreads / 32;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int w = 0; w < kWarps; ++w) s.cnt[w][tid] = 0;
+    const uint32_t first = offs[(size_t)tid * ntiles + blockIdx.x];
     __syncthreads();
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    size_t base = (size_t)blockIdx.x * kSortTile;
+    const size_t base = (size_t)blockIdx.x * kSortTile, mine = base + (size_t)warp * (32 * kSortRounds) + lane;
+    K key[kSortRounds];
+    uint32_t val[kSortRounds], rank[kSortRounds];
+#pragma unroll
     for (int r = 0; r < kSortRounds; ++r) {
-        size_t idx = base + (size_t)r * kSortThreads + tid;
-        bool valid = idx < n;
-        K key = valid ? kin[idx] : K(0);
-        uint32_t val = valid ? vin[idx] : 0u;
-        uint32_t d = valid ? ((uint32_t)(key >> shift) & 255u) : 256u;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t lrank = __popc(peers & lt_mask);
-        if (valid && lrank == 0) s_wcnt[warp][d] = __popc(peers);
-        __syncthreads();
+        const size_t idx = mine + 32u * r;
+        key[r] = idx < n ? kin[idx] ^ xin : K(0);
+        val[r] = idx >= n ? 0u : vin ? vin[idx] : (uint32_t)idx;
+    }
+    uint32_t *cnt = s.cnt[warp];
+#pragma unroll
+    for (int r = 0; r < kSortRounds; ++r) {
+        const bool valid = mine + 32u * r < n;
+        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 256u);
+        const uint32_t before = valid ? cnt[d] : 0u;
+        __syncwarp();
+        const uint32_t at = __popc(peers & ((1u << lane) - 1u));
+        if (valid && at == 0) cnt[d] = before + __popc(peers);
+        __syncwarp();
+        rank[r] = before + at;
+    }
+    __syncthreads();
+    {
         uint32_t run = 0;
-        for (int w = 0; w < kSortThreads / 32; ++w) {
-            uint32_t c = s_wcnt[w][tid];
-            s_wcnt[w][tid] = run;
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t c = s.cnt[w][tid];
+            s.cnt[w][tid] = run;
             run += c;
         }
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = s_base[d] + s_wcnt[warp][d] + lrank;
-            kout[pos] = key;
-            vout[pos] = val;
-        }
-        __syncthreads();
-        s_base[tid] += run;
-        for (int w = 0; w < kSortThreads / 32; ++w) s_wcnt[w][tid] = 0;
-        __syncthreads();
+        uint32_t total;
+        const uint32_t st = block_excl_scan<uint32_t>(run, &total);
+        s.start[tid] = st;
+        s.to[tid] = first - st;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortRounds; ++r) {
+        if (mine + 32u * r >= n) continue;
+        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+        const uint32_t pos = s.start[d] + cnt[d] + rank[r];
+        s.key[pos] = key[r];
+        s.val[pos] = val[r];
+    }
+    __syncthreads();
+    const uint32_t have = n - base < (size_t)kSortTile ? (uint32_t)(n - base) : (uint32_t)kSortTile;
+    for (uint32_t i = tid; i < have; i += kSortThreads) {
+        const K k = s.key[i];
+        const uint32_t pos = s.to[(uint32_t)(k >> shift) & 255u] + i;
+        if (kout) kout[pos] = k ^ xout;
+        vout[pos] = s.val[i];
     }
 }
 
@@ -168,14 +214,16 @@ cudaError_t radix_impl(K *keys, uint32_t *vals, K *tk, uint32_t *tv, size_t n, i
     K *ka = keys, *kb = tk;
     uint32_t *va = vals, *vb = tv;
     int passes = (bits + 7) / 8;
+    BT_CUDA(cudaFuncSetAttribute(k_radix_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(SortShared<K>)));
     for (int p = 0; p < passes; ++p) {
         int shift = 8 * p;
-        k_radix_hist<K><<<ntiles, kSortThreads, 0, al.stream>>>(ka, n, shift, hist, ntiles);
+        k_radix_hist<K><<<ntiles, kSortThreads, 0, al.stream>>>(ka, K(0), n, shift, hist, ntiles);
         al.launches++;
         cudaError_t e = scan_impl<uint32_t>(hist, hist, (size_t)256 * ntiles, nullptr, al);
         if (e != cudaSuccess) return e;
-        k_radix_scatter<K><<<ntiles, kSortThreads, 0, al.stream>>>(ka, va, kb, vb, n, shift, hist,
-                                                                    ntiles);
+        k_radix_scatter<K><<<ntiles, kSortThreads, sizeof(SortShared<K>), al.stream>>>(ka, K(0), va, kb, K(0), vb, n,
+                                                                                       shift, hist, ntiles);
         al.launches++;
         K *t = ka; ka = kb; kb = t;
         uint32_t *u = va; va = vb; vb = u;
@@ -216,6 +264,32 @@ cudaError_t exclusive_scan_u64(const uint64_t *in, uint64_t *out, size_t n, uint
 cudaError_t radix_sort_u32(uint32_t *keys, uint32_t *vals, uint32_t *tk, uint32_t *tv, size_t n,
                            int bits, Alloc &al) {
     return radix_impl<uint32_t>(keys, vals, tk, tv, n, bits, al);
+}
+cudaError_t radix_order_desc_u32(const uint32_t *keys, size_t n, uint32_t *order, uint32_t *sorted, Alloc &al) {
+    if (n == 0) return cudaSuccess;
+    const uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
+    uint32_t *hist = al.get<uint32_t>((size_t)256 * ntiles);
+    uint32_t *ka = al.get<uint32_t>(n), *va = al.get<uint32_t>(n), *kb = al.get<uint32_t>(n);
+    if (al.err != cudaSuccess) return al.err;
+    const size_t smem = sizeof(SortShared<uint32_t>);
+    BT_CUDA(cudaFuncSetAttribute(k_radix_scatter<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // keys -> a -> (kb, order) -> a -> (sorted, order)
+    for (int p = 0; p < 4; ++p) {
+        const uint32_t *kin = p == 0 ? keys : p == 2 ? kb : ka, *vin = p == 0 ? nullptr : p == 2 ? order : va;
+        uint32_t *kout = p == 3 ? sorted : p == 1 ? kb : ka, *vout = p & 1 ? order : va;
+        const uint32_t xin = p == 0 ? ~0u : 0u, xout = p == 3 ? ~0u : 0u;
+        k_radix_hist<uint32_t><<<ntiles, kSortThreads, 0, al.stream>>>(kin, xin, n, 8 * p, hist, ntiles);
+        cudaError_t e = scan_impl<uint32_t>(hist, hist, (size_t)256 * ntiles, nullptr, al);
+        if (e != cudaSuccess) return e;
+        k_radix_scatter<uint32_t><<<ntiles, kSortThreads, smem, al.stream>>>(kin, xin, vin, kout, xout, vout, n, 8 * p,
+                                                                             hist, ntiles);
+        al.launches += 2;
+    }
+    al.put(hist);
+    al.put(ka);
+    al.put(va);
+    al.put(kb);
+    return cudaGetLastError();
 }
 cudaError_t radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t *tk, uint32_t *tv, size_t n,
                            int bits, Alloc &al) {
