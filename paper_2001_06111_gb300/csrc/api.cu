@@ -538,38 +538,49 @@ static int build_index_impl(bt_handle *h, const int32_t *edges, uint64_t m, uint
 // Whether a peel of m edges runs as one part (the index then has twin links).
 static bool as_one_part(const bt_handle *h, uint64_t m) { return !grid_peel_only(h) && m <= kWholeEdges; }
 
-// Peels the handle's index: its edges are first told apart by ranges of bitruss
+// Peels index ix by parts: its edges are first told apart by ranges of bitruss
 // numbers (a coarse peel by the whole grid), then the ranges are peeled
-// independently of one another (local.cu).
-static cudaError_t peel_index(bt_handle *h, const uint64_t *sup, uint32_t *phi, bt::PeelResult &pr, int seg,
-                              bt::Alloc &al) {
-    const bt::Index &ix = h->index;
-    if (grid_peel_only(h)) return bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg);
+// independently of one another (local.cu).  pc: the limits of a pass of the
+// progressive compression, or null.
+static cudaError_t peel_by_parts(bt_handle *h, const bt::Index &ix, const uint64_t *sup, uint32_t *phi,
+                                 bt::PeelResult &pr, int seg, const bt::PeelOpts *pc, bt::Alloc &al) {
     bt::PartGraph g;
     cudaError_t e = cudaSuccess;
     const size_t held = al.live.size();
     al.mark(bt::kPhPeel, false);
     if (ix.twin_links) {
         e = bt::one_part(ix, sup, g, peel_sms(h), al);
-        if (e == cudaSuccess) e = bt::peel_parts(g, phi, pr, peel_sms(h), al);
+        if (e == cudaSuccess) e = bt::peel_parts(g, phi, 0, pr, peel_sms(h), al);
     } else {
         uint32_t *part = al.get<uint32_t>(ix.m);
         int *snap = al.get<int>(ix.m);
         e = al.err;
         bt::PeelOpts o;
+        if (pc) o = *pc;
+        o.assign_from = 0;
         o.snap = snap;
         o.max_parts = bt::kPartsMax;
         // more parts cost the coarse peel more rounds, fewer leave SMs idle in
         // the fine one; the best counts grew with the cube root of the twin
         // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150)
         o.parts_hint = (uint32_t)(0.305 * std::cbrt((double)ix.w2)) + 1;
-        if (e == cudaSuccess) e = bt::peel(ix, sup, part, pr, peel_sms(h), al, seg, &o);
-        if (e == cudaSuccess && pr.status == BT_OK) {
-            const bt::PeelResult coarse = pr;
-            e = bt::parts_of_ranges(ix, part, snap, coarse.parts, g, peel_sms(h), al);
-            if (e == cudaSuccess) e = bt::peel_parts(g, phi, pr, peel_sms(h), al);
-            pr.slots += coarse.slots;
-            pr.scanned += coarse.scanned;
+        bt::PeelResult c;
+        if (e == cudaSuccess) e = bt::peel(ix, sup, part, c, peel_sms(h), al, seg, &o);
+        pr = bt::PeelResult{};
+        pr.status = c.status;
+        if (e == cudaSuccess && c.status == BT_OK) {
+            // a pass's first part lies below the level from which phi is recorded
+            const bool first = o.k_init > 0;
+            e = bt::parts_of_ranges(ix, part, snap, c.parts, o.assigned, first, g, peel_sms(h), al);
+            if (e == cudaSuccess && g.np > 0)
+                e = bt::peel_parts(g, phi, pc ? pc->assign_from : 0, pr, peel_sms(h), al);
+            pr.rounds += c.first_rounds;
+            pr.levels += c.first_levels;
+            pr.updates += c.first_updates;
+            const uint64_t lim = h->limits.peel_round_limit;
+            if (lim && pr.rounds > lim + 1 && pr.status == BT_OK) pr.status = BT_ERR_NOCONVERGE;
+            pr.slots += c.slots;
+            pr.scanned += c.scanned;
         }
         al.put(part);
         al.put(snap);
@@ -582,10 +593,17 @@ static cudaError_t peel_index(bt_handle *h, const uint64_t *sup, uint32_t *phi, 
         al.undo_to(held);
         al.err = cudaSuccess;
         e = cudaStreamSynchronize(h->stream);
-        return e == cudaSuccess ? bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg) : e;
+        return e == cudaSuccess ? bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg, pc) : e;
     }
     bt::free_parts(g, al);
     return e;
+}
+
+// Peels the handle's index.
+static cudaError_t peel_index(bt_handle *h, const uint64_t *sup, uint32_t *phi, bt::PeelResult &pr, int seg,
+                              bt::Alloc &al) {
+    if (grid_peel_only(h)) return bt::peel(h->index, sup, phi, pr, peel_sms(h), al, seg);
+    return peel_by_parts(h, h->index, sup, phi, pr, seg, nullptr, al);
 }
 
 int bt_build_index(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL,
@@ -1229,7 +1247,11 @@ int bt_decompose_progressive(bt_handle *h, const int32_t *edges, uint64_t m, uin
                 o.k_init = (!recount && eps > 0) ? (long long)eps - 1 : 0;
                 o.assign_from = (long long)eps;
                 e = cudaMemsetAsync(phi_local, 0xFF, 4 * pc_n, h->stream);
-                if (e == cudaSuccess) e = bt::peel(ix, sup_c, phi_local, pr, peel_sms(h), al, h->peel_seg, &o);
+                // (a pass over few edges is over before its parts would be made)
+                const bool parts = !grid_peel_only(h) && o.m_active > kWholeEdges;
+                if (e == cudaSuccess)
+                    e = parts ? peel_by_parts(h, ix, sup_c, phi_local, pr, h->peel_seg, &o, al)
+                              : bt::peel(ix, sup_c, phi_local, pr, peel_sms(h), al, h->peel_seg, &o);
                 if (e == cudaSuccess) e = bt::gather_u32(phi_local, ix.newid, phi_c, pc_n, al);
                 if (e == cudaSuccess) e = bt::settle(pc_map, pc_n, pc_ass, phi_c, d_phi, d_asg, al);
                 if (e != cudaSuccess) rc = cuda_fail(h, e, "peeling a candidate subgraph");

@@ -256,6 +256,8 @@ struct PeelResult {
     uint64_t rounds = 0, levels = 0, updates = 0, kmax = 0, windows = 0, slots = 0, scanned = 0;
     uint64_t inc_phases = 0;  // rounds that ran a separate incidence phase
     uint32_t parts = 0;       // coarse peel: parts made
+    // coarse peel with k_init: rounds, levels and updates of the first part
+    uint64_t first_rounds = 0, first_levels = 0, first_updates = 0;
     int status = BT_OK;
 };
 // support: [m] initial supports (device, preserved); phi_out: [m] device.
@@ -271,7 +273,8 @@ struct PeelOpts {
     // bitruss number falls in.  A level is a range of bitruss numbers that
     // aims at 1/parts_hint of all links and edges; phi_out receives the part of every edge (parts
     // ascend with phi) and snap its support when its part began, all edges of
-    // lower parts being gone.
+    // lower parts being gone.  With k_init > 0 the first part is every edge up to
+    // k_init (it may be empty), in the batches of the fine peel.
     int *snap = nullptr;
     uint32_t parts_hint = 0, max_parts = 0;
 };
@@ -284,14 +287,18 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
 // and touches at most part_b[p + 1] - part_b[p] blooms.
 constexpr uint32_t kBlockEdges = 43008;  // edges of a part whose supports fit one block's shared memory
 constexpr uint32_t kPartsMax = 1024;     // parts of a coarse peel
-// A bloom inside a part, one 32-byte sector.
+constexpr uint32_t kAssigned = 0xFFFFFFFFu;  // an edge whose bitruss number is known, as a twin
+// A bloom inside a part, one 32-byte sector.  With assigned edges, those among
+// the pairs of higher parts are counted in `first` (n <= 2) or pair[0].x.
 struct __align__(32) BloomRec {
     uint32_t first, n;   // its pairs: here if n <= 2, else from pairs[first]
     uint32_t k, c;       // k_B, pairs that died in the current round
     uint2 pair[2];
 };
 struct PartGraph {
-    uint64_t m = 0, nb = 0;
+    uint64_t m = 0, nb = 0;   // edges of all parts (assigned edges are in none)
+    uint64_t deep = 0;        // edges of the graph: supports are below it
+    bool assigned = false;    // some twins are assigned edges (kAssigned); records count their place
     uint32_t np = 0;
     const uint32_t *part_e = nullptr, *part_b = nullptr;  // [np + 1]
     const uint32_t *order = nullptr;  // [np] parts in the order they are taken (null: last first)
@@ -313,11 +320,13 @@ void free_parts(PartGraph &g, Alloc &al);
 // The whole graph as one part (an index with twin links).
 cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al);
 // The ranges of a coarse peel as parts: part[e] in [0, np), snap[e] the support
-// of e when its part begins.
-cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np, PartGraph &g,
-                            int num_sms, Alloc &al);
-// Peel of all parts.
-cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, PeelResult &res, int num_sms, Alloc &al);
+// of e when its part begins.  assigned (nullable): edges that are in no part.
+// skip_first: part 0 is not to be peeled.
+cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
+                            const uint8_t *assigned, bool skip_first, PartGraph &g, int num_sms, Alloc &al);
+// Peel of all parts; phi_out receives bitruss numbers of at least assign_from.
+cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_from, PeelResult &res, int num_sms,
+                       Alloc &al);
 
 // ---------------------------------------------------------------- serving
 // The peel of handle h spans 1/ways of the SMs (server workers share the GPU).

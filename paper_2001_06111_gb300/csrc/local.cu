@@ -86,6 +86,8 @@ struct LocalArgs {
     unsigned long long *stats;  // updates, pair slots, scanned entries
     uint32_t *err;
     uint64_t round_limit;
+    long long assign_from;
+    bool assigned;  // some twins are assigned edges: no update is counted for them
 };
 
 struct Shared {
@@ -187,7 +189,7 @@ struct Part {
     // Edge e joins, as number j, the batch that starts at place `base` of the queue.
     __device__ __forceinline__ void settle(uint32_t e, uint32_t stamp, uint32_t base, uint32_t j) {
         if constexpr (!kS) st[e] = stamp;
-        a.phi[e0 + e] = (uint32_t)k;
+        if (k >= a.assign_from) a.phi[e0 + e] = (uint32_t)k;
         if (!kC && j < kFront) {
             // the link range follows by itself: no thread waits for it before
             // the phase ends
@@ -308,7 +310,7 @@ struct Part {
             dec[u] = 0;
             if (!die[u]) continue;
             if (ts[u] == 2u && kB[u] > 1u) {
-                ++upd;
+                upd += l[u].x != kAssigned;
                 if (!(l[u].x >> 31)) dec[u] = (int)(kB[u] - 1u);
             }
         }
@@ -401,6 +403,7 @@ struct Part {
             const bool act = w + 32u * u + lane < hi;
             const uint32_t x = pr[u].x - e0, y = pr[u].y - e0;
             const bool al = act && (pr[u].x >> 31 || remains(x)) && (pr[u].y >> 31 || remains(y));
+            if (al) upd -= (pr[u].x == kAssigned) + (pr[u].y == kAssigned);
             ed[2 * u] = x;
             ed[2 * u + 1] = y;
             dec[2 * u] = al && !(pr[u].x >> 31) ? (int)c[u] : 0;
@@ -428,7 +431,10 @@ struct Part {
         __syncthreads();  // the tables are free again
         if (tid < n) {
             *reinterpret_cast<uint2 *>(&a.bl[B].k) = make_uint2(r.z - r.w, 0u);
-            upd += 2ull * (r.z - r.w);
+            if (r.z != r.w) {
+                upd += 2ull * (r.z - r.w);
+                if (a.assigned) upd -= r.y <= 2u ? r.x : __ldcg(&a.bl[B].pair[0].x);
+            }
             slots += r.y;
         }
     }
@@ -653,7 +659,8 @@ inline unsigned grid_for(uint64_t items, int threads, unsigned cap) {
 
 }  // namespace
 
-cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, PeelResult &res, int num_sms, Alloc &al) {
+cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_from, PeelResult &res, int num_sms,
+                       Alloc &al) {
     const uint64_t m = g.m;
     res = PeelResult{};
     if (m == 0) return cudaSuccess;
@@ -681,17 +688,21 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, PeelResult &res, i
     }
     a.touch = al.get<uint32_t>(g.nb);
     a.phi = g.out_id ? al.get<uint32_t>(m) : phi_out;
-    a.depth = al.get<uint32_t>(m + 1);
+    const uint64_t deep = g.deep;  // levels are below it
+    a.depth = al.get<uint32_t>(deep + 1);
     Head *hd = al.get<Head>(1);
     if (al.err != cudaSuccess) return al.err;
     a.stats = hd->stats;
     a.err = &hd->err;
+    a.assign_from = assign_from;
+    a.assigned = g.assigned;
     a.queue = &hd->queue;
     const bt_limits *lim = al.limits;
-    a.round_limit = lim && lim->peel_round_limit && lim->peel_round_limit < m + 1 ? lim->peel_round_limit : m + 1;
+    a.round_limit = lim && lim->peel_round_limit && lim->peel_round_limit < deep + 1 ? lim->peel_round_limit : deep + 1;
     cudaStream_t st = al.stream;
     BT_CUDA(cudaMemsetAsync(hd, 0, sizeof(Head), st));
-    BT_CUDA(cudaMemsetAsync(a.depth, 0, sizeof(uint32_t) * (m + 1), st));
+    BT_CUDA(cudaMemsetAsync(a.depth, 0, sizeof(uint32_t) * (deep + 1), st));
+    if (g.out_id && assign_from > 0) BT_CUDA(cudaMemsetAsync(a.phi, 0xFF, sizeof(uint32_t) * m, st));
     if (g.n_heavy) {
         // the heavy parts, each by a cluster of blocks, beside the kernel of the
         // others, which fills the rest of the SMs
@@ -739,7 +750,7 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, PeelResult &res, i
         k_unplace<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(a.phi, g.out_id, m, phi_out);
         al.launches++;
     }
-    k_depth_sum<<<grid_for(m + 1, 256, (unsigned)num_sms * 8), 256, 0, st>>>(a.depth, m, hd->sums);
+    k_depth_sum<<<grid_for(deep + 1, 256, (unsigned)num_sms * 8), 256, 0, st>>>(a.depth, deep, hd->sums);
     al.launches++;
     BT_CUDA(cudaGetLastError());
     Head h{};

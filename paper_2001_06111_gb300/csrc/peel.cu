@@ -123,6 +123,7 @@ struct Ctl {
     unsigned long long kfinal;
     unsigned long long inc_phases;  // rounds that ran a separate incidence phase
     unsigned int n_parts;           // coarse peel: parts made
+    unsigned long long first_rounds, first_levels, first_updates;  // of its first part, with k_init
     unsigned int hist[2][kBins];    // coarse peel: supports of the alive edges, ping-pong
 };
 
@@ -483,6 +484,12 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     // coarse: parts begun, the weight the last one began with, all weight then
     uint32_t pno = 0, picked = 1, total_jump = 0;
     float aim = (float)a.target;
+    // with k_init > 0 part 0 is given; the parts whose tops are chosen here follow
+    bool in_first = kCoarse && a.k_init > 0;
+    const uint32_t first_free = in_first ? 1u : 0u;
+    pno = first_free;
+    uint32_t hno = 0;                  // level jumps
+    long long first_top = LLONG_MIN, lim = 0;  // the first part's window, what a jump takes
     if (threadIdx.x == 0) s_jn = 0;
     __syncthreads();
     // list sizes, kept identically by every thread from the barrier snapshots
@@ -502,110 +509,151 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
         }
         if constexpr (kCoarse) {
             if (level_jump) {
-                // C1: the alive edges again, with their supports' histogram and
-                // a copy of each support (the last copy an edge gets is its
-                // support when its part begins)
-                for (uint32_t i = threadIdx.x; i < kBins; i += kT) s_hist[i] = 0;
-                __syncthreads();
-                if (gtid == 0) atomicAdd(&ctl->scanned, 2ull * v_alive);
-                // the list is written anew only once a quarter of it is gone:
-                // its places come from one counter, which is what that costs
-                const bool anew = remaining < v_alive - v_alive / 4u;
-                constexpr uint32_t U = 4;  // entries a lane has in flight
-                for (uint32_t i0 = gwarp * 32u * U; i0 < v_alive; i0 += nthreads * U) {
-                    uint32_t e[U], stv[U];
-                    long long sv[U];
-                    bool keep[U];
-#pragma unroll
-                    for (uint32_t r = 0; r < U; ++r) {
-                        const uint32_t i = i0 + 32u * r + lane;
-                        keep[r] = i < v_alive;
-                        e[r] = keep[r] ? ldcg_u32(&a.alive[ap][i]) : 0u;
+                // The first part of a given top k_init: the batches are those of the
+                // fine peel, whose level jumps take what its window lists.  While
+                // the least support is within it, a jump is one reading for the
+                // minimum and one for the batch.
+                bool within = false;
+                if (in_first) {
+                    unsigned long long least = ~0ull;
+                    for (uint32_t i = gtid; i < v_alive; i += nthreads) {
+                        const uint32_t e = ldcg_u32(&a.alive[ap][i]);
+                        const uint32_t stv = ldcg_u32(&a.state[e]);
+                        const unsigned long long sv = (unsigned long long)ldcg_ll(&a.sup[e]);
+                        if (stv == kAlive && sv < least) least = sv;
                     }
+                    if (gtid == 0) atomicAdd(&ctl->scanned, (unsigned long long)v_alive);
 #pragma unroll
-                    for (uint32_t r = 0; r < U; ++r) {
-                        stv[r] = keep[r] ? ldcg_u32(&a.state[e[r]]) : 0u;
-                        sv[r] = keep[r] ? ldcg_ll(&a.sup[e[r]]) : 0ll;
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const unsigned long long y = __shfl_xor_sync(kFull, least, o);
+                        least = y < least ? y : least;
                     }
-                    uint32_t n = 0, at[U];
-#pragma unroll
-                    for (uint32_t r = 0; r < U; ++r) {
-                        keep[r] = keep[r] && stv[r] == kAlive;
-                        if (keep[r]) {
-                            a.snap[e[r]] = (int)sv[r];
-                            const uint64_t d = a.inc_off[e[r] + 1] - a.inc_off[e[r]];
-                            atomicAdd(&s_hist[bin_of((unsigned long long)sv[r])], 1u + (uint32_t)(d >> a.wshift));
-                        }
-                        const unsigned int mask = __ballot_sync(kFull, keep[r]);
-                        at[r] = n + __popc(mask & ((1u << lane) - 1u));
-                        n += __popc(mask);
-                    }
-                    if (anew && n) {
-                        uint32_t base = 0;
-                        if (lane == 0) base = atomicAdd(&ctl->n_alive[ap ^ 1u], n);
-                        base = __shfl_sync(kFull, base, 0);
-#pragma unroll
-                        for (uint32_t r = 0; r < U; ++r)
-                            if (keep[r]) a.alive[ap ^ 1u][base + at[r]] = e[r];
-                    }
-                }
-                __syncthreads();
-                for (uint32_t i = threadIdx.x; i < kBins; i += kT)
-                    if (s_hist[i]) atomicAdd(&ctl->hist[pno & 1u][i], s_hist[i]);
-                {
-                    const Snap sn{{nullptr, nullptr, nullptr, nullptr, nullptr}, nullptr};
+                    if (lane == 0 && least != ~0ull) atomicMin(&ctl->minsup, least);
+                    const Snap sn{{nullptr, nullptr, nullptr, nullptr, nullptr}, &ctl->minsup};
                     if (!grid_barrier(a, bar_no, sn, &s_v)) break;
+                    const long long mn = (long long)s_v.w;
+                    within = mn <= a.k_init;
+                    if (within) {
+                        if (mn >= first_top) first_top = window_top(mn);
+                        L.k = a.k_init;
+                        lim = first_top <= a.k_init ? first_top - 1 : L.k;
+                        L.label = 0;
+                        if (gtid == 0) ++ctl->first_levels;
+                    } else {
+                        in_first = false;
+                        upd = dev::warp_sum(upd);
+                        if (lane == 0 && upd) atomicAdd(&ctl->first_updates, upd);
+                        upd = 0;
+                        if (gtid == 0) ctl->first_rounds = round;
+                    }
                 }
-                if (anew) {
-                    v_alive = (uint32_t)remaining;
-                    ap ^= 1u;
-                    if (gtid == 0) ctl->n_alive[ap ^ 1u] = 0;
-                }
-                L.label = pno;
-                // every block finds the class up to which the edges of the next
-                // part reach
-                {
-                    constexpr uint32_t kPer = (kBins + kT - 1) / kT;
-                    uint32_t mine[kPer], sum = 0;
+                constexpr uint32_t U = 4;  // entries a lane has in flight
+                if (!within) {
+                    // C1: the alive edges again, with their supports' histogram and
+                    // a copy of each support (the last copy an edge gets is its
+                    // support when its part begins)
+                    for (uint32_t i = threadIdx.x; i < kBins; i += kT) s_hist[i] = 0;
+                    __syncthreads();
+                    if (gtid == 0) atomicAdd(&ctl->scanned, 2ull * v_alive);
+                    // the list is written anew only once a quarter of it is gone:
+                    // its places come from one counter, which is what that costs
+                    const bool anew = remaining < v_alive - v_alive / 4u;
+                    for (uint32_t i0 = gwarp * 32u * U; i0 < v_alive; i0 += nthreads * U) {
+                        uint32_t e[U], stv[U];
+                        long long sv[U];
+                        bool keep[U];
 #pragma unroll
-                    for (uint32_t r = 0; r < kPer; ++r) {
-                        const uint32_t b = threadIdx.x * kPer + r;
-                        mine[r] = b < kBins ? __ldcg(&ctl->hist[pno & 1u][b]) : 0u;
-                        sum += mine[r];
-                    }
-                    uint32_t total;
-                    uint32_t cum = dev::block_excl_scan<uint32_t>(sum, &total);
-                    if (pno + 1u >= a.max_parts || total <= a.target + a.target / 2u) {
-                        // the rest is the last part: nothing is left to be told apart
-                        for (uint32_t i = gtid; i < v_alive; i += nthreads) {
-                            const uint32_t e = ldcg_u32(&a.alive[ap][i]);
-                            if (ldcg_u32(&a.state[e]) == kAlive) a.phi[e] = pno;
+                        for (uint32_t r = 0; r < U; ++r) {
+                            const uint32_t i = i0 + 32u * r + lane;
+                            keep[r] = i < v_alive;
+                            e[r] = keep[r] ? ldcg_u32(&a.alive[ap][i]) : 0u;
                         }
-                        ++pno;
-                        break;
-                    }
-                    // the peel takes more edges than the class holds: the target
-                    // is scaled by what the last part grew by
-                    if (pno > 0) {
-                        const float grew = (float)(total_jump - total) / (float)picked;
-                        aim = fminf(fmaxf((float)a.target / grew, (float)a.target / 32.f), (float)a.target);
-                    }
-                    const uint32_t want = aim < 1.f ? 1u : (uint32_t)aim;
 #pragma unroll
-                    for (uint32_t r = 0; r < kPer; ++r) {
-                        // the first class with a weight of at least `want` up to it
-                        if (cum < want && cum + mine[r] >= want) {
-                            s_bin = threadIdx.x * kPer + r;
-                            s_cum = cum + mine[r];
+                        for (uint32_t r = 0; r < U; ++r) {
+                            stv[r] = keep[r] ? ldcg_u32(&a.state[e[r]]) : 0u;
+                            sv[r] = keep[r] ? ldcg_ll(&a.sup[e[r]]) : 0ll;
                         }
-                        cum += mine[r];
+                        uint32_t n = 0, at[U];
+#pragma unroll
+                        for (uint32_t r = 0; r < U; ++r) {
+                            keep[r] = keep[r] && stv[r] == kAlive;
+                            if (keep[r]) {
+                                a.snap[e[r]] = (int)sv[r];
+                                const uint64_t d = a.inc_off[e[r] + 1] - a.inc_off[e[r]];
+                                atomicAdd(&s_hist[bin_of((unsigned long long)sv[r])], 1u + (uint32_t)(d >> a.wshift));
+                            }
+                            const unsigned int mask = __ballot_sync(kFull, keep[r]);
+                            at[r] = n + __popc(mask & ((1u << lane) - 1u));
+                            n += __popc(mask);
+                        }
+                        if (anew && n) {
+                            uint32_t base = 0;
+                            if (lane == 0) base = atomicAdd(&ctl->n_alive[ap ^ 1u], n);
+                            base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+                            for (uint32_t r = 0; r < U; ++r)
+                                if (keep[r]) a.alive[ap ^ 1u][base + at[r]] = e[r];
+                        }
                     }
                     __syncthreads();
-                    L.k = bin_top(s_bin);
-                    picked = s_cum;
-                    total_jump = total;
-                    for (uint32_t i = gtid; i < kBins; i += nthreads) ctl->hist[(pno & 1u) ^ 1u][i] = 0;
-                    ++pno;
+                    for (uint32_t i = threadIdx.x; i < kBins; i += kT)
+                        if (s_hist[i]) atomicAdd(&ctl->hist[hno & 1u][i], s_hist[i]);
+                    {
+                        const Snap sn{{nullptr, nullptr, nullptr, nullptr, nullptr}, nullptr};
+                        if (!grid_barrier(a, bar_no, sn, &s_v)) break;
+                    }
+                    if (anew) {
+                        v_alive = (uint32_t)remaining;
+                        ap ^= 1u;
+                        if (gtid == 0) ctl->n_alive[ap ^ 1u] = 0;
+                    }
+                    L.label = pno;
+                    // every block finds the class up to which the edges of the next
+                    // part reach
+                    {
+                        constexpr uint32_t kPer = (kBins + kT - 1) / kT;
+                        uint32_t mine[kPer], sum = 0;
+#pragma unroll
+                        for (uint32_t r = 0; r < kPer; ++r) {
+                            const uint32_t b = threadIdx.x * kPer + r;
+                            mine[r] = b < kBins ? __ldcg(&ctl->hist[hno & 1u][b]) : 0u;
+                            sum += mine[r];
+                        }
+                        uint32_t total;
+                        uint32_t cum = dev::block_excl_scan<uint32_t>(sum, &total);
+                        if (pno + 1u >= a.max_parts || total <= a.target + a.target / 2u) {
+                            // the rest is the last part: nothing is left to be told apart
+                            for (uint32_t i = gtid; i < v_alive; i += nthreads) {
+                                const uint32_t e = ldcg_u32(&a.alive[ap][i]);
+                                if (ldcg_u32(&a.state[e]) == kAlive) a.phi[e] = pno;
+                            }
+                            ++pno;
+                            break;
+                        }
+                        // the peel takes more edges than the class holds: the target
+                        // is scaled by what the last part grew by
+                        if (pno > first_free) {
+                            const float grew = (float)(total_jump - total) / (float)picked;
+                            aim = fminf(fmaxf((float)a.target / grew, (float)a.target / 32.f), (float)a.target);
+                        }
+                        const uint32_t want = aim < 1.f ? 1u : (uint32_t)aim;
+#pragma unroll
+                        for (uint32_t r = 0; r < kPer; ++r) {
+                            // the first class with a weight of at least `want` up to it
+                            if (cum < want && cum + mine[r] >= want) {
+                                s_bin = threadIdx.x * kPer + r;
+                                s_cum = cum + mine[r];
+                            }
+                            cum += mine[r];
+                        }
+                        __syncthreads();
+                        L.k = lim = bin_top(s_bin);
+                        picked = s_cum;
+                        total_jump = total;
+                        for (uint32_t i = gtid; i < kBins; i += nthreads) ctl->hist[(hno & 1u) ^ 1u][i] = 0;
+                        ++hno;
+                        ++pno;
+                    }
                 }
                 // C2: their links become incidence items of this round
                 uint32_t sel = 0;
@@ -627,7 +675,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                     }
 #pragma unroll
                     for (uint32_t r = 0; r < U; ++r) {
-                        in[r] = in[r] && stv[r] == kAlive && sv[r] <= L.k;
+                        in[r] = in[r] && stv[r] == kAlive && sv[r] <= lim;
                         ib[r] = in[r] ? a.inc_off[e[r]] : 0ull;
                         ie[r] = in[r] ? a.inc_off[e[r] + 1] : 0ull;
                     }
@@ -668,6 +716,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                 n_items = s_v.u[1];
                 nb_cur = s_v.u[2];
                 nb_prev = s_v.u[3];
+                if (gtid == 0) ctl->minsup = ~0ull;
             }
         } else if (level_jump) {
             if (gtid == 0) atomicAdd(&ctl->scanned, (unsigned long long)v_near);
@@ -1028,9 +1077,10 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
         level_jump = remaining > 0 && n_batch == 0;
     }
     upd = dev::warp_sum(upd);
-    if (lane == 0 && upd) atomicAdd(&ctl->updates, upd);
+    if (lane == 0 && upd) atomicAdd(in_first ? &ctl->first_updates : &ctl->updates, upd);
     slots = dev::warp_sum(slots);
     if (lane == 0 && slots) atomicAdd(&ctl->slots, slots);
+    if (gtid == 0 && in_first) ctl->first_rounds = round;
     if (gtid == 0) {
         ctl->rounds = round;
         ctl->kfinal = (unsigned long long)L.k;
@@ -1165,6 +1215,9 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     res.kmax = h.kfinal;
     res.inc_phases = h.inc_phases;
     res.parts = h.n_parts;
+    res.first_rounds = h.first_rounds;
+    res.first_levels = h.first_levels;
+    res.first_updates = h.first_updates;
     al.put(a.sup);
     al.put(a.state);
     al.put(a.died);

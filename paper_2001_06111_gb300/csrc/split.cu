@@ -62,20 +62,22 @@ __global__ void k_edge_rec(const uint64_t *inc_off, const uint64_t *support, uin
     }
 }
 
-__global__ void k_iota2(const uint32_t *part, uint64_t m, uint32_t *keys, uint32_t *vals) {
+// Sort keys: the part of an edge, np for an assigned one.
+__global__ void k_iota2(const uint32_t *part, const uint8_t *assigned, uint32_t np, uint64_t m, uint32_t *keys,
+                        uint32_t *vals) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
-        keys[i] = part[i];
+        keys[i] = assigned && assigned[i] ? np : part[i];
         vals[i] = (uint32_t)i;
     }
 }
 
-// keys: parts in ascending order (np of them), order: the edges.  place[e] = (new id, part);
-// part_e[q]: the first edge of part q.
+// keys: parts in ascending order (np of them; np: assigned), order: the edges.
+// place[e] = (new id, part); part_e[q]: the first edge of part q.
 __global__ void k_place(const uint32_t *keys, const uint32_t *order, uint64_t m, uint32_t np, uint2 *place,
                         uint32_t *part_e) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t q = keys[i];
-        place[order[i]] = make_uint2((uint32_t)i, q);
+        place[order[i]] = make_uint2(q < np ? (uint32_t)i : kAssigned, q);
         const uint32_t before = i ? keys[i - 1] + 1u : 0u;  // a part may be empty
         for (uint32_t x = before; x <= q; ++x) part_e[x] = (uint32_t)i;
         if (i + 1 == m)
@@ -94,6 +96,7 @@ struct SplitArgs {
     BloomRec *bl;         // group records, part by part
     uint32_t *groups;     // [np] groups of each part: counted, then (the exclusive sums) handed out
     uint32_t *members;    // [np] their pairs (of groups of more than two), likewise
+    bool assigned;        // some edges are assigned (part np): flagged in the index's pairs
 };
 
 __device__ __forceinline__ uint2 placed(uint2 a, uint2 b) {
@@ -144,8 +147,8 @@ __global__ void __launch_bounds__(kT) k_split_small(const SplitArgs a) {
 #pragma unroll
         for (int i = 0; i < kSmall; ++i) {
             const uint2 pr = px[i];
-            py[i] = (uint32_t)i < K ? a.place[pr.y] : make_uint2(0u, 0u);
-            px[i] = (uint32_t)i < K ? a.place[pr.x] : make_uint2(0u, 0u);
+            py[i] = (uint32_t)i < K ? a.place[pr.y & ~kFlag] : make_uint2(0u, 0u);
+            px[i] = (uint32_t)i < K ? a.place[pr.x & ~kFlag] : make_uint2(0u, 0u);
         }
 #pragma unroll
         for (int i = 0; i < kSmall; ++i) q[i] = (uint32_t)i < K ? (px[i].y < py[i].y ? px[i].y : py[i].y) : kNone;
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(kT) k_split_small(const SplitArgs a) {
                 size[i] += q[j] == q[i];
                 if (q[j] == q[i]) first[i] = j;
             }
-            if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u) {
+            if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u && q[i] < a.np) {
                 atomicAdd(&s.groups[q[i]], 1u);
                 if (size[i] > 2u) atomicAdd(&s.members[q[i]], size[i]);
             }
@@ -177,10 +180,16 @@ __global__ void __launch_bounds__(kT) k_split_small(const SplitArgs a) {
             for (int i = 0; i < kSmall; ++i) {
                 id[i] = kNone;
                 at[i] = 0;
-                if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u) {
+                if ((uint32_t)i < K && first[i] == (uint32_t)i && left[i] >= 2u && q[i] < a.np) {
                     id[i] = atomicAdd(&s.groups[q[i]], 1u);
                     if (size[i] > 2u) at[i] = atomicAdd(&s.members[q[i]], size[i]);
-                    head(a.bl + id[i], at[i], size[i], left[i]);
+                    uint32_t known = 0;  // assigned edges among the pairs of higher parts
+                    if (a.assigned)
+#pragma unroll
+                        for (int j = 0; j < kSmall; ++j)
+                            if ((uint32_t)j < K && q[j] > q[i]) known += (px[j].y == a.np) + (py[j].y == a.np);
+                    head(a.bl + id[i], size[i] > 2u ? at[i] : known, size[i], left[i]);
+                    if (size[i] > 2u) a.bl[id[i]].pair[0].x = known;
                 }
 #pragma unroll
                 for (int j = 0; j < i; ++j)
@@ -211,12 +220,13 @@ __global__ void __launch_bounds__(kT) k_split_small(const SplitArgs a) {
 template <bool kPlace>
 __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
     constexpr int kWarps = kT / 32;
-    extern __shared__ uint32_t s_tab[];  // two rows of np a warp; then the block's tally
+    extern __shared__ uint32_t s_tab[];  // three rows a warp; then the block's tally
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t *cur = s_tab + (size_t)w * 2 * a.np, *gid = cur + a.np;
-    uint32_t *t_groups = s_tab + (size_t)kWarps * 2 * a.np, *t_members = t_groups + a.np;
+    const uint32_t row = a.np + 1u;
+    uint32_t *cur = s_tab + (size_t)w * 3 * row, *gid = cur + row, *known = gid + row;
+    uint32_t *t_groups = s_tab + (size_t)kWarps * 3 * row, *t_members = t_groups + row;
     if constexpr (!kPlace) {
-        for (uint32_t i = threadIdx.x; i < 2 * a.np; i += kT) t_groups[i] = 0;
+        for (uint32_t i = threadIdx.x; i < 2 * row; i += kT) t_groups[i] = 0;
         __syncthreads();
     }
     const uint64_t nw = (uint64_t)gridDim.x * kWarps;
@@ -231,23 +241,35 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
             const int src = __ffs(big) - 1;
             big &= big - 1u;
             const uint32_t off = __shfl_sync(kFull, my_off, src), K = __shfl_sync(kFull, my_k, src);
-            for (uint32_t i = lane; i < a.np; i += 32) cur[i] = 0;
+            for (uint32_t i = lane; i < row; i += 32) cur[i] = known[i] = 0;
             __syncwarp();
+            uint32_t all_known = 0;  // assigned edges of the bloom
             for (uint32_t i = lane; i < K; i += 32) {
                 const uint2 pr = a.pairs[off + i];
-                const uint32_t qx = a.place[pr.x].y, qy = a.place[pr.y].y;
-                atomicAdd(&cur[qx < qy ? qx : qy], 1u);
+                const uint32_t qx = a.place[pr.x & ~kFlag].y, qy = a.place[pr.y & ~kFlag].y;
+                const uint32_t qi = qx < qy ? qx : qy, kn = (qx == a.np) + (qy == a.np);
+                atomicAdd(&cur[qi], 1u);
+                if (kn) atomicAdd(&known[qi], kn);
+                all_known += kn;
             }
+            all_known = dev::warp_sum(all_known);
             __syncwarp();
             // parts in order, 32 at a time: pairs below; a group for each
             // non-empty part that leaves a butterfly
-            uint32_t run = 0;
+            uint32_t run = 0, run_known = 0;
+            if (lane == 0) gid[a.np] = kNone;
             for (uint32_t i0 = 0; i0 < a.np; i0 += 32) {
                 const uint32_t i = i0 + lane;
                 const uint32_t n = i < a.np ? cur[i] : 0u;
                 const uint32_t incl = dev::warp_incl_scan(n);
                 const uint32_t left = K - (run + incl - n);
                 run += __shfl_sync(kFull, incl, 31);
+                uint32_t higher = 0;  // assigned edges among the pairs of higher parts
+                if (a.assigned) {
+                    const uint32_t ki = dev::warp_incl_scan(i < a.np ? known[i] : 0u);
+                    higher = all_known - run_known - ki;
+                    run_known += __shfl_sync(kFull, ki, 31);
+                }
                 if (i >= a.np) continue;
                 const bool g = n > 0u && left >= 2u;
                 if constexpr (kPlace) {
@@ -257,7 +279,8 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
                         const uint32_t at = n > 2u ? atomicAdd(&a.members[i], n) : 0u;
                         gid[i] = id;
                         cur[i] = n > 2u ? at : kFlag;  // up to two go to the record
-                        head(a.bl + id, at, n, left);
+                        head(a.bl + id, n > 2u ? at : higher, n, left);
+                        if (n > 2u) a.bl[id].pair[0].x = higher;
                     }
                 } else if (g) {
                     atomicAdd(&t_groups[i], 1u);
@@ -268,7 +291,7 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
             if constexpr (kPlace) {
                 for (uint32_t i = lane; i < K; i += 32) {
                     const uint2 pr = a.pairs[off + i];
-                    const uint2 x = a.place[pr.x], y = a.place[pr.y];
+                    const uint2 x = a.place[pr.x & ~kFlag], y = a.place[pr.y & ~kFlag];
                     const uint32_t qi = x.y < y.y ? x.y : y.y, id = gid[qi];
                     a.sub[off + i] = id;
                     if (id != kNone) {
@@ -298,50 +321,76 @@ __global__ void __launch_bounds__(kT) k_split_room(const uint64_t *inc_off, cons
     for (uint32_t i = threadIdx.x; i < np; i += kT) s_n[i] = 0;
     __syncthreads();
     for (uint64_t e = blockIdx.x * (uint64_t)kT + threadIdx.x; e < m; e += (uint64_t)gridDim.x * kT)
-        atomicAdd(&s_n[place[e].y], (unsigned long long)(inc_off[e + 1] - inc_off[e]));
+        if (place[e].y < np) atomicAdd(&s_n[place[e].y], (unsigned long long)(inc_off[e + 1] - inc_off[e]));
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < np; i += kT)
         if (s_n[i]) atomicAdd(&room[i], s_n[i]);
 }
 
+// One link of an edge in part `part`: whether it is kept (its pair belongs to the
+// edge's part and its group holds a butterfly), and as what.
+__device__ __forceinline__ bool part_link(uint2 l, uint2 pr, uint32_t s, const uint2 *place, uint32_t part, uint2 &out) {
+    const uint2 t = place[(l.y >> 31 ? pr.x : pr.y) & ~kFlag];
+    out = make_uint2(t.x | (t.y > part ? kFlag : 0u), s);
+    return s != kNone && t.y >= part;
+}
+
 // Links of every edge (a warp each): those whose pair belongs to the edge's part,
-// as (twin, group), into the part's own range (next: its next free place).  The
-// links are read twice, first to know their number.
+// as (twin, group), into the part's own range (next: its next free place).  Each
+// link costs three scattered reads, which bound this, so a lane has kLU links in
+// flight; an edge of more than 32 kLU links is read twice, first to know how many
+// it keeps (one link in flight and two readings for all but the smallest: 5.6 ms
+// on the 2M-edge graph).
+constexpr int kLU = 4;
 __global__ void __launch_bounds__(kT) k_split_links(const uint64_t *inc_off, const uint2 *inc, const uint2 *pairs,
                                                     const uint32_t *sub, const uint2 *place, const int *snap,
                                                     uint64_t m, unsigned long long *next, uint2 *out, uint4 *er) {
     const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
     const uint64_t nw = ((uint64_t)gridDim.x * kT) >> 5;
     for (uint64_t e = ((uint64_t)blockIdx.x * kT + threadIdx.x) >> 5; e < m; e += nw) {
         const uint64_t lb = inc_off[e], le = inc_off[e + 1];
         const uint2 me = place[e];
+        if (me.x == kAssigned) continue;
+        const bool once = le - lb <= 32u * kLU;
         uint32_t n = 0;
         unsigned long long at = 0;
-        for (int pass = 0; pass < 2; ++pass) {
+        for (int pass = once ? 1 : 0; pass < 2; ++pass) {
             uint32_t k = 0;
-            for (uint64_t j0 = lb; j0 < le; j0 += 32) {
-                const uint64_t j = j0 + lane;
-                uint2 nl = make_uint2(0u, 0u);
-                bool keep = false;
-                if (j < le) {
-                    const uint2 l = inc[j];
-                    const uint2 pr = pairs[l.x];
-                    const uint32_t s = sub[l.x];
-                    const uint2 t = place[l.y >> 31 ? pr.x : pr.y];
-                    keep = s != kNone && t.y >= me.y;
-                    nl = make_uint2(t.x | (t.y > me.y ? kFlag : 0u), s);
+            for (uint64_t j0 = lb; j0 < le; j0 += 32u * kLU) {
+                uint2 l[kLU], pr[kLU], nl[kLU];
+                uint32_t s[kLU], keep[kLU], cnt = 0;
+#pragma unroll
+                for (int r = 0; r < kLU; ++r) {
+                    const uint64_t j = j0 + 32u * r + lane;
+                    l[r] = j < le ? inc[j] : make_uint2(0u, 0u);
                 }
-                const unsigned mask = __ballot_sync(kFull, keep);
-                if (pass == 0 && le - lb <= 32) {  // all its links at once: no second reading
-                    n = __popc(mask);
+#pragma unroll
+                for (int r = 0; r < kLU; ++r) {
+                    const bool in = j0 + 32u * r + lane < le;
+                    s[r] = in ? sub[l[r].x] : kNone;
+                    pr[r] = in ? pairs[l[r].x] : make_uint2(0u, 0u);
+                }
+#pragma unroll
+                for (int r = 0; r < kLU; ++r) {
+                    const bool in = j0 + 32u * r + lane < le;
+                    keep[r] = __ballot_sync(kFull, in && part_link(l[r], pr[r], s[r], place, me.y, nl[r]));
+                    cnt += __popc(keep[r]);
+                }
+                if (once) {
+                    n = cnt;
                     if (lane == 0 && n) at = atomicAdd(&next[me.y], (unsigned long long)n);
                     at = __shfl_sync(kFull, at, 0);
-                    if (keep) out[at + __popc(mask & ((1u << lane) - 1u))] = nl;
-                    pass = 1;
-                } else if (pass == 1 && keep) {
-                    out[at + k + __popc(mask & ((1u << lane) - 1u))] = nl;
                 }
-                k += __popc(mask);
+                if (pass == 1) {
+                    uint32_t x = k;
+#pragma unroll
+                    for (int r = 0; r < kLU; ++r) {
+                        if (keep[r] >> lane & 1u) out[at + x + __popc(keep[r] & below)] = nl[r];
+                        x += __popc(keep[r]);
+                    }
+                }
+                k += cnt;
             }
             if (pass == 0) {
                 n = k;
@@ -361,7 +410,7 @@ void free_parts(PartGraph &g, Alloc &al) {
 }
 
 cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al) {
-    g.m = ix.m;
+    g.m = g.deep = ix.m;
     g.nb = ix.nb;
     g.np = 1;
     g.inc = ix.inc;
@@ -382,12 +431,13 @@ cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int
     return cudaGetLastError();
 }
 
-cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np, PartGraph &g,
-                            int num_sms, Alloc &al) {
+cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
+                            const uint8_t *assigned, bool skip_first, PartGraph &g, int num_sms, Alloc &al) {
     const uint64_t m = ix.m, nb = ix.nb;
     const unsigned wide = (unsigned)num_sms * 16;
-    g.m = m;
-    g.np = np;
+    g.deep = m;
+    g.assigned = assigned != nullptr;
+    g.np = np - skip_first;
     uint32_t *part_e = g.keep(al.get<uint32_t>((size_t)np + 1));
     uint32_t *part_b = g.keep(al.get<uint32_t>((size_t)np + 1));
     uint32_t *order = g.keep(al.get<uint32_t>(np));
@@ -404,9 +454,9 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     unsigned long long *room = al.get<unsigned long long>((size_t)np + 1);  // links; their places
     if (al.err != cudaSuccess) return al.err;
     // edges by part
-    k_iota2<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(part, m, keys, out_id);
+    k_iota2<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(part, assigned, np, m, keys, out_id);
     al.launches++;
-    BT_CUDA(radix_sort_u32(keys, out_id, tk, tv, m, bits_for(np - 1), al));
+    BT_CUDA(radix_sort_u32(keys, out_id, tk, tv, m, bits_for(assigned ? np : np - 1), al));
     k_place<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(keys, out_id, m, np, place, part_e);
     al.launches++;
     al.put(keys);
@@ -415,11 +465,12 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     // groups and pairs of each part, then their places
     BT_CUDA(cudaMemsetAsync(tally, 0, 8 * ((size_t)np + 1), al.stream));
     BT_CUDA(cudaMemsetAsync(room, 0, 8 * ((size_t)np + 1), al.stream));
-    SplitArgs s{ix.bloom_off, nb, ix.pairs, place, np, nullptr, nullptr, nullptr, tally, tally + np + 1};
-    const size_t smem = sizeof(uint32_t) * 2 * np * (kT / 32 + 1);
+    SplitArgs s{ix.bloom_off, nb, ix.pairs, place, np, nullptr, nullptr, nullptr, tally, tally + np + 1,
+                assigned != nullptr};
+    const size_t smem = sizeof(uint32_t) * (np + 1) * (3 * (kT / 32) + 2);
     // (the attribute belongs to the process: always the same value, so that
     // calls of several threads do not lower one another's)
-    const int most = (int)(sizeof(uint32_t) * 2 * kMaxParts * (kT / 32 + 1));
+    const int most = (int)(sizeof(uint32_t) * (kMaxParts + 1) * (3 * (kT / 32) + 2));
     BT_CUDA(cudaFuncSetAttribute(k_split_large<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     BT_CUDA(cudaFuncSetAttribute(k_split_large<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     if (nb) {
@@ -448,19 +499,21 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
         lsum += hr[i];
     }
     g.nb = gsum;
+    g.m = he[np];
     // the heaviest first; those that one block would be long at by a cluster
     const double lim = kHeavy * (double)lsum / np;
     auto heavy = [&](uint32_t p) { return he[p + 1] - he[p] > kBlockEdges || (double)hr[p] > lim; };
     for (uint32_t i = 0; i < np; ++i) ord[i] = i;
+    if (skip_first) ord.erase(ord.begin());
     std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) {
         const bool hx = heavy(x), hy = heavy(y);
         return hx != hy ? hx : hr[x] > hr[y];
     });
-    for (uint32_t i = 0; i < np; ++i) g.n_heavy += heavy(i);
+    for (const uint32_t p : ord) g.n_heavy += heavy(p);
     BT_CUDA(cudaMemcpyAsync(cursor, ht.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
     BT_CUDA(cudaMemcpyAsync(part_b, ht.data(), 4 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
     BT_CUDA(cudaMemcpyAsync(room, at.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
-    BT_CUDA(cudaMemcpyAsync(order, ord.data(), 4 * (size_t)np, cudaMemcpyHostToDevice, al.stream));
+    BT_CUDA(cudaMemcpyAsync(order, ord.data(), 4 * ord.size(), cudaMemcpyHostToDevice, al.stream));
     uint32_t *sub = al.get<uint32_t>(ix.w2);
     uint2 *pairs = g.keep(al.get<uint2>(psum)), *inc = g.keep(al.get<uint2>(lsum));
     g.bl = g.keep(al.get<BloomRec>(gsum));

@@ -82,3 +82,18 @@ def test_batches_same_as_the_grid_peel(h, n, hi):
     for (s0, p0), (s1, p1) in zip(ref, out):
         np.testing.assert_array_equal(s0, s1)
         np.testing.assert_array_equal(p0, p1)
+
+
+# passes of the progressive compression: assigned edges among the pairs, a first part
+# below the recorded levels (the default reading) or none (Alg. 7's)
+@pytest.mark.parametrize("flags", [0, bt.BT_PC_RECOUNT])
+@pytest.mark.parametrize("m,tau,nplant", [(1500, 0.5, 0), (12000, 0.1, 0), (40001, 0.3, 4), (90001, 1.0, 3)])
+def test_progressive_same_as_the_grid_peel(h, m, tau, nplant, flags):
+    g = synth.chunglu(m // 8, m // 14, m, 2.1, 2.4, seed=m, nplant=nplant, plant_lo=20, plant_hi=60, plant_p=0.9)
+    bt.bt_set_limits(h, join_cap=1 << 30)
+    ref = bt.bt_decompose_progressive(h, g.edges, g.nU, g.nL, tau=tau, flags=flags)
+    bt.bt_set_limits(h)
+    out = bt.bt_decompose_progressive(h, g.edges, g.nU, g.nL, tau=tau, flags=flags)
+    np.testing.assert_array_equal(out[0], ref[0])
+    np.testing.assert_array_equal(out[1], ref[1])
+    assert out[2] == ref[2]
