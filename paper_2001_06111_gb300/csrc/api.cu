@@ -188,12 +188,11 @@ cudaError_t deliver(bt_handle *h, void *dst, const void *src, size_t bytes, uint
 // internal edge id (P.g.newid maps input ids to them; with an index, the map
 // moves to ix.newid).
 int count_and_index(bt_handle *h, Prepared &P, uint64_t *d_support, bool want_index,
-                    bt::Index &ix, uint64_t &butterflies, bt::Alloc &al,
+                    bt::Index &ix, bt::Alloc &al,
                     const uint8_t *assigned = nullptr) {
     bt::CountOut co;
     co.support = d_support;
     co.assigned = assigned;
-    uint64_t W = 0;
     if (want_index) {
         co.inc_cnt = al.get<uint32_t>(P.g.m);
         co.w2v = al.get<uint64_t>(P.g.n);
@@ -202,25 +201,7 @@ int count_and_index(bt_handle *h, Prepared &P, uint64_t *d_support, bool want_in
     }
     cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al);
     if (e != cudaSuccess) return cuda_fail(h, e, "counting wedges");
-    unsigned long long bf = 0;
-    e = cudaMemcpyAsync(&bf, co.butterflies_dev, sizeof(bf), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    al.put(co.butterflies_dev);
-    if (e != cudaSuccess) return cuda_fail(h, e, "counting wedges");
-    bf /= 2;  // every butterfly gives each of its two wedges in a bloom one
-    butterflies = bf;
     if (want_index) {
-        // W for the statistics: sum of wedges per start vertex
-        uint64_t *tot = al.get<uint64_t>(1);
-        uint64_t *scratch = al.get<uint64_t>(P.g.n);
-        if (al.err != cudaSuccess) return cuda_fail(h, al.err, "allocating");
-        e = bt::exclusive_scan_u64(P.g.wv, scratch, P.g.n, tot, al);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&W, tot, sizeof(W), cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        al.put(tot);
-        al.put(scratch);
-        if (e != cudaSuccess) return cuda_fail(h, e, "summing wedges");
         e = bt::emit_index(P.g, co, ix, h->num_sms, al, h->stream);
         al.put(co.inc_cnt);
         al.put(co.w2v);
@@ -228,8 +209,6 @@ int count_and_index(bt_handle *h, Prepared &P, uint64_t *d_support, bool want_in
         if (e == cudaErrorInvalidValue)
             return fail(h, BT_ERR_OVERFLOW, "BE-Index has >= 2^32 twin pairs or blooms");
         if (e != cudaSuccess) return cuda_fail(h, e, "emitting the BE-Index");
-        ix.w = W;
-        ix.butterflies = bf;
         ix.newid = P.g.newid;  // the index speaks internal edge ids
         P.g.newid = nullptr;
     }
@@ -324,8 +303,7 @@ int bt_count_support(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU
         if (al.err != cudaSuccess) rc = cuda_fail(h, al.err, "allocating supports");
     }
     bt::Index unused;
-    uint64_t bf = 0;
-    if (rc == BT_OK) rc = count_and_index(h, P, d_int, false, unused, bf, al);
+    if (rc == BT_OK) rc = count_and_index(h, P, d_int, false, unused, al);
     if (rc == BT_OK) {
         cudaError_t e = bt::gather_u64(d_int, P.g.newid, d_sup, m, al);  // back to input order
         if (e == cudaSuccess) e = deliver(h, support_out, d_sup, sizeof(uint64_t) * m, flags);
@@ -388,7 +366,6 @@ int bt_count_support_part(bt_handle *h, const int32_t *edges, uint64_t m, uint32
         co.support = d_int;
         cudaError_t e = bt::count_wedges(P.g, co, h->num_sms, al, hb[0], hb[1]);
         if (e == cudaSuccess) {
-            al.put(co.butterflies_dev);
             e = bt::gather_u64(d_int, P.g.newid, d_sup, m, al);  // back to input order
         }
         if (e == cudaSuccess) e = deliver(h, support_out, d_sup, sizeof(uint64_t) * m, flags);
@@ -523,8 +500,7 @@ static int build_index_impl(bt_handle *h, const int32_t *edges, uint64_t m, uint
     }
     bt::Index ix;
     ix.twin_links = one_part;
-    uint64_t bf = 0;
-    if (rc == BT_OK) rc = count_and_index(h, P, d_sup, true, ix, bf, al);
+    if (rc == BT_OK) rc = count_and_index(h, P, d_sup, true, ix, al);
     release(P, al);
     if (rc == BT_OK) {
         h->index = ix;
@@ -1150,10 +1126,9 @@ int bt_decompose_progressive(bt_handle *h, const int32_t *edges, uint64_t m, uin
         cass2 = al.get<uint8_t>(m);
     }
     if (rc == BT_OK && al.err != cudaSuccess) rc = cuda_fail(h, al.err, "allocating");
-    uint64_t bf = 0;
     bt::Index unused;
     // supports of G (the counting process of Alg. 7)
-    if (rc == BT_OK) rc = count_and_index(h, P, sup_c, false, unused, bf, al);
+    if (rc == BT_OK) rc = count_and_index(h, P, sup_c, false, unused, al);
     if (rc == BT_OK) {
         cudaError_t eg = bt::gather_u64(sup_c, P.g.newid, d_sup0, m, al);  // input order
         if (eg != cudaSuccess) rc = cuda_fail(h, eg, "counting");
@@ -1203,7 +1178,7 @@ int bt_decompose_progressive(bt_handle *h, const int32_t *edges, uint64_t m, uin
             // phi-bitruss lies inside G_{>=eps}, so it keeps >= phi butterflies)
             Prepared R;
             rc = prepare(h, cand, hc[0], nU, nL, (flags & BT_TIE_LOWER_FIRST) | BT_DEVICE_PTRS, R, al);
-            if (rc == BT_OK) rc = count_and_index(h, R, sup_c, false, unused, bf, al);
+            if (rc == BT_OK) rc = count_and_index(h, R, sup_c, false, unused, al);
             if (rc == BT_OK) {
                 unsigned long long h2[2] = {0, 0};
                 e = bt::gather_u64(sup_c, R.g.newid, sup_r, hc[0], al);  // candidate order
@@ -1235,7 +1210,7 @@ int bt_decompose_progressive(bt_handle *h, const int32_t *edges, uint64_t m, uin
                 cudaError_t es = bt::scatter_u8(pc_ass, Q.g.newid, cass_int, pc_n, al);
                 if (es != cudaSuccess) rc = cuda_fail(h, es, "extracting a candidate subgraph");
             }
-            if (rc == BT_OK) rc = count_and_index(h, Q, sup_c, true, ix, bf, al, cass_int);
+            if (rc == BT_OK) rc = count_and_index(h, Q, sup_c, true, ix, al, cass_int);
             bt::free_csr(Q.g, al);
             bt::PeelResult pr;
             if (rc == BT_OK) {

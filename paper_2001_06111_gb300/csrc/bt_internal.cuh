@@ -162,6 +162,9 @@ struct Csr {
     // start vertices that the counting kernel gives a block each (the others get a
     // warp): n_heavy[64] ranks, by the power of two of their wedges, most first
     uint32_t *heavy = nullptr, *n_heavy = nullptr;
+    // what the host reads once, before the index is allocated: wedges, twice the
+    // butterflies (count_wedges), blooms, bloom wedges, links (emit_index)
+    uint64_t *totals = nullptr;  // [5]
     // Internal edge ids: an edge is numbered by its position in the lower-rank
     // prefix of its higher-ranked endpoint, so the edges of one vertex are
     // contiguous (blooms anchored there touch neighbouring words).  eid holds
@@ -213,7 +216,6 @@ struct CountOut {
     uint32_t *inc_cnt = nullptr;  // [m] links per edge (index mode) or nullptr
     uint64_t *w2v = nullptr;      // [n] bloom wedges per start vertex (index mode)
     uint64_t *nbv = nullptr;      // [n] blooms per start vertex (index mode)
-    unsigned long long *butterflies_dev = nullptr;  // [1] twice the butterflies, set by count_wedges; caller frees
     // [m] or nullptr: edges whose bitruss number is already known (progressive
     // compression); they get no links and are flagged in bit 31 inside pairs
     const uint8_t *assigned = nullptr;

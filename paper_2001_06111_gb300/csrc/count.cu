@@ -742,7 +742,7 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     a.cold_n = g.cnt_n > width ? g.cnt_n - width : 0u;
     a.cold = al.get<uint32_t>((size_t)blocks * a.cold_n);
     a.queue = al.get<uint32_t>(1);
-    a.totals = al.get<unsigned long long>(1);
+    a.totals = reinterpret_cast<unsigned long long *>(g.totals + 1);
     if (al.err != cudaSuccess) return al.err;
     a.support = reinterpret_cast<unsigned long long *>(o.support);
     a.inc_cnt = o.inc_cnt;
@@ -751,7 +751,6 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     a.assigned = index ? o.assigned : nullptr;
     if (a.cold_n) BT_CUDA(cudaMemsetAsync(a.cold, 0, sizeof(uint32_t) * (size_t)blocks * a.cold_n, al.stream));
     BT_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), al.stream));
-    BT_CUDA(cudaMemsetAsync(a.totals, 0, sizeof(unsigned long long), al.stream));
     BT_CUDA(cudaMemsetAsync(o.support, 0, sizeof(uint64_t) * g.m, al.stream));
     if (index) BT_CUDA(cudaMemsetAsync(o.inc_cnt, 0, sizeof(uint32_t) * g.m, al.stream));
     const size_t smem = sizeof(CountShared) + kHot * sizeof(uint16_t);
@@ -770,7 +769,6 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     al.launches += 2;
     al.mark(kPhCount, true);
     BT_CUDA(cudaGetLastError());
-    o.butterflies_dev = a.totals;
     al.put(a.cold);
     al.put(a.queue);
     return cudaSuccess;
@@ -783,7 +781,7 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     // layout prefix sums
     uint64_t *bloom_base = al.get<uint64_t>(n);
     uint64_t *pair_base = al.get<uint64_t>(n);
-    uint64_t *tot = al.get<uint64_t>(3);
+    uint64_t *tot = g.totals + 2;
     uint64_t *incc64 = al.get<uint64_t>(m + 1);
     ix.inc_off = al.get<uint64_t>(m + 1);
     if (al.err != cudaSuccess) return al.err;
@@ -792,17 +790,18 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     BT_CUDA(widen_u32(c.inc_cnt, incc64, m, al));
     BT_CUDA(cudaMemsetAsync(incc64 + m, 0, sizeof(uint64_t), al.stream));
     BT_CUDA(exclusive_scan_u64(incc64, ix.inc_off, m + 1, tot + 2, al));
-    uint64_t h_tot[3];
-    BT_CUDA(cudaMemcpyAsync(h_tot, tot, sizeof(h_tot), cudaMemcpyDeviceToHost, stream));
+    uint64_t h_tot[5];
+    BT_CUDA(cudaMemcpyAsync(h_tot, g.totals, sizeof(h_tot), cudaMemcpyDeviceToHost, stream));
     BT_CUDA(cudaStreamSynchronize(stream));
-    ix.nb = h_tot[0];
-    ix.w2 = h_tot[1];
-    ix.links = h_tot[2];  // 2 w2, less the links of assigned edges in a compressed index
+    ix.w = h_tot[0];
+    ix.butterflies = h_tot[1] / 2;  // every butterfly gives each of its two wedges in a bloom one
+    ix.nb = h_tot[2];
+    ix.w2 = h_tot[3];
+    ix.links = h_tot[4];  // 2 w2, less the links of assigned edges in a compressed index
     // pair ids are u32; bloom ids keep bit 31 free for the link's side
     if (ix.w2 >= 0xFFFFFFFFull || ix.nb >= 0x80000000ull) {
         al.put(bloom_base);
         al.put(pair_base);
-        al.put(tot);
         al.put(incc64);
         return cudaErrorInvalidValue;  // reported as overflow by the caller
     }
@@ -865,7 +864,6 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     al.put(incc64);
     al.put(bloom_base);
     al.put(pair_base);
-    al.put(tot);
     return cudaSuccess;
 }
 

@@ -1,6 +1,7 @@
 // Degree, priority rank and rank-ordered CSR (the preprocessing of Alg. 3:
 // "compute p(u) for each u", Def. 7), plus the per-arc wedge prefix lengths
 // that bound the priority-obeyed wedge loops (Def. 10, Lemma 6).
+#include "bt_device.cuh"
 #include "bt_internal.cuh"
 
 namespace bt {
@@ -175,17 +176,21 @@ __global__ void k_relabel(const uint32_t *row_of, const uint32_t *adj, uint64_t 
 
 // Start vertices that get a block each, by the power of two of their wedges: the
 // counting kernels take the heaviest first, so that none is begun when the other
-// blocks are done.  tab[0 .. 64): how many of each class, [64]: all, [65 .. 129): placed.
+// blocks are done.  tab[0 .. 64): how many of each class, [64]: of all, [65 .. 129):
+// placed.  all: the sum of the wedges (a scan and a copy of its own before).
 __device__ __forceinline__ uint32_t wedge_class(uint64_t W) { return (uint32_t)__clzll((long long)W); }
-__global__ void k_heavy_count(const uint64_t *wv, const uint32_t *hv, uint32_t n, uint32_t *tab) {
+__global__ void k_heavy_count(const uint64_t *wv, const uint32_t *hv, uint32_t n, uint32_t *tab, uint64_t *all) {
     __shared__ uint32_t s_n[64];
     if (threadIdx.x < 64) s_n[threadIdx.x] = 0;
     __syncthreads();
+    unsigned long long sum = 0;
     for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
         const uint64_t W = wv[u];
+        sum += W;
         if (W && !is_light(W, hv[u])) atomicAdd(&s_n[wedge_class(W)], 1u);
     }
-    __syncthreads();
+    sum = dev::block_sum(sum);
+    if (threadIdx.x == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long *>(all), sum);
     if (threadIdx.x < 64 && s_n[threadIdx.x]) {
         atomicAdd(&tab[threadIdx.x], s_n[threadIdx.x]);
         atomicAdd(&tab[64], s_n[threadIdx.x]);
@@ -337,11 +342,13 @@ cudaError_t build_csr(const int32_t *d_edges, uint64_t m, uint32_t nU, uint32_t 
     g.wv = al.get<uint64_t>(n);
     g.heavy = al.get<uint32_t>(n);
     g.n_heavy = al.get<uint32_t>(129);
+    g.totals = al.get<uint64_t>(5);
     g.newid = al.get<uint32_t>(m);
     uint32_t *low = al.get<uint32_t>(m), *hoff = al.get<uint32_t>(n), *row_of = al.get<uint32_t>(na);
     if (al.err != cudaSuccess) return al.err;
     BT_CUDA(cudaMemsetAsync(g.hv, 0, sizeof(uint32_t) * n, al.stream));
     BT_CUDA(cudaMemsetAsync(g.wv, 0, sizeof(uint64_t) * n, al.stream));
+    BT_CUDA(cudaMemsetAsync(g.totals, 0, sizeof(uint64_t) * 5, al.stream));
     BT_CUDA(cudaMemsetAsync(g.n_heavy, 0, sizeof(uint32_t) * 129, al.stream));
     k_csr_fill<<<grid_for(na, 256), 256, 0, al.stream>>>(keys, vals, na, n, g.off, row_of, g.adj, g.eid, low, g.hv,
                                                          err_word);
@@ -353,7 +360,7 @@ cudaError_t build_csr(const int32_t *d_edges, uint64_t m, uint32_t nU, uint32_t 
     k_wedge_prefix<<<grid_for(na, 256), 256, 0, al.stream>>>(g.off, row_of, g.adj, g.eid, low, hoff, na, g.pl,
                                                              reinterpret_cast<unsigned long long *>(g.wv), g.newid);
     k_relabel<<<grid_for(na, 256), 256, 0, al.stream>>>(row_of, g.adj, na, g.eid, g.newid);
-    k_heavy_count<<<grid_for(n, 256, 152 * 4), 256, 0, al.stream>>>(g.wv, g.hv, n, g.n_heavy);
+    k_heavy_count<<<grid_for(n, 256, 152 * 4), 256, 0, al.stream>>>(g.wv, g.hv, n, g.n_heavy, g.totals);
     k_heavy_place<<<grid_for(n, 256, 152 * 4), 256, 0, al.stream>>>(g.wv, g.hv, n, g.n_heavy, g.heavy);
     al.launches += 4;
     al.put(low);
@@ -400,6 +407,7 @@ void free_csr(Csr &g, Alloc &al) {
     al.put(g.wv);
     al.put(g.heavy);
     al.put(g.n_heavy);
+    al.put(g.totals);
     g = Csr{};
 }
 

@@ -55,6 +55,7 @@
 // anew only after a quarter has gone: taking places from one counter at every
 // jump cost 130 us of it at 2M edges (now 30 us).
 #include <limits.h>
+#include <stddef.h>
 
 #include "bt_device.cuh"
 #include "bt_internal.cuh"
@@ -1189,7 +1190,8 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     h.n_alive[0] = (unsigned int)m;
     h.minsup = ~0ull;
     h.minsup2 = ~0ull;
-    BT_CUDA(cudaMemcpyAsync(a.ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
+    BT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), st));
+    BT_CUDA(cudaMemcpyAsync(a.ctl, &h, offsetof(Ctl, hist), cudaMemcpyHostToDevice, st));
     int bps = 0;
     void *kfn = coarse ? (kSeg == 128 ? (void *)k_peel<128, true> : (void *)k_peel<32, true>)
                        : kSeg == 128 ? (void *)k_peel<128, false>
@@ -1200,7 +1202,7 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     void *kargs[] = {&a};
     BT_CUDA(cudaLaunchCooperativeKernel(kfn, grid, block, kargs, 0, st));
     al.launches++;
-    BT_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+    BT_CUDA(cudaMemcpyAsync(&h, a.ctl, offsetof(Ctl, hist), cudaMemcpyDeviceToHost, st));
     BT_CUDA(cudaStreamSynchronize(st));
     if (!coarse) al.mark(kPhPeel, true);
     if (h.err & kErrBarrier) res.status = BT_ERR_CUDA;

@@ -438,9 +438,14 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     g.deep = m;
     g.assigned = assigned != nullptr;
     g.np = np - skip_first;
-    uint32_t *part_e = g.keep(al.get<uint32_t>((size_t)np + 1));
-    uint32_t *part_b = g.keep(al.get<uint32_t>((size_t)np + 1));
-    uint32_t *order = g.keep(al.get<uint32_t>(np));
+    // tables of np + 1 entries, one copy each way: room (64 bits: links of each part,
+    // then their first places), first edges, groups and pairs of each part (then
+    // their first places, handed out by `cursor`), first blooms, order
+    const size_t row = (size_t)np + 1;
+    unsigned long long *room = al.get<unsigned long long>(5 * row);
+    uint32_t *part_e = reinterpret_cast<uint32_t *>(room + row), *tally = part_e + row;
+    uint32_t *cursor = tally, *part_b = tally + 2 * row, *order = part_b + row;
+    g.keep(room);
     uint32_t *out_id = g.keep(al.get<uint32_t>(m));
     g.part_e = part_e;
     g.part_b = part_b;
@@ -449,9 +454,6 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     g.er = g.keep(al.get<uint4>(m));
     uint32_t *keys = al.get<uint32_t>(m), *tk = al.get<uint32_t>(m), *tv = al.get<uint32_t>(m);
     uint2 *place = al.get<uint2>(m);
-    uint32_t *tally = al.get<uint32_t>(2 * ((size_t)np + 1));  // groups, pairs of each part
-    uint32_t *cursor = al.get<uint32_t>(2 * ((size_t)np + 1));
-    unsigned long long *room = al.get<unsigned long long>((size_t)np + 1);  // links; their places
     if (al.err != cudaSuccess) return al.err;
     // edges by part
     k_iota2<<<grid_for(m, 256, wide), 256, 0, al.stream>>>(part, assigned, np, m, keys, out_id);
@@ -463,8 +465,8 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     al.put(tk);
     al.put(tv);
     // groups and pairs of each part, then their places
-    BT_CUDA(cudaMemsetAsync(tally, 0, 8 * ((size_t)np + 1), al.stream));
-    BT_CUDA(cudaMemsetAsync(room, 0, 8 * ((size_t)np + 1), al.stream));
+    BT_CUDA(cudaMemsetAsync(tally, 0, 8 * row, al.stream));
+    BT_CUDA(cudaMemsetAsync(room, 0, 8 * row, al.stream));
     SplitArgs s{ix.bloom_off, nb, ix.pairs, place, np, nullptr, nullptr, nullptr, tally, tally + np + 1,
                 assigned != nullptr};
     const size_t smem = sizeof(uint32_t) * (np + 1) * (3 * (kT / 32) + 2);
@@ -481,19 +483,18 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     k_split_room<<<grid_for(m, kT, wide), kT, 0, al.stream>>>(ix.inc_off, place, m, np, room);
     al.launches++;
     BT_CUDA(cudaGetLastError());
-    std::vector<uint32_t> he(np + 1), ht(2 * (np + 1)), ord(np);
-    std::vector<unsigned long long> hr(np + 1), at(np + 1);
-    BT_CUDA(cudaMemcpyAsync(ht.data(), tally, 8 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
-    BT_CUDA(cudaMemcpyAsync(he.data(), part_e, 4 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
-    BT_CUDA(cudaMemcpyAsync(hr.data(), room, 8 * ((size_t)np + 1), cudaMemcpyDeviceToHost, al.stream));
+    std::vector<unsigned long long> tab(5 * row);
+    BT_CUDA(cudaMemcpyAsync(tab.data(), room, 8 * row + 12 * row, cudaMemcpyDeviceToHost, al.stream));
     BT_CUDA(cudaStreamSynchronize(al.stream));
+    const std::vector<unsigned long long> hr(tab.begin(), tab.begin() + (long)row);
+    uint32_t *he = reinterpret_cast<uint32_t *>(tab.data() + row), *ht = he + row, *hb = ht + 2 * row, *ho = hb + row;
     uint32_t gsum = 0, psum = 0;
     unsigned long long lsum = 0;
     for (uint32_t i = 0; i <= np; ++i) {
-        const uint32_t gi = ht[i], pi = ht[np + 1 + i];
-        ht[i] = gsum;
-        ht[np + 1 + i] = psum;
-        at[i] = lsum;
+        const uint32_t gi = ht[i], pi = ht[row + i];
+        hb[i] = ht[i] = gsum;
+        ht[row + i] = psum;
+        tab[i] = lsum;
         gsum += gi;
         psum += pi;
         lsum += hr[i];
@@ -503,6 +504,7 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     // the heaviest first; those that one block would be long at by a cluster
     const double lim = kHeavy * (double)lsum / np;
     auto heavy = [&](uint32_t p) { return he[p + 1] - he[p] > kBlockEdges || (double)hr[p] > lim; };
+    std::vector<uint32_t> ord(np);
     for (uint32_t i = 0; i < np; ++i) ord[i] = i;
     if (skip_first) ord.erase(ord.begin());
     std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) {
@@ -510,10 +512,8 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
         return hx != hy ? hx : hr[x] > hr[y];
     });
     for (const uint32_t p : ord) g.n_heavy += heavy(p);
-    BT_CUDA(cudaMemcpyAsync(cursor, ht.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
-    BT_CUDA(cudaMemcpyAsync(part_b, ht.data(), 4 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
-    BT_CUDA(cudaMemcpyAsync(room, at.data(), 8 * ((size_t)np + 1), cudaMemcpyHostToDevice, al.stream));
-    BT_CUDA(cudaMemcpyAsync(order, ord.data(), 4 * ord.size(), cudaMemcpyHostToDevice, al.stream));
+    std::copy(ord.begin(), ord.end(), ho);
+    BT_CUDA(cudaMemcpyAsync(room, tab.data(), 40 * row, cudaMemcpyHostToDevice, al.stream));
     uint32_t *sub = al.get<uint32_t>(ix.w2);
     uint2 *pairs = g.keep(al.get<uint2>(psum)), *inc = g.keep(al.get<uint2>(lsum));
     g.bl = g.keep(al.get<BloomRec>(gsum));
@@ -524,7 +524,7 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     s.sub = sub;
     s.bl = g.bl;
     s.groups = cursor;
-    s.members = cursor + np + 1;
+    s.members = cursor + row;
     if (nb) {
         k_split_small<true><<<grid_for(nb, kT, wide), kT, 0, al.stream>>>(s);
         k_split_large<true><<<grid_for(nb, kT, wide), kT, smem, al.stream>>>(s);
@@ -537,9 +537,6 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     BT_CUDA(cudaStreamSynchronize(al.stream));  // the host tables above
     al.put(place);
     al.put(sub);
-    al.put(tally);
-    al.put(cursor);
-    al.put(room);
     return cudaSuccess;
 }
 
