@@ -9,9 +9,10 @@
 // support updates, are those of the one peel of the whole graph (an update of an
 // edge of a higher part is counted where Alg. 5 makes it and left out).  On the
 // 2M-edge graph 39,928 rounds of about 10 us became at most 3,000 a part, of
-// 6-15 us, in 100 parts side by side: the peel went from 384 to 70 ms, the call
-// from 411 to 90; with planted bicliques (2.4M edges) from 539 to 149 ms; 20,000
-// edges from 7.9 to 2.8 ms; a batch of 384 graphs from 237 to 114 ms.
+// 6-15 us, in 85 parts side by side: the peel went from 384 to 69 ms (39 of them
+// the coarse peel, 10 the split, 20 this kernel); with planted bicliques (2.4M
+// edges) from 484 to 118 ms; 20,000 edges from 7.8 to 2.0 ms; a batch of 384
+// graphs from 209 to 84 ms.
 //
 // One round (batch S of edges with support <= k, bloom numbers k_B):
 //   phase 1, over the links of S: a pair of bloom B dies when its other edge is
@@ -55,6 +56,9 @@ namespace cg = cooperative_groups;
 namespace bt {
 namespace {
 
+// threads a block: with 512 the peel of the 2M-edge graph took 73.3 instead of
+// 69.0 ms, of planted bicliques 131 instead of 118, of 1,003 edges 0.69 instead
+// of 0.74
 constexpr int kNT = 1024;
 constexpr unsigned kAll = 0xffffffffu;
 constexpr uint32_t kCluster = 16;  // blocks of the cluster that peels a heavy part
@@ -347,7 +351,6 @@ struct Part {
             mark(head, F, kBatch);
             if (F > kNT) __syncthreads();  // (lay's barrier does for one turn)
         }
-        const uint32_t warp = rank * (kNT / 32) + (tid >> 5);
         for (uint32_t c0 = 0; c0 < F;) {
             uint32_t n = F - c0 < kNT ? F - c0 : kNT;
             const uint32_t i = c0 + tid;
@@ -372,6 +375,12 @@ struct Part {
                 total = lay(n, tid == 0 ? d : 0u, e, 0u, a.inc + lb);
             }
             c0 += n;
+            // a block peels on the blooms it touches: when there are fewer links
+            // than threads, neighbouring shares go to different blocks (else the
+            // first blocks had all the blooms of a small batch; the last part of a
+            // 2M-edge graph, 1,516 rounds by a cluster, went from 77 to 53 ms)
+            const uint32_t warp =
+                total < (uint64_t)nranks * kNT ? (tid >> 5) * nranks + rank : rank * (kNT / 32) + (tid >> 5);
             uint32_t lo, hi;
             dev::share_of((uint32_t)total, warp, nranks * (kNT / 32), lo, hi);
             uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
