@@ -177,6 +177,11 @@ struct Csr {
     // cnt_n entries each (the largest graph) instead of n.
     uint32_t *vbase = nullptr;  // [n], or null for one graph
     uint32_t cnt_n = 0;
+    // Graphs of more vertices than a block has counters in shared memory: the
+    // place of a vertex among those of its own layer, by rank (all wedges of a start
+    // vertex end in its layer), and that of every neighbour; else null.
+    uint32_t *place = nullptr;   // [n]
+    uint32_t *wplace = nullptr;  // [2m]
 };
 
 // The graphs of a disjoint union (bt_decompose_batch): offU/offL (device,
@@ -187,6 +192,11 @@ struct GraphSplit {
     const uint32_t *offU = nullptr, *offL = nullptr;
     uint32_t max_n = 0;
 };
+
+// Graphs of up to this many vertices have all their counters in shared memory
+// (kHotE in count.cu) by rank; above, places in a layer are worth a pass over the
+// arcs (0.1 ms at 2M edges, against 1.7 ms off the index).
+constexpr uint32_t kPlacesFrom = 80 * 1024;
 
 // A start vertex of up to kLightW wedges over up to kLightH middle vertices is
 // counted by a warp.

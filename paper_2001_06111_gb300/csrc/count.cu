@@ -18,8 +18,14 @@
 // (dev::items_of), so every lane has four wedges in flight whatever the degrees.
 // What bounded the dense counters of a block in global memory was the rate of
 // scattered accesses (3 GB of them on the 30M-edge graph): now the counters of the
-// ranks just below the start vertex, the ones most wedges end at, are in shared
-// memory, and only those of lower ranks are in global memory.
+// vertices ranked just below the start vertex, the ones most wedges end at, are in
+// shared memory, and only those of lower ones are in global memory.  Wedges end in
+// the layer they start from, so on graphs with more vertices than counters there
+// the counters go by places in the layer: by rank, half of them were of the other
+// layer.  Wedges that end below the window: 48 to 35 % at 30M edges, 23 to 7 % at
+// 2M; counting 30M edges 320 -> 151 -> 132 ms, building the index of 2M edges 20.4
+// -> 11.2 -> 9.6.  What bounds it at 30M edges are those accesses; at 3M the shared
+// memory path is busy 57 % of the time and the issue slots 41 %.
 #include "bt_device.cuh"
 #include "bt_internal.cuh"
 
@@ -36,6 +42,7 @@ constexpr uint32_t kHot = 88 * 1024;     // 16-bit counters in shared memory
 struct CountArgs {
     const uint64_t *off;
     const uint32_t *adj, *eid, *hv, *pl;
+    const uint32_t *wend, *place;  // what counters go by: places in a layer, or adj and null
     const uint64_t *wv;
     uint32_t lo, hi;
     const uint32_t *heavy, *n_heavy;
@@ -90,7 +97,7 @@ __device__ __forceinline__ uint32_t lay_wedges(CountShared &s, const CountArgs &
 }
 
 // Start vertices with many wedges, one block each, heaviest first.  The counters
-// of the kHot ranks below u are in shared memory (ranks ascend with degree, so
+// of the kHot places below u are in shared memory (they ascend with degree, so
 // they are met by most wedges of a skewed graph), 16 bits each; a start vertex of
 // 2^16 or more middle vertices uses half the ranks with 32 bits.  Those of lower
 // ranks are 32-bit words of this block in global memory: when a count fits 16
@@ -123,7 +130,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
             const uint32_t vb = a.vbase ? a.vbase[u] : 0u;
             const bool narrow = h < 0x10000u;  // a count never exceeds h
             const uint32_t width = narrow ? kHot : kHot / 2;
-            const uint32_t ru = u - vb;
+            const uint32_t ru = a.place ? a.place[u] : u - vb;
             const uint32_t base = ru > width ? ru - width : 0u;  // hot counters are those of ranks [base, ru)
             unsigned long long w2 = 0, nb = 0;
             // pass A: cnt[w] += 1; the second wedge of an end vertex makes its bloom
@@ -137,7 +144,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
 #pragma unroll
                     for (uint32_t r = 0; r < kCU; ++r) {
                         const uint32_t x = x0 + 32u * r + lane, j = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
-                        w[r] = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
+                        w[r] = x < hi ? a.wend[s.at[j] + x] - vb : 0xFFFFFFFFu;
                     }
 #pragma unroll
                     for (uint32_t r = 0; r < kCU; ++r) {
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
                     for (uint32_t r = 0; r < kCU; ++r) {
                         const uint32_t x = x0 + 32u * r + lane;
                         jj[r] = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
-                        w[r] = x < hi ? a.adj[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
+                        w[r] = x < hi ? a.wend[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
                     }
 #pragma unroll
                     for (uint32_t r = 0; r < kCU; ++r) {
@@ -228,7 +235,7 @@ __global__ void __launch_bounds__(kCT) k_count(const __grid_constant__ CountArgs
                     uint32_t j0 = lo < hi ? dev::item_of(s.off, s.n, lo) : 0u;
                     for (uint32_t x0 = lo; x0 < hi; x0 += 32u) {
                         const uint32_t x = x0 + lane, j = dev::items_of(s.off, s.n, x0, j0);
-                        const uint32_t w = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
+                        const uint32_t w = x < hi ? a.wend[s.at[j] + x] - vb : 0xFFFFFFFFu;
                         if (w < base) cold[w] = 0u;
                     }
                     __syncthreads();
@@ -482,7 +489,7 @@ __global__ void __launch_bounds__(kCT) k_emit(const __grid_constant__ EmitArgs e
         const uint32_t vb = a.vbase ? a.vbase[u] : 0u;
         const bool narrow = h < 0x10000u;
         const uint32_t width = narrow ? kHotE : kHotE / 2;
-        const uint32_t ru = u - vb;
+        const uint32_t ru = a.place ? a.place[u] : u - vb;
         const uint32_t base = ru > width ? ru - width : 0u;
         __syncthreads();
         // counts, as in k_count; end vertices of lower ranks with a bloom are listed
@@ -496,7 +503,7 @@ __global__ void __launch_bounds__(kCT) k_emit(const __grid_constant__ EmitArgs e
 #pragma unroll
                 for (uint32_t r = 0; r < kCU; ++r) {
                     const uint32_t x = x0 + 32u * r + lane, j = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
-                    w[r] = x < hi ? a.adj[s.at[j] + x] - vb : 0xFFFFFFFFu;
+                    w[r] = x < hi ? a.wend[s.at[j] + x] - vb : 0xFFFFFFFFu;
                 }
 #pragma unroll
                 for (uint32_t r = 0; r < kCU; ++r) {
@@ -547,7 +554,7 @@ __global__ void __launch_bounds__(kCT) k_emit(const __grid_constant__ EmitArgs e
                 for (uint32_t r = 0; r < kCU; ++r) {
                     const uint32_t x = x0 + 32u * r + lane;
                     jj[r] = dev::items_of(s.off, s.n, x0 + 32u * r, j0);
-                    w[r] = x < hi ? a.adj[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
+                    w[r] = x < hi ? a.wend[s.at[jj[r]] + x] - vb : 0xFFFFFFFFu;
                 }
 #pragma unroll
                 for (uint32_t r = 0; r < kCU; ++r) {
@@ -730,6 +737,8 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     CountArgs a{};
     a.off = g.off;
     a.adj = g.adj;
+    a.place = g.place;
+    a.wend = g.place ? g.wplace : g.adj;
     a.eid = g.eid;
     a.hv = g.hv;
     a.pl = g.pl;
@@ -813,6 +822,8 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     EmitArgs a{};
     a.c.off = g.off;
     a.c.adj = g.adj;
+    a.c.place = g.place;
+    a.c.wend = g.place ? g.wplace : g.adj;
     a.c.eid = g.eid;
     a.c.hv = g.hv;
     a.c.pl = g.pl;

@@ -167,11 +167,26 @@ __global__ void k_wedge_prefix(const uint64_t *off, const uint32_t *row_of, cons
     }
 }
 
-// Internal ids of the other arcs.
-__global__ void k_relabel(const uint32_t *row_of, const uint32_t *adj, uint64_t na, uint32_t *eid, const uint32_t *newid) {
+// Internal ids of the other arcs, and the places of the neighbours (Csr::wplace) if asked for.
+__global__ void k_relabel(const uint32_t *row_of, const uint32_t *adj, uint64_t na, uint32_t *eid, const uint32_t *newid,
+                          const uint32_t *place, uint32_t *wplace) {
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < na;
-         j += (uint64_t)gridDim.x * blockDim.x)
-        if (adj[j] > row_of[j]) eid[j] = newid[eid[j]];
+         j += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t v = adj[j];
+        if (v > row_of[j]) eid[j] = newid[eid[j]];
+        if (place) wplace[j] = place[v];
+    }
+}
+
+// Layer of the vertex of each rank: 1 for the ids from `first` on.
+__global__ void k_layer(const uint32_t *order, uint32_t n, uint32_t first, uint32_t *layer) {
+    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+        layer[r] = order[r] >= first;
+}
+// ones[r]: vertices of layer 1 below rank r.
+__global__ void k_place_in_layer(const uint32_t *layer, const uint32_t *ones, uint32_t n, uint32_t *place) {
+    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+        place[r] = layer[r] ? ones[r] : r - ones[r];
 }
 
 // Start vertices that get a block each, by the power of two of their wedges: the
@@ -359,7 +374,22 @@ cudaError_t build_csr(const int32_t *d_edges, uint64_t m, uint32_t nU, uint32_t 
     BT_CUDA(exclusive_scan_u32(g.hv, hoff, n, nullptr, al));
     k_wedge_prefix<<<grid_for(na, 256), 256, 0, al.stream>>>(g.off, row_of, g.adj, g.eid, low, hoff, na, g.pl,
                                                              reinterpret_cast<unsigned long long *>(g.wv), g.newid);
-    k_relabel<<<grid_for(na, 256), 256, 0, al.stream>>>(row_of, g.adj, na, g.eid, g.newid);
+    // (a fixed arena has no room for it)
+    if (!g.vbase && n > kPlacesFrom && !al.arena) {
+        g.place = al.get<uint32_t>(n);
+        g.wplace = al.get<uint32_t>(na);
+        uint32_t *layer = al.get<uint32_t>(n), *ones = al.get<uint32_t>(n);
+        if (al.err != cudaSuccess) return al.err;
+        const bool upper_first = (flags & BT_TIE_LOWER_FIRST) != 0;
+        k_layer<<<grid_for(n, 256), 256, 0, al.stream>>>(order, n, upper_first ? nU : nL, layer);
+        BT_CUDA(exclusive_scan_u32(layer, ones, n, nullptr, al));
+        k_place_in_layer<<<grid_for(n, 256), 256, 0, al.stream>>>(layer, ones, n, g.place);
+        al.launches += 2;
+        al.put(layer);
+        al.put(ones);
+        g.cnt_n = nU > nL ? nU : nL;
+    }
+    k_relabel<<<grid_for(na, 256), 256, 0, al.stream>>>(row_of, g.adj, na, g.eid, g.newid, g.place, g.wplace);
     k_heavy_count<<<grid_for(n, 256, 152 * 4), 256, 0, al.stream>>>(g.wv, g.hv, n, g.n_heavy, g.totals);
     k_heavy_place<<<grid_for(n, 256, 152 * 4), 256, 0, al.stream>>>(g.wv, g.hv, n, g.n_heavy, g.heavy);
     al.launches += 4;
@@ -399,6 +429,8 @@ cudaError_t scatter_u8(const uint8_t *in, const uint32_t *newid, uint8_t *out, u
 void free_csr(Csr &g, Alloc &al) {
     al.put(g.newid);
     al.put(g.vbase);
+    al.put(g.place);
+    al.put(g.wplace);
     al.put(g.off);
     al.put(g.adj);
     al.put(g.eid);

@@ -69,3 +69,15 @@ def test_start_vertex_of_many_middles(h, nL):
 def test_skewed_graph(h):
     g = synth.chunglu(9000, 4000, 60000, 2.0, 2.2, seed=5)
     check(h, g.edges, g.nU, g.nL)
+
+
+# around 81,920 vertices, above which counters go by places in a layer instead of
+# ranks; either layer larger, either convention of ids
+@pytest.mark.parametrize("flags", [0, bt.BT_TIE_LOWER_FIRST])
+@pytest.mark.parametrize("nU,nL", [(61920, 20000), (61921, 20000), (20000, 61921), (3000, 120000), (180000, 3000)])
+def test_places_in_a_layer(h, nU, nL, flags):
+    g = synth.chunglu(nU, nL, 50000, 2.0, 2.2, seed=nU)
+    sup = oracle.support(g.edges, nU, nL)
+    np.testing.assert_array_equal(bt.bt_count_support(h, g.edges, nU, nL, flags=flags), sup)
+    st = bt.bt_build_index(h, g.edges, nU, nL, flags=flags)
+    assert 4 * st["n_butterflies"] == int(sup.sum())
