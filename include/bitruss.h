@@ -234,6 +234,8 @@ int bt_profile_read(const bt_handle *h, bt_profile *out);
  *                       (instead of two a thread) links itself; longer lists become
  *                       incidence items.  (These two change no result; they
  *                       make small graphs take the paths large ones take.)
+ * hold_barrier, join_cap and block_links belong to the peel by the whole grid:
+ * with one of them set, calls peel that way throughout.
  * limits == NULL restores every default.  Errors: BT_ERR_ARG (h NULL).
  */
 typedef struct {
@@ -285,13 +287,14 @@ typedef struct {
     uint32_t *phi_out;      /* uint32[m] */
 } bt_graph;
 
-/* Batch schedule.  Zero fields are chosen by the library: the autotuner
- * times candidate schedules on a sample of the batch (about 8M edges of its
- * graphs) and caches the winner in the handle per batch signature (log4 of
- * the total edges and of the largest graph). */
+/* Batch schedule.  Zero fields are chosen by the library, per batch signature
+ * (log4 of the total edges and of the largest graph), and kept in the handle.
+ * Counting and the part peel pick their own schedules; where the whole peel
+ * is one launch of the grid (a server with one worker, bt_set_limits) candidate
+ * schedules are timed on a sample of the batch (about 8M edges of its graphs). */
 typedef struct {
     uint64_t max_edges_per_launch;  /* graphs are packed into unions of at most this many edges */
-    uint32_t count_threads;         /* wedge-count / index block size: 256, 512 or 1024 */
+    uint32_t count_threads;         /* 256, 512 or 1024 (reported; no longer changes anything) */
     uint32_t peel_item;             /* peel work item: 32, 64 or 128 links / pair slots per warp */
     uint32_t reserved[2];
 } bt_tune;
@@ -315,8 +318,8 @@ typedef struct {
  * decompositions (Defs. 4-5): the graphs are relabelled on the device into
  * one union (upper and lower ids shifted per graph, keeping every graph's own
  * priority order, Def. 7) and decomposed by one pipeline -- one count, one
- * index emit and one persistent peeling launch -- so the peel's rounds are
- * shared by all graphs instead of paid per graph.  Results are exactly those
+ * index emit and one peel -- so the peel's coarse rounds are shared by all
+ * graphs instead of paid per graph.  Results are exactly those
  * of bt_decompose on each graph alone.  Graphs are packed into unions of at
  * most tune->max_edges_per_launch edges (0: as many as device memory allows;
  * a union that does not fit is split in two and retried).

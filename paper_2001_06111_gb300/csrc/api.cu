@@ -26,7 +26,7 @@ struct bt_handle {
     std::string err;
     bt::Prof prof;
     bt_profile last{};
-    int count_nt = 1024;  // schedule used by the next pipeline run (1024: fewest per-block counter arrays)
+    int count_nt = 1024;  // reported (counting and emit pick their own tiers)
     int peel_seg = 32;
     int peel_sms = 0;     // SMs the peel kernel spans (0: all); a server worker takes its share
     bt::Side side;
@@ -84,7 +84,7 @@ bool grid_peel_only(const bt_handle *h) {
 
 // Up to this many edges (of all graphs of a batch) are peeled by one block as one
 // part.  Below about 1,000 edges that takes less than the rounds of a coarse
-// peel do (300 edges: 0.26 against 0.43 ms; 1,003: 0.72 / 0.75; 2,500: 1.19 / 0.93).
+// peel do (peel of 300 edges: 0.26 against 0.43 ms; 1,003: 0.72 / 0.75; 2,500: 1.19 / 0.93).
 constexpr uint64_t kWholeEdges = 1024;
 
 int peel_sms(const bt_handle *h) { return h->peel_sms > 0 ? h->peel_sms : h->num_sms; }
@@ -538,7 +538,10 @@ static cudaError_t peel_by_parts(bt_handle *h, const bt::Index &ix, const uint64
         o.max_parts = bt::kPartsMax;
         // more parts cost the coarse peel more rounds, fewer leave SMs idle in
         // the fine one; the best counts grew with the cube root of the twin
-        // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150)
+        // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150).
+        // Peel with 0.2 / 0.305 / 0.45 times it: 200,000 edges 6.9 / 7.4 / 11.3
+        // ms, 2M 70.4 / 69.0 / 80.0, planted bicliques 136 / 118 / 117, 384
+        // graphs 97 / 84 / 87
         o.parts_hint = (uint32_t)(0.305 * std::cbrt((double)ix.w2)) + 1;
         bt::PeelResult c;
         if (e == cudaSuccess) e = bt::peel(ix, sup, part, c, peel_sms(h), al, seg, &o);

@@ -12,7 +12,7 @@
 // 6-15 us, in 85 parts side by side: the peel went from 384 to 69 ms (39 of them
 // the coarse peel, 10 the split, 20 this kernel); with planted bicliques (2.4M
 // edges) from 484 to 118 ms; 20,000 edges from 7.8 to 2.0 ms; a batch of 384
-// graphs from 209 to 84 ms.
+// graphs from 209 to 82 ms.
 //
 // One round (batch S of edges with support <= k, bloom numbers k_B):
 //   phase 1, over the links of S: a pair of bloom B dies when its other edge is

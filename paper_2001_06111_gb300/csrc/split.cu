@@ -27,7 +27,10 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kFlag = 0x80000000u;
 constexpr uint32_t kMaxParts = kPartsMax;
 constexpr int kT = 256;
-// a part with more links than this many times the mean is peeled by a cluster
+// A part with more links than this many times the mean is peeled by a cluster.  Peel
+// with 2.5 instead: 200,000 edges 8.9 against 7.4 ms, 2M edges 74.2 against 69.0
+// (the clusters take the SMs of the other parts, and their barriers cost more);
+// with 6 or 12: the same within 1 %.
 constexpr double kHeavy = 4.0;
 constexpr int kSmall = 8;  // pairs of a bloom that one thread groups by itself
 constexpr unsigned kFull = 0xffffffffu;
