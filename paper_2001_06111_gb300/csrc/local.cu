@@ -11,7 +11,7 @@
 // 2M-edge graph 39,928 rounds of about 10 us became at most 3,000 a part, of
 // 6-15 us, in 85 parts side by side: the peel went from 384 to 69 ms (39 of them
 // the coarse peel, 10 the split, 20 this kernel); with planted bicliques (2.4M
-// edges) from 484 to 118 ms; 20,000 edges from 7.8 to 2.0 ms; a batch of 384
+// edges) from 484 to 112 ms; 20,000 edges from 7.8 to 2.0 ms; a batch of 384
 // graphs from 209 to 82 ms.
 //
 // One round (batch S of edges with support <= k, bloom numbers k_B):
