@@ -1125,17 +1125,27 @@ inline unsigned grid_for(uint64_t items, int threads, unsigned cap) {
 
 cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, PeelResult &res,
                  int num_sms, Alloc &al, int seg, const PeelOpts *opts) {
-    const uint32_t kSeg = seg == 128 ? 128u : seg == 64 ? 64u : 32u;
+    const bool coarse = opts && opts->snap;
+    // (a coarse peel has no kernel of 64-entry items: every size below goes by the
+    // items of the kernel that is launched)
+    const uint32_t kSeg = seg == 128 ? 128u : seg == 64 && !coarse ? 64u : 32u;
     const uint32_t kT = (uint32_t)peel_threads(kSeg);
     const uint32_t kJoinCap = kT, kBlockLinks = 2 * kT;
     const uint64_t m = ix.m;
     res = PeelResult{};
     if (m == 0 || (opts && opts->assigned && opts->m_active == 0)) return cudaSuccess;
+    int bps = 0;
+    void *kfn = coarse ? (kSeg == 128 ? (void *)k_peel<128, true> : (void *)k_peel<32, true>)
+                       : kSeg == 128 ? (void *)k_peel<128, false>
+                                     : kSeg == 64 ? (void *)k_peel<64, false> : (void *)k_peel<32, false>;
+    BT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, (int)kT, 0));
+    if (bps < 1) return cudaErrorCooperativeLaunchTooLarge;
+    const dim3 grid((unsigned)(num_sms * bps)), block(kT);
     // one round queues each edge and each bloom at most once
     const uint64_t item_cap = m + (2 * ix.w2) / kSeg + 2;
     // (each bloom at most once), beside the places a warp takes and leaves empty
     // in an incidence phase: fewer than it fills each time, and a last stock
-    const uint64_t bseg_cap = 2 * (ix.nb + ix.w2 / kSeg) + (uint64_t)num_sms * (kT / 32) * kTake + 2;
+    const uint64_t bseg_cap = 2 * (ix.nb + ix.w2 / kSeg) + (uint64_t)grid.x * (kT / 32) * kTake + 2;
     PeelArgs a{};
     a.m = m;
     a.inc_off = ix.inc_off;
@@ -1169,7 +1179,6 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     a.m_active = (opts && opts->assigned) ? opts->m_active : m;
     a.k_init = opts ? opts->k_init : 0;
     a.assign_from = opts ? opts->assign_from : 0;
-    const bool coarse = opts && opts->snap;
     a.snap = coarse ? opts->snap : nullptr;
     if (coarse) {
         // weights add up to less than 2^31
@@ -1195,13 +1204,6 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     h.minsup2 = ~0ull;
     BT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), st));
     BT_CUDA(cudaMemcpyAsync(a.ctl, &h, offsetof(Ctl, hist), cudaMemcpyHostToDevice, st));
-    int bps = 0;
-    void *kfn = coarse ? (kSeg == 128 ? (void *)k_peel<128, true> : (void *)k_peel<32, true>)
-                       : kSeg == 128 ? (void *)k_peel<128, false>
-                                     : kSeg == 64 ? (void *)k_peel<64, false> : (void *)k_peel<32, false>;
-    BT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, (int)kT, 0));
-    if (bps < 1) return cudaErrorCooperativeLaunchTooLarge;
-    dim3 grid((unsigned)(num_sms * bps)), block(kT);
     void *kargs[] = {&a};
     BT_CUDA(cudaLaunchCooperativeKernel(kfn, grid, block, kargs, 0, st));
     al.launches++;

@@ -84,6 +84,21 @@ def test_batches_same_as_the_grid_peel(h, n, hi):
         np.testing.assert_array_equal(p0, p1)
 
 
+# every item size a batch may ask for, on blocks of many links an edge and one level:
+# all edges leave in one jump, so one round queues every link (K_{60,60} is the
+# smallest of these whose 32-entry items number more than its 64-entry items
+# leave room for)
+@pytest.mark.parametrize("item", [32, 64, 128])
+@pytest.mark.parametrize("sides", [[(60, 60)], [(100, 100)], [(128, 336)], [(200, 200)],
+                                   [(60, 60), (33, 40), (128, 200), (200, 200)]])
+def test_bicliques_by_item_size(h, sides, item):
+    out, st = bt.bt_decompose_batch(h, [(pins.biclique(a, b), a, b) for a, b in sides], count_threads=512,
+                                    peel_item=item)
+    assert (st["rounds"], st["levels"]) == (len({(a - 1) * (b - 1) for a, b in sides}),) * 2
+    for (a, b), (sup, phi) in zip(sides, out):
+        assert (sup == (a - 1) * (b - 1)).all() and (phi == (a - 1) * (b - 1)).all()
+
+
 # passes of the progressive compression: assigned edges among the pairs, a first part
 # below the recorded levels (the default reading) or none (Alg. 7's)
 @pytest.mark.parametrize("flags", [0, bt.BT_PC_RECOUNT])
