@@ -62,9 +62,14 @@ struct CountShared {
     uint32_t off[kCT + 1];           // first wedge of each middle vertex
     uint32_t e[kCT + 1];             // its edge (u, v)
     unsigned long long at[kCT + 1];  // wedge x of item j is arc at[j] + x
-    uint32_t acc[kCT], inc[kCT];     // support and links of (u, v) from these (supports are below m < 2^31)
+    uint32_t acc[kCT + 1], inc[kCT + 1];  // support and links of (u, v) from these (supports are below m < 2^31)
     uint32_t u;
 };
+// lanes past the last wedge get item n (dev::items_of), which has a place in every table
+static_assert(sizeof(CountShared::e) == sizeof(CountShared::off) && sizeof(CountShared::acc) == sizeof(CountShared::off) &&
+                  sizeof(CountShared::inc) == sizeof(CountShared::off) &&
+                  sizeof(CountShared::at) == 2 * sizeof(CountShared::off),
+              "tables of kCT items and one more");
 
 // Lays the wedges over middle vertices [c0, c0 + kCT) of u side by side, empty
 // ones left out.  Returns their number.
@@ -431,7 +436,7 @@ __device__ __forceinline__ void put_pair(const EmitArgs &a, uint32_t slot, uint3
 
 struct EmitShared {
     CountShared c;
-    unsigned long long front[kCT];  // first free place of (u, v)'s list
+    unsigned long long front[kCT + 1];  // first free place of (u, v)'s list
     unsigned long long alloc;       // blooms (high) and pairs (low) of the start vertex handed out
     uint32_t n_found;
 };
@@ -578,7 +583,7 @@ __global__ void __launch_bounds__(kCT) k_emit(const __grid_constant__ EmitArgs e
                 bool fu[kCU], fw[kCU];
 #pragma unroll
                 for (uint32_t r = 0; r < kCU; ++r) {
-                    fu[r] = s.inc[jj[r]] != 0u;
+                    fu[r] = in[r] && s.inc[jj[r]] != 0u;
                     fw[r] = in[r] && a.assigned && a.assigned[ev[r]];
                     back[r] = in[r] && !fw[r] ? atomicAdd(&ea.cursor[ev[r]], ~0ull) : 0ull;
                     at[r] = in[r] && !fu[r] ? atomicAdd(&es.front[jj[r]], 1ull) : 0ull;

@@ -37,6 +37,19 @@ def test_bicliques(h, a, b):
     assert st["n_butterflies"] == a * (a - 1) * b * (b - 1) // 4
 
 
+# tiles of exactly 1,024 middle vertices, whose last windows of wedges are not full,
+# with assigned edges among them (a pass of the progressive compression at every
+# level): all edges of K_{a,b} and b more upper vertices of one edge each
+@pytest.mark.parametrize("a,b", [(2, 1024), (3, 1024), (2, 2047), (3, 2048)])
+def test_full_tiles_with_assigned_edges(h, a, b):
+    e = np.concatenate([pins.biclique(a, b), np.stack([a + np.arange(b), np.arange(b)], 1)]).astype(np.int32)
+    want = np.where(e[:, 0] < a, (a - 1) * (b - 1), 0)
+    for tau in (0.5, 1.0):
+        sup, phi, _ = bt.bt_decompose_progressive(h, e, a + b, b, tau=tau)
+        np.testing.assert_array_equal(sup.astype(np.int64), want)
+        np.testing.assert_array_equal(phi.astype(np.int64), want)
+
+
 # a hub pair over all lower vertices beside many vertices of low degree: end vertices
 # far below the hub, in and out of the counters in shared memory
 @pytest.mark.parametrize("nU,nL", [(90110, 700), (90112, 700), (140000, 3000)])
