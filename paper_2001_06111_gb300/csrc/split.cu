@@ -226,7 +226,10 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
     extern __shared__ uint32_t s_tab[];  // three rows a warp; then the block's tally
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t row = a.np + 1u;
-    uint32_t *cur = s_tab + (size_t)w * 3 * row, *gid = cur + row, *known = gid + row;
+    // a part's pairs, then the next place of its group's; its group; its assigned
+    // edges, then the size of its group (places take all 32 bits, so what tells a
+    // group in the record from one in `out` is a row of its own)
+    uint32_t *cur = s_tab + (size_t)w * 3 * row, *gid = cur + row, *known = gid + row, *size = known;
     uint32_t *t_groups = s_tab + (size_t)kWarps * 3 * row, *t_members = t_groups + row;
     if constexpr (!kPlace) {
         for (uint32_t i = threadIdx.x; i < 2 * row; i += kT) t_groups[i] = 0;
@@ -281,7 +284,8 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
                         const uint32_t id = atomicAdd(&a.groups[i], 1u);
                         const uint32_t at = n > 2u ? atomicAdd(&a.members[i], n) : 0u;
                         gid[i] = id;
-                        cur[i] = n > 2u ? at : kFlag;  // up to two go to the record
+                        cur[i] = at;
+                        size[i] = n;
                         head(a.bl + id, n > 2u ? at : higher, n, left);
                         if (n > 2u) a.bl[id].pair[0].x = higher;
                     }
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(kT) k_split_large(const SplitArgs a) {
                     a.sub[off + i] = id;
                     if (id != kNone) {
                         const uint32_t c = atomicAdd(&cur[qi], 1u);
-                        if (c & kFlag) a.bl[id].pair[c & 1u] = placed(x, y);
+                        if (size[qi] <= 2u) a.bl[id].pair[c] = placed(x, y);
                         else a.out[c] = placed(x, y);
                     }
                 }

@@ -84,6 +84,21 @@ def test_batches_same_as_the_grid_peel(h, n, hi):
         np.testing.assert_array_equal(p0, p1)
 
 
+# K_{n,n} without one edge: the 2n - 2 edges at its ends leave first, then the rest
+# at the same level, so all pairs are groups of more than two in one part; 1,640
+# a side make 2.2e9 pairs, more than 2^31 of them in such groups
+@pytest.mark.parametrize("n", [61, 300, 1640])
+def test_pair_places_of_all_32_bits(n):
+    e = pins.biclique(n, n)
+    e = e[(e[:, 0] > 0) | (e[:, 1] > 0)]
+    with bt.bt_create(0) as own:  # (its memory goes back with it: 150 GB for 1,640)
+        sup, phi, st = bt.bt_decompose(own, e, n, n)
+    at_end = (e[:, 0] == 0) | (e[:, 1] == 0)
+    assert (sup == np.where(at_end, (n - 1) * (n - 2), n * (n - 2))).all()
+    assert (phi == (n - 1) * (n - 2)).all()
+    assert (st["rounds"], st["levels"], st["phi_max"]) == (2, 1, (n - 1) * (n - 2))
+
+
 # every item size a batch may ask for, on blocks of many links an edge and one level:
 # all edges leave in one jump, so one round queues every link (K_{60,60} is the
 # smallest of these whose 32-entry items number more than its 64-entry items
