@@ -36,6 +36,35 @@ struct Side {
     cudaEvent_t fork = nullptr, join = nullptr;
 };
 
+// A fork to the side stream and its join.  Whichever way the call goes on, an error
+// return between the two among them, its stream waits for the side stream's
+// work before anything that work uses can be freed (stream-ordered).
+class Forked {
+public:
+    Forked(const Side &side, cudaStream_t stream) : side_(side), stream_(stream) {}
+    Forked(const Forked &) = delete;
+    ~Forked() { join(); }
+    cudaError_t fork() {
+        cudaError_t e = cudaEventRecord(side_.fork, stream_);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(side_.stream, side_.fork, 0);
+        open_ = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join() {
+        if (!open_) return cudaSuccess;
+        open_ = false;
+        cudaError_t e = cudaEventRecord(side_.join, side_.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream_, side_.join, 0);
+        if (e != cudaSuccess) cudaStreamSynchronize(side_.stream);
+        return e;
+    }
+
+private:
+    const Side &side_;
+    cudaStream_t stream_;
+    bool open_ = false;
+};
+
 // Stream-ordered scratch allocation from the handle's memory pool, plus the
 // call's launch counter and profiler.
 struct Alloc {

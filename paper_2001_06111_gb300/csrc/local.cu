@@ -712,12 +712,11 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_f
     BT_CUDA(cudaMemsetAsync(hd, 0, sizeof(Head), st));
     BT_CUDA(cudaMemsetAsync(a.depth, 0, sizeof(uint32_t) * (deep + 1), st));
     if (g.out_id && assign_from > 0) BT_CUDA(cudaMemsetAsync(a.phi, 0xFF, sizeof(uint32_t) * m, st));
+    Forked side(*al.side, st);
     if (g.n_heavy) {
         // the heavy parts, each by a cluster of blocks, beside the kernel of the
         // others, which fills the rest of the SMs
-        const Side &side = *al.side;
-        BT_CUDA(cudaEventRecord(side.fork, st));
-        BT_CUDA(cudaStreamWaitEvent(side.stream, side.fork, 0));
+        BT_CUDA(side.fork());
         const int smem = (int)sizeof(Shared);
         BT_CUDA(cudaFuncSetAttribute(k_peel_parts<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         BT_CUDA(cudaFuncSetAttribute(k_peel_parts<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -731,7 +730,7 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_f
         cfg.blockDim = dim3(kNT);
         cfg.gridDim = dim3(kCluster);
         cfg.dynamicSmemBytes = sizeof(Shared);
-        cfg.stream = side.stream;
+        cfg.stream = al.side->stream;
         int nc = 0;
         BT_CUDA(cudaOccupancyMaxActiveClusters(&nc, k_peel_parts<true>, &cfg));
         if (nc > num_sms / (int)kCluster) nc = num_sms / (int)kCluster;
@@ -742,7 +741,6 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_f
         h.np = g.n_heavy;
         h.queue = &hd->heavy_queue;
         BT_CUDA(cudaLaunchKernelEx(&cfg, k_peel_parts<true>, h));
-        BT_CUDA(cudaEventRecord(side.join, side.stream));
         al.launches++;
         a.order = g.order + g.n_heavy;
         a.np = g.np - g.n_heavy;
@@ -754,7 +752,7 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_f
         k_peel_parts<false><<<grid, kNT, smem, st>>>(a);
         al.launches++;
     }
-    if (g.n_heavy) BT_CUDA(cudaStreamWaitEvent(st, al.side->join, 0));
+    BT_CUDA(side.join());
     if (g.out_id) {
         k_unplace<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(a.phi, g.out_id, m, phi_out);
         al.launches++;
