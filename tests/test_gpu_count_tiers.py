@@ -94,3 +94,17 @@ def test_places_in_a_layer(h, nU, nL, flags):
     np.testing.assert_array_equal(bt.bt_count_support(h, g.edges, nU, nL, flags=flags), sup)
     st = bt.bt_build_index(h, g.edges, nU, nL, flags=flags)
     assert 4 * st["n_butterflies"] == int(sup.sum())
+
+
+# the pairs of a bloom of many lie about in the order of their middle vertices (the peel
+# of dense blooms walks along their edges): a block places 4,096 neighbouring wedges
+# at a time, some 30 middle vertices here, where 32 shares of the wedges would
+# spread any 32 neighbouring pairs over nearly all 1,000
+def test_pairs_of_dense_blooms_in_order(h):
+    a, b = 150, 1000
+    st = bt.bt_build_index(h, pins.biclique(a, b), a, b)
+    k, first, pairs, _ = bt.bt_index_export(h, st, a * b)
+    for i in range(len(k) - 100, len(k)):
+        mid = pairs[first[i]:first[i] + k[i], 0].astype(np.int64) % b
+        assert k[i] == b and len(np.unique(mid)) == b
+        assert np.median([np.ptp(mid[j:j + 32]) for j in range(0, b - 32, 32)]) < b / 2
