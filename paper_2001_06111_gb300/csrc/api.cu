@@ -517,72 +517,81 @@ static bool as_one_part(const bt_handle *h, uint64_t m) { return !grid_peel_only
 // Peels index ix by parts: its edges are first told apart by ranges of bitruss
 // numbers (a coarse peel by the whole grid), then the ranges are peeled
 // independently of one another (local.cu).  pc: the limits of a pass of the
-// progressive compression, or null.
-static cudaError_t peel_by_parts(bt_handle *h, const bt::Index &ix, const uint64_t *sup, uint32_t *phi,
-                                 bt::PeelResult &pr, int seg, const bt::PeelOpts *pc, bt::Alloc &al) {
-    bt::PartGraph g;
-    cudaError_t e = cudaSuccess;
-    const size_t held = al.live.size();
-    al.mark(bt::kPhPeel, false);
-    if (ix.twin_links) {
-        e = bt::one_part(ix, sup, g, peel_sms(h), al);
-        if (e == cudaSuccess) e = bt::peel_parts(g, phi, 0, pr, peel_sms(h), al);
-    } else {
-        uint32_t *part = al.get<uint32_t>(ix.m);
-        int *snap = al.get<int>(ix.m);
-        e = al.err;
-        bt::PeelOpts o;
-        if (pc) o = *pc;
-        o.assign_from = 0;
-        o.snap = snap;
-        o.max_parts = bt::kPartsMax;
-        // more parts cost the coarse peel more rounds, fewer leave SMs idle in
-        // the fine one; the best counts grew with the cube root of the twin
-        // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150).
-        // Peel with 0.2 / 0.305 / 0.45 times it: 200,000 edges 6.9 / 7.4 / 11.3
-        // ms, 2M 70.4 / 69.0 / 80.0, planted bicliques 136 / 118 / 117, 384
-        // graphs 97 / 84 / 87
-        o.parts_hint = (uint32_t)(0.305 * std::cbrt((double)ix.w2)) + 1;
-        bt::PeelResult c;
-        if (e == cudaSuccess) e = bt::peel(ix, sup, part, c, peel_sms(h), al, seg, &o);
-        pr = bt::PeelResult{};
-        pr.status = c.status;
-        if (e == cudaSuccess && c.status == BT_OK) {
-            // a pass's first part lies below the level from which phi is recorded
-            const bool first = o.k_init > 0;
-            e = bt::parts_of_ranges(ix, part, snap, c.parts, o.assigned, first, g, peel_sms(h), al);
-            if (e == cudaSuccess && g.np > 0)
-                e = bt::peel_parts(g, phi, pc ? pc->assign_from : 0, pr, peel_sms(h), al);
-            pr.rounds += c.first_rounds;
-            pr.levels += c.first_levels;
-            pr.updates += c.first_updates;
-            const uint64_t lim = h->limits.peel_round_limit;
-            if (lim && pr.rounds > lim + 1 && pr.status == BT_OK) pr.status = BT_ERR_NOCONVERGE;
-            pr.slots += c.slots;
-            pr.scanned += c.scanned;
-        }
-        al.put(part);
-        al.put(snap);
+// progressive compression, or null.  whole: nothing was peeled, the graph is not
+// one for parts.
+static cudaError_t peel_ranges(bt_handle *h, const bt::Index &ix, const uint64_t *sup, uint32_t *phi,
+                               bt::PeelResult &pr, int seg, const bt::PeelOpts *pc, bt::Alloc &al, bool &whole) {
+    uint32_t *part = al.get<uint32_t>(ix.m);
+    int *snap = al.get<int>(ix.m);
+    if (al.err != cudaSuccess) return al.err;
+    bt::PeelOpts o;
+    if (pc) o = *pc;
+    o.assign_from = 0;
+    o.snap = snap;
+    o.max_parts = bt::kPartsMax;
+    // more parts cost the coarse peel more rounds, fewer leave SMs idle in
+    // the fine one; the best counts grew with the cube root of the twin
+    // pairs (33 k: 8-12, 249 k: 24, 1.8 M: 40, 52 M: 60-160, 129 M: 150).
+    // Peel with 0.2 / 0.305 / 0.45 times it: 200,000 edges 6.9 / 7.4 / 11.3
+    // ms, 2M 70.4 / 69.0 / 80.0, planted bicliques 136 / 118 / 117, 384
+    // graphs 97 / 84 / 87
+    o.parts_hint = (uint32_t)(0.305 * std::cbrt((double)ix.w2)) + 1;
+    bt::PeelResult c;
+    BT_CUDA(bt::peel(ix, sup, part, c, peel_sms(h), al, seg, &o));
+    pr = bt::PeelResult{};
+    pr.status = c.status;
+    whole = c.status == BT_OK && c.narrow;
+    if (c.status != BT_OK || whole) return cudaSuccess;
+    const long long from = pc ? pc->assign_from : 0;
+    // part 0 is not peeled again: a pass's first part lies below the level from
+    // which phi is recorded, and edges in no butterfly are one batch of level 0
+    const bool first = o.k_init > 0 || c.zero_edges > 0;
+    if (c.zero_edges && from <= 0) BT_CUDA(cudaMemsetAsync(phi, 0, sizeof(uint32_t) * ix.m, h->stream));
+    if (c.parts > (uint32_t)first) {
+        bt::PartGraph g;
+        BT_CUDA(bt::parts_of_ranges(ix, part, snap, c.parts, o.assigned, first, c.first_rounds, g, peel_sms(h),
+                                    al));
+        whole = g.lopsided;
+        if (whole) return cudaSuccess;
+        BT_CUDA(bt::peel_parts(g, phi, from, pr, peel_sms(h), al));
     }
-    al.mark(bt::kPhPeel, true);
-    if (e == cudaErrorMemoryAllocation && !al.injected && !ix.twin_links) {
-        // parts need about 46 more bytes a twin pair than the grid-wide peel
-        // alone: an index that leaves no room for them is still peeled
-        cudaGetLastError();
-        al.undo_to(held);
-        al.err = cudaSuccess;
-        e = cudaStreamSynchronize(h->stream);
-        return e == cudaSuccess ? bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg, pc) : e;
-    }
-    bt::free_parts(g, al);
-    return e;
+    pr.rounds += c.zero_edges ? 1 : c.first_rounds;
+    pr.levels += c.zero_edges ? 1 : c.first_levels;
+    pr.updates += c.first_updates;
+    const uint64_t lim = h->limits.peel_round_limit;
+    if (lim && pr.rounds > lim + 1 && pr.status == BT_OK) pr.status = BT_ERR_NOCONVERGE;
+    pr.slots += c.slots;
+    pr.scanned += c.scanned;
+    return cudaSuccess;
 }
 
-// Peels the handle's index.
-static cudaError_t peel_index(bt_handle *h, const uint64_t *sup, uint32_t *phi, bt::PeelResult &pr, int seg,
-                              bt::Alloc &al) {
-    if (grid_peel_only(h)) return bt::peel(h->index, sup, phi, pr, peel_sms(h), al, seg);
-    return peel_by_parts(h, h->index, sup, phi, pr, seg, nullptr, al);
+// Peels index ix.  parts: by parts where that pays.
+static cudaError_t peel_index(bt_handle *h, const bt::Index &ix, const uint64_t *sup, uint32_t *phi,
+                              bt::PeelResult &pr, int seg, const bt::PeelOpts *pc, bool parts, bt::Alloc &al) {
+    const size_t held = al.live.size();
+    cudaError_t e = cudaSuccess;
+    bool whole = !parts;
+    al.mark(bt::kPhPeel, false);
+    if (parts && ix.twin_links) {
+        bt::PartGraph g;
+        e = bt::one_part(ix, sup, g, peel_sms(h), al);
+        if (e == cudaSuccess) e = bt::peel_parts(g, phi, 0, pr, peel_sms(h), al);
+    } else if (parts) {
+        e = peel_ranges(h, ix, sup, phi, pr, seg, pc, al, whole);
+        if (e == cudaErrorMemoryAllocation && !al.injected) {
+            // parts need about 46 more bytes a twin pair than the grid-wide peel
+            // alone: an index that leaves no room for them is still peeled
+            cudaGetLastError();
+            al.err = cudaSuccess;
+            al.undo_to(held);
+            e = cudaStreamSynchronize(h->stream);
+            whole = true;
+        }
+    }
+    al.undo_to(held);  // what the parts were made of
+    if (e == cudaSuccess && whole) e = bt::peel(ix, sup, phi, pr, peel_sms(h), al, seg, pc);
+    al.mark(bt::kPhPeel, true);
+    return e;
 }
 
 int bt_build_index(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL,
@@ -689,7 +698,7 @@ int bt_decompose(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, ui
         // and 21.9 s with 32; on graphs with up to 2e8 pairs 32 measured
         // 3-8 % faster than 64
         const int seg = h->index.w2 > (1ull << 30) ? 128 : h->peel_seg;
-        cudaError_t e = peel_index(h, s_int, p_int, pr, seg, al);
+        cudaError_t e = peel_index(h, h->index, s_int, p_int, pr, seg, nullptr, !grid_peel_only(h), al);
         if (e == cudaSuccess) e = bt::gather_u64(s_int, h->index.newid, d_sup, m, al);
         if (e == cudaSuccess) e = bt::gather_u32(p_int, h->index.newid, d_phi, m, al);
         if (e != cudaSuccess) rc = cuda_fail(h, e, "peeling");
@@ -870,7 +879,7 @@ static int decompose_union(bt_handle *h, const bt_graph *graphs, uint32_t n, uin
     }
     bt::PeelResult pr;
     if (rc == BT_OK && M > 0) {
-        e = peel_index(h, d_sup, d_phi, pr, h->peel_seg, al);
+        e = peel_index(h, h->index, d_sup, d_phi, pr, h->peel_seg, nullptr, !grid_peel_only(h), al);
         // results back to input order (the edge array is free by now: reuse it)
         uint64_t *g_sup = reinterpret_cast<uint64_t *>(d_edges);
         uint32_t *g_phi = al.get<uint32_t>(M);
@@ -1227,9 +1236,7 @@ int bt_decompose_progressive(bt_handle *h, const int32_t *edges, uint64_t m, uin
                 e = cudaMemsetAsync(phi_local, 0xFF, 4 * pc_n, h->stream);
                 // (a pass over few edges is over before its parts would be made)
                 const bool parts = !grid_peel_only(h) && o.m_active > kWholeEdges;
-                if (e == cudaSuccess)
-                    e = parts ? peel_by_parts(h, ix, sup_c, phi_local, pr, h->peel_seg, &o, al)
-                              : bt::peel(ix, sup_c, phi_local, pr, peel_sms(h), al, h->peel_seg, &o);
+                if (e == cudaSuccess) e = peel_index(h, ix, sup_c, phi_local, pr, h->peel_seg, &o, parts, al);
                 if (e == cudaSuccess) e = bt::gather_u32(phi_local, ix.newid, phi_c, pc_n, al);
                 if (e == cudaSuccess) e = bt::settle(pc_map, pc_n, pc_ass, phi_c, d_phi, d_asg, al);
                 if (e != cudaSuccess) rc = cuda_fail(h, e, "peeling a candidate subgraph");

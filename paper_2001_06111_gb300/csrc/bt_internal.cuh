@@ -297,6 +297,8 @@ struct PeelResult {
     uint64_t rounds = 0, levels = 0, updates = 0, kmax = 0, windows = 0, slots = 0, scanned = 0;
     uint64_t inc_phases = 0;  // rounds that ran a separate incidence phase
     uint32_t parts = 0;       // coarse peel: parts made
+    bool narrow = false;      // coarse peel: given up at its first jump, the grid should peel the whole graph
+    uint32_t zero_edges = 0;  // coarse peel without k_init: edges in no butterfly; if any, they are part 0
     // coarse peel with k_init: rounds, levels and updates of the first part
     uint64_t first_rounds = 0, first_levels = 0, first_updates = 0;
     int status = BT_OK;
@@ -315,7 +317,8 @@ struct PeelOpts {
     // aims at 1/parts_hint of all links and edges; phi_out receives the part of every edge (parts
     // ascend with phi) and snap its support when its part began, all edges of
     // lower parts being gone.  With k_init > 0 the first part is every edge up to
-    // k_init (it may be empty), in the batches of the fine peel.
+    // k_init (it may be empty), in the batches of the fine peel; else the edges in no
+    // butterfly, if there are any.
     int *snap = nullptr;
     uint32_t parts_hint = 0, max_parts = 0;
 };
@@ -336,9 +339,12 @@ struct __align__(32) BloomRec {
     uint32_t k, c;       // k_B, pairs that died in the current round
     uint2 pair[2];
 };
+// (Its arrays stay with the allocator: the caller gives back all of a peel's with undo_to.)
 struct PartGraph {
     uint64_t m = 0, nb = 0;   // edges of all parts (assigned edges are in none)
     uint64_t deep = 0;        // edges of the graph: supports are below it
+    uint32_t first_e = 0;     // edges of a part 0 that is not peeled
+    bool lopsided = false;    // one part would take longer than all by the grid: no part was made, the grid should peel the whole graph
     bool assigned = false;    // some twins are assigned edges (kAssigned); records count their place
     uint32_t np = 0;
     const uint32_t *part_e = nullptr, *part_b = nullptr;  // [np + 1]
@@ -349,22 +355,16 @@ struct PartGraph {
     const uint2 *pairs = nullptr;     // twin pairs (flagged the same way) of blooms of more than two
     BloomRec *bl = nullptr;           // consumed by the peel
     const uint32_t *out_id = nullptr;  // [m] the index's id of each edge, or null when the numbering is the same
-    void *own[8] = {};  // what free_parts gives back
-    int n_own = 0;
-    template <typename T>
-    T *keep(T *x) {
-        own[n_own++] = x;
-        return x;
-    }
 };
-void free_parts(PartGraph &g, Alloc &al);
 // The whole graph as one part (an index with twin links).
 cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al);
 // The ranges of a coarse peel as parts: part[e] in [0, np), snap[e] the support
 // of e when its part begins.  assigned (nullable): edges that are in no part.
-// skip_first: part 0 is not to be peeled.
+// skip_first: part 0 is not to be peeled, its first_rounds rounds being made.
+// May leave g without parts (g.lopsided).
 cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
-                            const uint8_t *assigned, bool skip_first, PartGraph &g, int num_sms, Alloc &al);
+                            const uint8_t *assigned, bool skip_first, uint64_t first_rounds, PartGraph &g,
+                            int num_sms, Alloc &al);
 // Peel of all parts; phi_out receives bitruss numbers of at least assign_from.
 cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_from, PeelResult &res, int num_sms,
                        Alloc &al);

@@ -655,8 +655,8 @@ __global__ void k_depth_sum(const uint32_t *depth, uint64_t m, unsigned long lon
     }
 }
 
-__global__ void k_unplace(const uint32_t *phi, const uint32_t *out_id, uint64_t m, uint32_t *out) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x)
+__global__ void k_unplace(const uint32_t *phi, const uint32_t *out_id, uint64_t first, uint64_t m, uint32_t *out) {
+    for (uint64_t i = first + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x)
         out[out_id[i]] = phi[i];
 }
 
@@ -754,7 +754,7 @@ cudaError_t peel_parts(const PartGraph &g, uint32_t *phi_out, long long assign_f
     }
     BT_CUDA(side.join());
     if (g.out_id) {
-        k_unplace<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(a.phi, g.out_id, m, phi_out);
+        k_unplace<<<grid_for(m - g.first_e, 256, (unsigned)num_sms * 16), 256, 0, st>>>(a.phi, g.out_id, g.first_e, m, phi_out);
         al.launches++;
     }
     k_depth_sum<<<grid_for(deep + 1, 256, (unsigned)num_sms * 8), 256, 0, st>>>(a.depth, deep, hd->sums);

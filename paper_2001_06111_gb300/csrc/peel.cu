@@ -106,6 +106,19 @@ __device__ __forceinline__ long long bin_top(uint32_t b) {
     return ((long long)(64u + (b & 63u) + 1u) << (e - 6u)) - 1;
 }
 
+// Parts pay where bitruss numbers spread: many levels, and ranges of a few per cent
+// of the links each.  Where the supports lie close together (dense blocks,
+// uniform random graphs) almost all edges go in one avalanche: few rounds, each of
+// them wide enough for the grid, and one range with nearly everything in it, which
+// a block or a cluster would peel by itself.  Supports tell: of the links, the
+// share on edges within a factor of 8 in support was 0.957 on a random graph of mean
+// degree 25, 1.0 on denser ones, blocks and equal bicliques, 0.29 to 0.67 on skewed graphs
+// of 1,000 to 30M edges, 0.89 and 0.95 on ones with a single dominating block.  From
+// kNarrow on the grid peels the whole graph (by parts instead: a random
+// graph of 2M edges, mean degree 100, 62 ms against 19; a block of 300 x 300 of
+// density 0.9, 14.1 against 2.2; K_{200,200} 10.9 against 0.3).
+constexpr float kNarrow = 0.955f;
+
 struct Ctl {
     unsigned long long bar_count;  // barrier arrivals (monotonic within a launch)
     unsigned int err;
@@ -127,6 +140,8 @@ struct Ctl {
     unsigned long long kfinal;
     unsigned long long inc_phases;  // rounds that ran a separate incidence phase
     unsigned int n_parts;           // coarse peel: parts made
+    unsigned int narrow;            // coarse peel: given up, the supports lie close together
+    unsigned int n_zero;            // coarse peel: edges without butterflies, part 0
     unsigned long long first_rounds, first_levels, first_updates;  // of its first part, with k_init
     unsigned int hist[2][kBins];    // coarse peel: supports of the alive edges, ping-pong
 };
@@ -470,7 +485,8 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t nthreads = gridDim.x * blockDim.x;
     Ctl *ctl = a.ctl;
-    uint64_t remaining = a.m_active;
+    const uint32_t n_zero = kCoarse ? ctl->n_zero : 0u;
+    uint64_t remaining = a.m_active - n_zero;
     uint32_t round = 0;
     // (a coarse peel keeps no window: khi below every support)
     Lvl L{a.k_init, kCoarse ? LLONG_MIN : 0ll, 0, (uint32_t)a.k_init};
@@ -488,9 +504,11 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
     // coarse: parts begun, the weight the last one began with, all weight then
     uint32_t pno = 0, picked = 1, total_jump = 0;
     float aim = (float)a.target;
-    // with k_init > 0 part 0 is given; the parts whose tops are chosen here follow
+    // part 0 may be given (k_init > 0: what lies up to k_init; else the edges without
+    // butterflies, if any); the parts whose tops are chosen here follow
     bool in_first = kCoarse && a.k_init > 0;
-    const uint32_t first_free = in_first ? 1u : 0u;
+    const uint32_t first_free = in_first || n_zero ? 1u : 0u;
+    bool narrow = false;
     pno = first_free;
     uint32_t hno = 0;                  // level jumps
     long long first_top = LLONG_MIN, lim = 0;  // the first part's window, what a jump takes
@@ -552,7 +570,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                     }
                 }
                 constexpr uint32_t U = 4;  // entries a lane has in flight
-                if (!within) {
+                if (!within || hno == 0) {
                     // C1: the alive edges again, with their supports' histogram and
                     // a copy of each support (the last copy an edge gets is its
                     // support when its part begins)
@@ -611,20 +629,47 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                         ap ^= 1u;
                         if (gtid == 0) ctl->n_alive[ap ^ 1u] = 0;
                     }
-                    L.label = pno;
                     // every block finds the class up to which the edges of the next
                     // part reach
-                    {
-                        constexpr uint32_t kPer = (kBins + kT - 1) / kT;
-                        uint32_t mine[kPer], sum = 0;
+                    constexpr uint32_t kPer = (kBins + kT - 1) / kT;
+                    uint32_t mine[kPer], sum = 0;
+#pragma unroll
+                    for (uint32_t r = 0; r < kPer; ++r) {
+                        const uint32_t b = threadIdx.x * kPer + r;
+                        mine[r] = b < kBins ? __ldcg(&ctl->hist[hno & 1u][b]) : 0u;
+                        sum += mine[r];
+                    }
+                    uint32_t total;
+                    uint32_t cum = dev::block_excl_scan<uint32_t>(sum, &total);
+                    if (hno == 0) {
+                        // the largest weight within a factor of 8 in support
+                        uint32_t run = cum, most = 0;
+                        if (threadIdx.x == 0) s_cum = 0;
 #pragma unroll
                         for (uint32_t r = 0; r < kPer; ++r) {
                             const uint32_t b = threadIdx.x * kPer + r;
-                            mine[r] = b < kBins ? __ldcg(&ctl->hist[hno & 1u][b]) : 0u;
-                            sum += mine[r];
+                            run += mine[r];
+                            if (b < kBins) s_hist[b] = run;
                         }
-                        uint32_t total;
-                        uint32_t cum = dev::block_excl_scan<uint32_t>(sum, &total);
+                        __syncthreads();
+                        run = cum;
+#pragma unroll
+                        for (uint32_t r = 0; r < kPer; ++r) {
+                            const uint32_t b = threadIdx.x * kPer + r;
+                            if (b < kBins && mine[r]) {
+                                const uint32_t w = s_hist[bin_of(8ull * (unsigned long long)bin_top(b))] - run;
+                                most = w > most ? w : most;
+                            }
+                            run += mine[r];
+                        }
+                        if (most) atomicMax(&s_cum, most);
+                        __syncthreads();
+                        narrow = (float)s_cum >= kNarrow * (float)total;
+                        if (narrow) break;
+                        __syncthreads();  // (s_cum is used again)
+                    }
+                    if (!within) {
+                        L.label = pno;
                         if (pno + 1u >= a.max_parts || total <= a.target + a.target / 2u) {
                             // the rest is the last part: nothing is left to be told apart
                             for (uint32_t i = gtid; i < v_alive; i += nthreads) {
@@ -654,10 +699,10 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                         L.k = lim = bin_top(s_bin);
                         picked = s_cum;
                         total_jump = total;
-                        for (uint32_t i = gtid; i < kBins; i += nthreads) ctl->hist[(hno & 1u) ^ 1u][i] = 0;
-                        ++hno;
                         ++pno;
                     }
+                    for (uint32_t i = gtid; i < kBins; i += nthreads) ctl->hist[(hno & 1u) ^ 1u][i] = 0;
+                    ++hno;
                 }
                 // C2: their links become incidence items of this round
                 uint32_t sel = 0;
@@ -1089,20 +1134,31 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
         ctl->rounds = round;
         ctl->kfinal = (unsigned long long)L.k;
         ctl->n_parts = pno;
+        ctl->narrow = narrow;
     }
 }
 
 // Edges already assigned (mask set) start in the permanent state: never alive,
-// never queued.
+// never queued.  So do, for a coarse peel from level 0 (zero_part not null), the
+// edges in no butterfly: they are the batch of level 0 and change nothing else.
 constexpr uint32_t kPerm = 0xFFFFFFFEu;
 __global__ void k_peel_init(const uint64_t *support, uint64_t m, int *sup, uint32_t *state,
-                            const uint8_t *assigned, uint32_t *alive) {
+                            const uint8_t *assigned, uint32_t *alive, uint32_t *zero_part, unsigned int *n_zero) {
+    uint32_t zeros = 0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        sup[i] = (int)support[i];
-        state[i] = (assigned && assigned[i]) ? kPerm : kAlive;
+        const uint64_t v = support[i];
+        const bool fixed = assigned && assigned[i], zero = !fixed && zero_part && v == 0;
+        sup[i] = (int)v;
+        state[i] = fixed || zero ? kPerm : kAlive;
         alive[i] = (uint32_t)i;
+        if (zero) {
+            zero_part[i] = 0;
+            ++zeros;
+        }
     }
+    zeros = dev::warp_sum(zeros);
+    if ((threadIdx.x & 31) == 0 && zeros) atomicAdd(n_zero, zeros);
 }
 
 // Bloom words: no round has touched the bloom yet, k_B from the index.
@@ -1189,27 +1245,26 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     a.max_parts = coarse ? opts->max_parts : 0;
     if (al.err != cudaSuccess) return al.err;
     cudaStream_t st = al.stream;
-    if (!coarse) al.mark(kPhPeel, false);  // (a coarse peel is part of its caller's phase)
-    k_peel_init<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(
-        support, m, a.sup, a.state, opts ? opts->assigned : nullptr, a.alive[0]);
-    al.launches++;
-    BT_CUDA(cudaMemsetAsync(a.died, 0xFF, sizeof(uint32_t) * (ix.w2 ? ix.w2 : 1), st));
-    if (ix.nb) {
-        k_bloom_words<<<grid_for(ix.nb, 256, (unsigned)num_sms * 16), 256, 0, st>>>(ix.bloom_k, ix.nb, a.blooms);
-        al.launches++;
-    }
     Ctl h{};
     h.n_alive[0] = (unsigned int)m;
     h.minsup = ~0ull;
     h.minsup2 = ~0ull;
     BT_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(Ctl), st));
     BT_CUDA(cudaMemcpyAsync(a.ctl, &h, offsetof(Ctl, hist), cudaMemcpyHostToDevice, st));
+    k_peel_init<<<grid_for(m, 256, (unsigned)num_sms * 16), 256, 0, st>>>(
+        support, m, a.sup, a.state, opts ? opts->assigned : nullptr, a.alive[0],
+        coarse && a.k_init == 0 ? a.phi : nullptr, &a.ctl->n_zero);
+    al.launches++;
+    BT_CUDA(cudaMemsetAsync(a.died, 0xFF, sizeof(uint32_t) * (ix.w2 ? ix.w2 : 1), st));
+    if (ix.nb) {
+        k_bloom_words<<<grid_for(ix.nb, 256, (unsigned)num_sms * 16), 256, 0, st>>>(ix.bloom_k, ix.nb, a.blooms);
+        al.launches++;
+    }
     void *kargs[] = {&a};
     BT_CUDA(cudaLaunchCooperativeKernel(kfn, grid, block, kargs, 0, st));
     al.launches++;
     BT_CUDA(cudaMemcpyAsync(&h, a.ctl, offsetof(Ctl, hist), cudaMemcpyDeviceToHost, st));
     BT_CUDA(cudaStreamSynchronize(st));
-    if (!coarse) al.mark(kPhPeel, true);
     if (h.err & kErrBarrier) res.status = BT_ERR_CUDA;
     else if (h.err & kErrPeelOverflow) res.status = BT_ERR_OVERFLOW;
     else if (h.err & kErrRounds) res.status = BT_ERR_NOCONVERGE;
@@ -1222,6 +1277,8 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     res.kmax = h.kfinal;
     res.inc_phases = h.inc_phases;
     res.parts = h.n_parts;
+    res.narrow = h.narrow != 0;
+    res.zero_edges = h.n_zero;
     res.first_rounds = h.first_rounds;
     res.first_levels = h.first_levels;
     res.first_updates = h.first_updates;

@@ -15,6 +15,7 @@
 // butterfly and is dropped.  Supports at the start of a part come from the
 // coarse peel, so each part is peeled without any other.
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "bt_device.cuh"
@@ -32,6 +33,24 @@ constexpr int kT = 256;
 // (the clusters take the SMs of the other parts, and their barriers cost more);
 // with 6 or 12: the same within 1 %.
 constexpr double kHeavy = 4.0;
+// The mean says nothing where there are few parts: with fewer than kFewParts the
+// limit is that of as many, but at least kBlockLinks links, 1 to 2 ms of one
+// block (K_{200,200} of 8M links beside smaller bicliques: 10 ms by one block).
+constexpr double kFewParts = 40.0;
+constexpr double kBlockLinks = 1 << 19;
+// What a part takes by itself, nanoseconds a link by a block (2.9 to 5.1: random
+// graphs of 20,000 edges, blocks of 100 x 100) and a link and an edge by a cluster
+// (0.37 to 0.57: random graphs of 1M and 2M edges, a block of 1000 x 1000; 4.3:
+// edges in no butterfly).  The grid takes 8 us for each round of every part in turn, 2
+// more than a block, and 0.1 ns a link.  Rounds of a part on skewed graphs: 57 at
+// 5,000 links, 82 at 24,000, 165 at 114,000, 471 at 1.2M, and no more than 600.  Where
+// the longest part takes longer than all that, the rounds of a first part that
+// would be made again among it, it is no range among others: the grid peels the graph.  (Three random graphs of 0.5M to 2M edges by
+// parts 157 ms, by the grid 122; two sizes of bicliques 13.4 and 1.8; a 300 x 300 block in
+// a skewed graph of 200,000 edges 15.4 and 32.)
+constexpr double kBlockLinkNs = 3.7, kClusterLinkNs = 0.45, kClusterEdgeNs = 4.3;
+constexpr double kGridRoundNs = 8000.0, kGridMoreNs = 2000.0, kGridLinkNs = 0.1;
+inline double rounds_of(double links) { return std::min(600.0, 57.0 * std::pow(links / 5000.0, 0.45)); }
 constexpr int kSmall = 8;  // pairs of a bloom that one thread groups by itself
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -411,22 +430,17 @@ __global__ void __launch_bounds__(kT) k_split_links(const uint64_t *inc_off, con
 
 }  // namespace
 
-void free_parts(PartGraph &g, Alloc &al) {
-    for (int i = 0; i < g.n_own; ++i) al.put(g.own[i]);
-    g = PartGraph{};
-}
-
 cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int num_sms, Alloc &al) {
     g.m = g.deep = ix.m;
     g.nb = ix.nb;
     g.np = 1;
     g.inc = ix.inc;
     g.pairs = ix.pairs;
-    uint32_t *ends = g.keep(al.get<uint32_t>(4));
+    uint32_t *ends = al.get<uint32_t>(4);
     g.part_e = ends;
     g.part_b = ends + 2;
-    g.er = g.keep(al.get<uint4>(ix.m));
-    g.bl = g.keep(al.get<BloomRec>(ix.nb));
+    g.er = al.get<uint4>(ix.m);
+    g.bl = al.get<BloomRec>(ix.nb);
     if (al.err != cudaSuccess) return al.err;
     const unsigned wide = (unsigned)num_sms * 16;
     k_edge_rec<<<grid_for(ix.m, 256, wide), 256, 0, al.stream>>>(ix.inc_off, support, ix.m, (uint32_t)ix.nb, ends, g.er);
@@ -439,7 +453,8 @@ cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int
 }
 
 cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
-                            const uint8_t *assigned, bool skip_first, PartGraph &g, int num_sms, Alloc &al) {
+                            const uint8_t *assigned, bool skip_first, uint64_t first_rounds, PartGraph &g,
+                            int num_sms, Alloc &al) {
     const uint64_t m = ix.m, nb = ix.nb;
     const unsigned wide = (unsigned)num_sms * 16;
     g.deep = m;
@@ -452,13 +467,12 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     unsigned long long *room = al.get<unsigned long long>(5 * row);
     uint32_t *part_e = reinterpret_cast<uint32_t *>(room + row), *tally = part_e + row;
     uint32_t *cursor = tally, *part_b = tally + 2 * row, *order = part_b + row;
-    g.keep(room);
-    uint32_t *out_id = g.keep(al.get<uint32_t>(m));
+    uint32_t *out_id = al.get<uint32_t>(m);
     g.part_e = part_e;
     g.part_b = part_b;
     g.order = order;
     g.out_id = out_id;
-    g.er = g.keep(al.get<uint4>(m));
+    g.er = al.get<uint4>(m);
     uint32_t *keys = al.get<uint32_t>(m), *tk = al.get<uint32_t>(m), *tv = al.get<uint32_t>(m);
     uint2 *place = al.get<uint2>(m);
     if (al.err != cudaSuccess) return al.err;
@@ -508,9 +522,27 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     }
     g.nb = gsum;
     g.m = he[np];
+    g.first_e = skip_first ? he[1] : 0u;
     // the heaviest first; those that one block would be long at by a cluster
-    const double lim = kHeavy * (double)lsum / np;
+    double lim = kHeavy * (double)lsum / np;
+    if (np < kFewParts) lim = std::min(lim, std::max(kBlockLinks, kHeavy * (double)lsum / kFewParts));
     auto heavy = [&](uint32_t p) { return he[p + 1] - he[p] > kBlockEdges || (double)hr[p] > lim; };
+    double longest = 0, its_rounds = 0, rounds = (double)first_rounds;
+    for (uint32_t p = skip_first; p < np; ++p) {
+        const double links = (double)hr[p], r = rounds_of(links);
+        const double t = heavy(p) ? kClusterLinkNs * links + kClusterEdgeNs * (he[p + 1] - he[p]) : kBlockLinkNs * links;
+        rounds += r;
+        if (t > longest) {
+            longest = t;
+            its_rounds = r;
+        }
+    }
+    g.lopsided =
+        longest > kGridRoundNs * (rounds - its_rounds) + kGridMoreNs * its_rounds + kGridLinkNs * (double)lsum;
+    if (g.lopsided) {
+        al.put(place);
+        return cudaSuccess;
+    }
     std::vector<uint32_t> ord(np);
     for (uint32_t i = 0; i < np; ++i) ord[i] = i;
     if (skip_first) ord.erase(ord.begin());
@@ -522,8 +554,8 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     std::copy(ord.begin(), ord.end(), ho);
     BT_CUDA(cudaMemcpyAsync(room, tab.data(), 40 * row, cudaMemcpyHostToDevice, al.stream));
     uint32_t *sub = al.get<uint32_t>(ix.w2);
-    uint2 *pairs = g.keep(al.get<uint2>(psum)), *inc = g.keep(al.get<uint2>(lsum));
-    g.bl = g.keep(al.get<BloomRec>(gsum));
+    uint2 *pairs = al.get<uint2>(psum), *inc = al.get<uint2>(lsum);
+    g.bl = al.get<BloomRec>(gsum);
     g.pairs = pairs;
     g.inc = inc;
     if (al.err != cudaSuccess) return al.err;

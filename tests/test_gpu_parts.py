@@ -70,6 +70,87 @@ def test_same_as_the_grid_peel(h, m, nplant, lo, hi, flags):
         assert out[2] == ref[2]
 
 
+def union(*gs):
+    """Graphs side by side, edges in one shuffled list: (edges, nU, nL)."""
+    oU = oL = 0
+    es = []
+    for e, a, b in gs:
+        es.append(np.asarray(e, np.int64) + [oU, oL])
+        oU, oL = oU + a, oL + b
+    e = np.concatenate(es)
+    return np.random.default_rng(len(e)).permutation(e).astype(np.int32), oU, oL
+
+
+def uniform(nU, nL, m):
+    k = np.random.default_rng(m).choice(nU * nL, m, replace=False)
+    return np.stack([k // nL, k % nL], 1), nU, nL
+
+
+def blocks(c, a, b):
+    return union(*[(pins.biclique(a, b), a, b)] * c)
+
+
+def skewed(m):
+    g = synth.chunglu(m // 8, m // 12, m, 2.2, 2.4, seed=m)
+    return g.edges, g.nU, g.nL
+
+
+# which way a graph is peeled: by the grid where nearly all links are on edges within a
+# factor of 8 in support, or where one range would take longer than that; edges in
+# no butterfly beside the ranges; a cluster for a part of few with many links
+ROUTES = {
+    "narrow-block": lambda: (pins.biclique(70, 70)[:-50], 70, 70),
+    "narrow-random": lambda: uniform(300, 400, 9000),
+    "narrow-low": lambda: uniform(900, 900, 12000),
+    "factor-8": lambda: union(blocks(3, 21, 21), blocks(1, 57, 57)),
+    "factor-8-and-more": lambda: union(blocks(3, 21, 21), blocks(1, 60, 60)),
+    "one-range": lambda: union(blocks(1, 200, 200), blocks(5, 100, 100)),
+    "few-parts": lambda: union(blocks(1, 200, 200), blocks(20, 60, 60), blocks(1000, 20, 20)),
+    "no-butterflies": lambda: (np.stack([np.arange(5000)] * 2, 1).astype(np.int32), 5000, 5000),
+    "almost-none": lambda: union((np.stack([np.arange(5000)] * 2, 1), 5000, 5000), blocks(1, 2, 2)),
+    "zeros-and-narrow": lambda: union(uniform(60000, 60000, 60000), blocks(4, 30, 30)),
+    "zeros-and-skewed": lambda: union(uniform(60000, 60000, 60000), skewed(20000)),
+    "skewed": lambda: skewed(20000),
+    "skewed-and-block": lambda: union(skewed(60000), blocks(1, 100, 120)),
+    "skewed-and-narrow": lambda: union(skewed(3000), blocks(1, 100, 120)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(ROUTES))
+def test_routes_same_as_the_grid_peel(h, name):
+    e, nU, nL = ROUTES[name]()
+    ref = grid_peel(h, e, nU, nL)
+    out = bt.bt_decompose(h, e, nU, nL)
+    np.testing.assert_array_equal(out[0], ref[0])
+    np.testing.assert_array_equal(out[1], ref[1])
+    assert out[2] == ref[2]
+
+
+# a graph not for parts is given up after the coarse peel's first look (its two kernels of
+# preparation and itself), not after a split; one without butterflies needs nothing more
+@pytest.mark.parametrize("name,more", [("narrow-block", 3), ("narrow-random", 3), ("narrow-low", 3), ("factor-8", 3),
+                                       ("zeros-and-narrow", 3), ("almost-none", 3), ("no-butterflies", 0)])
+def test_given_up_early(h, name, more):
+    e, nU, nL = ROUTES[name]()
+    grid_peel(h, e, nU, nL)
+    launches = bt.bt_profile_read(h)["launches"]
+    bt.bt_decompose(h, e, nU, nL)
+    assert bt.bt_profile_read(h)["launches"] == launches + more
+
+
+@pytest.mark.parametrize("flags", [0, bt.BT_PC_RECOUNT])
+@pytest.mark.parametrize("name", ["narrow-random", "one-range", "few-parts", "zeros-and-narrow", "zeros-and-skewed"])
+def test_routes_of_progressive_passes(h, name, flags):
+    e, nU, nL = ROUTES[name]()
+    bt.bt_set_limits(h, join_cap=1 << 30)
+    ref = bt.bt_decompose_progressive(h, e, nU, nL, tau=0.3, flags=flags)
+    bt.bt_set_limits(h)
+    out = bt.bt_decompose_progressive(h, e, nU, nL, tau=0.3, flags=flags)
+    np.testing.assert_array_equal(out[0], ref[0])
+    np.testing.assert_array_equal(out[1], ref[1])
+    assert out[2] == ref[2]
+
+
 @pytest.mark.parametrize("n,hi", [(3, 300), (5, 600), (40, 20000)])
 def test_batches_same_as_the_grid_peel(h, n, hi):
     gs = [synth.batch_graph(900 + i, hi=hi) for i in range(n)]
