@@ -472,10 +472,11 @@ int bt_server_poll(bt_server *s, uint64_t request_id, int wait, bt_request_info 
 int bt_server_stats_read(bt_server *s, bt_server_stats *out);
 
 /*
- * Device bytes a bt_decompose of this graph needs (host computation, O(m)
- * time; edges are host pointers).  It counts priority-obeyed wedges exactly,
- * so the estimate for the BE-Index is an upper bound (every wedge assumed to
- * lie in a bloom).
+ * Device bytes a bt_decompose of this graph may hold (host computation, O(m)
+ * time; edges are host pointers), an upper bound: it counts priority-obeyed wedges
+ * exactly and takes every one to lie in a bloom of two wedges.  Skewed graphs
+ * hold about half of it.  A call that finds less room than the peel by parts
+ * takes peels by the grid, in up to a third less.
  * Errors: BT_ERR_ARG, BT_ERR_RANGE.
  */
 int bt_estimate_bytes(const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL, uint32_t flags,

@@ -1331,26 +1331,21 @@ int bt_estimate_bytes(const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL
                             (adj.begin() + off[v]));
         }
     if (wedges_out) *wedges_out = W;
-    // CSR + sort scratch + counters (peak), supports/phi/peel state, and an
-    // index bound of 16 bytes per wedge plus per-bloom records (<= W/2 blooms)
-    uint64_t csr = (n + 1) * 8 + 2 * m * (4 + 4 + 4) + n * 12;
-    uint64_t sort_scratch = 2 * m * 24;
-    // two u32 counters per vertex for every resident count block (at most
-    // SMs x resident threads per SM / 256-thread blocks, read from the
-    // current device; a GB300's 152 x 2048 when no device answers)
-    uint64_t resident = 152ull * 2048 / 256;
-    {
-        int dev = 0, sms = 0, tpm = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&tpm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) == cudaSuccess &&
-            sms > 0 && tpm > 0)
-            resident = (uint64_t)sms * (uint64_t)tpm / 256;
-    }
-    uint64_t counters = 2ull * 4 * n * resident;
-    uint64_t edges_b = m * (8 + 8 + 4 + 4 + 4 + 4 + 8 + 8 + 4);
-    uint64_t index_b = W * (8 + 4 + 8 + 1) + (W / 2 + 1) * 16;
-    *bytes_out = csr + std::max(sort_scratch, counters) + edges_b + index_b + (1ull << 20);
+    // Vertices and edges: CSR, sort and peel state.  Wedges, each taken to lie in a
+    // bloom of two: index (pair 8, links 16, half a bloom of 8), then either the peel
+    // by the grid (death stamp 4, items 4, half of 32 of bloom state and of four
+    // lists' 16) or by parts (its group 4, pair 8, links 16, a record of 32 a group):
+    // 84 bytes either way.
+    const uint64_t per_vertex = 64, per_edge = 128, per_wedge = 84;
+    // per-block arrays of the counting and emit kernels, 16 bytes for every vertex (of
+    // the larger layer, above the size from which they go by places in a layer)
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 152;  // a GB300's
+    const uint64_t counters = 16ull * (uint64_t)sms * (n > bt::kPlacesFrom ? std::max(nU, nL) : n);
+    // work lists' room for every block of the peel, and what the memory pool rounds up to
+    const uint64_t fixed = 96ull << 20;
+    *bytes_out = per_vertex * (n + 1) + per_edge * m + per_wedge * W + counters + fixed;
     return BT_OK;
 }
 

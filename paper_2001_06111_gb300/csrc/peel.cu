@@ -337,7 +337,8 @@ __device__ __forceinline__ void kill_pairs(const PeelArgs &a, const uint2 (&l)[N
 // Places of bloom items a warp has taken from the list's counter and not filled
 // yet: in an incidence phase a warp takes kTake at a time, since millions of
 // first kills would otherwise queue on the one counter (about 4 ns each).
-// What is left at the end is filled with empty items.
+// All of them are filled before more are taken, so the list needs room for one
+// stock a warp beside its items; what is left at the end is filled with empty items.
 constexpr uint32_t kTake = 128;
 struct Slots {
     uint32_t next = 0, left = 0;
@@ -371,7 +372,7 @@ __device__ __forceinline__ void warp_kills(const PeelArgs &a, uint32_t q, const 
         mine += nseg[r];
     }
     const uint32_t qb = q & 3u;
-    uint32_t slot;
+    uint32_t slot, cut = 0xFFFFFFFFu, jump = 0;  // places from `cut` on lie `jump` further
     if constexpr (kMode == 1) {
         uint32_t all;
         slot = dev::block_excl_scan<uint32_t>(mine, &all);
@@ -385,17 +386,20 @@ __device__ __forceinline__ void warp_kills(const PeelArgs &a, uint32_t q, const 
         const uint32_t all = __shfl_sync(kFull, incl, 31);
         if (all == 0) return;
         if constexpr (kMode == 2) {
+            slot = t.next + incl - mine;
             if (all > t.left) {
-                fill_empty(a, qb, t, lane);
-                const uint32_t take = all > kTake ? all : kTake;
+                const uint32_t more = all - t.left, take = more > kTake ? more : kTake;
                 uint32_t base = 0;
                 if (lane == 0) base = atomicAdd(&a.ctl->n_bseg[qb], take);
-                t.next = __shfl_sync(kFull, base, 0);
-                t.left = take;
+                base = __shfl_sync(kFull, base, 0);
+                cut = t.next + t.left;
+                jump = base - cut;
+                t.next = base + more;
+                t.left = take - more;
+            } else {
+                t.next += all;
+                t.left -= all;
             }
-            slot = t.next + incl - mine;
-            t.next += all;
-            t.left -= all;
         } else {
             uint32_t base = 0;
             if (lane == 31) base = atomicAdd(&a.ctl->n_bseg[qb], all);
@@ -406,7 +410,7 @@ __device__ __forceinline__ void warp_kills(const PeelArgs &a, uint32_t q, const 
     for (uint32_t r = 0; r < N; ++r)
         for (uint32_t s = 0; s < nseg[r]; ++s, ++slot) {
             const uint32_t left = span[r] - s * kSeg;
-            a.bseg[qb][slot] =
+            a.bseg[qb][kMode == 2 && slot >= cut ? slot + jump : slot] =
                 make_uint4(B[r], bo0[r] + s * kSeg, (left < kSeg ? left : kSeg) | (s == 0 ? 0x80000000u : 0u), 0u);
         }
 }
@@ -1199,9 +1203,8 @@ cudaError_t peel(const Index &ix, const uint64_t *support, uint32_t *phi_out, Pe
     const dim3 grid((unsigned)(num_sms * bps)), block(kT);
     // one round queues each edge and each bloom at most once
     const uint64_t item_cap = m + (2 * ix.w2) / kSeg + 2;
-    // (each bloom at most once), beside the places a warp takes and leaves empty
-    // in an incidence phase: fewer than it fills each time, and a last stock
-    const uint64_t bseg_cap = 2 * (ix.nb + ix.w2 / kSeg) + (uint64_t)grid.x * (kT / 32) * kTake + 2;
+    // (beside the places a warp has taken and not filled)
+    const uint64_t bseg_cap = ix.nb + ix.w2 / kSeg + (uint64_t)grid.x * (kT / 32) * kTake + 2;
     PeelArgs a{};
     a.m = m;
     a.inc_off = ix.inc_off;

@@ -15,8 +15,9 @@
 // Admission: a request's device footprint is bounded from its degrees in O(m)
 // (priority-obeyed wedges W <= sum over edges of min(d(u), d(v)), Lemma 6;
 // BE-Index bytes grow with W) and the sum over in-flight requests must stay
-// under the configured budget.  A request whose bound alone exceeds the
-// budget is rejected with BT_ERR_NOMEM.
+// under the configured budget.  A request that cannot do with the
+// budget alone is rejected with BT_ERR_NOMEM; one that can, peeled by the grid
+// (a call that has no room for parts is), but not by parts, is charged the former.
 #include <algorithm>
 #include <chrono>
 #include <condition_variable>
@@ -36,6 +37,7 @@ struct Request {
     uint64_t id;
     bt_graph g;
     uint64_t bytes;      // admission bound, without the counting kernels' per-block counters
+    uint64_t least;      // what it can do with, without them
     uint64_t cnt_bytes;  // those counters for this graph (a batch needs them once, for its largest graph)
     int status = -1; // -1 pending
     double t_submit = 0, t_start = 0, t_done = 0;
@@ -45,16 +47,13 @@ double now_s() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
 
-// Per-block counters of the counting kernels: two u32 arrays per resident
-// block, one entry per vertex of the largest graph of a batch; at most
-// (SMs x resident threads per SM) / 256-thread blocks are resident.
-uint64_t counter_bound(const bt_graph &g, uint64_t resident_blocks) {
-    return ((uint64_t)g.nU + g.nL) * 8ull * resident_blocks;
-}
+// Per-block arrays of the counting and emit kernels: at most 16 bytes for each vertex
+// of the largest graph of a batch in each of the blocks, one an SM.
+uint64_t counter_bound(const bt_graph &g, uint64_t blocks) { return ((uint64_t)g.nU + g.nL) * 16ull * blocks; }
 
-// Upper bound on the device bytes a decomposition of g needs (host, O(m)),
-// apart from the counters above.
-uint64_t footprint_bound(const bt_graph &g, uint32_t flags, bool device_ptrs) {
+// Device bytes a decomposition of g may hold (host, O(m)), apart from the counters
+// above; least: what it can do with.
+uint64_t footprint_bound(const bt_graph &g, bool device_ptrs, uint64_t &least) {
     const uint64_t m = g.m;
     const uint64_t n = (uint64_t)g.nU + g.nL;
     uint64_t W = 0;
@@ -75,10 +74,11 @@ uint64_t footprint_bound(const bt_graph &g, uint32_t flags, bool device_ptrs) {
     } else {
         W = m * m;  // no host view of the edges: the trivial bound
     }
-    (void)flags;
     // CSR and sort scratch, per-edge peel state, index (pairs, bloom ids,
-    // links, death stamps, blooms) and per-SM counters
-    return (n + 1) * 32 + m * 160 + W * 32 + (64ull << 20);
+    // links, death stamps, blooms); by parts, these of the parts too (37 bytes of each
+    // W of the bound above at most, 33 on the 2M-edge graph, 36 with one planted block)
+    least = (n + 1) * 32 + m * 160 + W * 32 + (64ull << 20);
+    return (n + 1) * 64 + m * 160 + W * 64 + (96ull << 20);
 }
 
 }  // namespace
@@ -94,7 +94,7 @@ struct bt_server {
     bool stop = false;
     uint64_t next_id = 1;
     uint64_t in_flight_bytes = 0;
-    uint64_t resident_blocks = 0;  // 256-thread blocks the device holds at once
+    uint64_t sms = 0;
     bt_server_stats stats{};
     std::vector<bt_handle *> handles;
 
@@ -114,7 +114,7 @@ struct bt_server {
                 // requests that can never fit are rejected first
                 for (auto it = queue.begin(); it != queue.end();) {
                     Request *r = *it;
-                    if (r->bytes + r->cnt_bytes <= cfg.memory_budget_bytes) {
+                    if (r->least + r->cnt_bytes <= cfg.memory_budget_bytes) {
                         ++it;
                         continue;
                     }
@@ -252,13 +252,12 @@ int bt_server_create(bt_server **out, int device, const bt_server_config *cfg) {
         delete s;
         return BT_ERR_ARG;
     }
-    int sms = 0, tpm = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&tpm, cudaDevAttrMaxThreadsPerMultiProcessor, device) != cudaSuccess) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         delete s;
         return BT_ERR_CUDA;
     }
-    s->resident_blocks = (uint64_t)sms * (uint64_t)tpm / 256;
+    s->sms = (uint64_t)sms;
     for (uint32_t i = 0; i < s->cfg.workers; ++i) {
         bt_handle *h = nullptr;
         int rc = bt_create(&h, device, nullptr);
@@ -319,8 +318,9 @@ int bt_server_submit(bt_server *s, const bt_graph *g, uint64_t *request_id) {
     Request *r = new (std::nothrow) Request();
     if (!r) return BT_ERR_NOMEM;
     r->g = *g;
-    r->bytes = footprint_bound(*g, s->cfg.flags, false);
-    r->cnt_bytes = counter_bound(*g, s->resident_blocks);
+    r->bytes = footprint_bound(*g, false, r->least);
+    r->cnt_bytes = counter_bound(*g, s->sms);
+    if (r->bytes + r->cnt_bytes > s->cfg.memory_budget_bytes) r->bytes = r->least;
     r->t_submit = now_s();
     {
         std::lock_guard<std::mutex> lk(s->mu);

@@ -1,0 +1,77 @@
+"""Device memory a call may hold: the estimate of bt_estimate_bytes and the server's
+admission bound against what calls really take from the GPU."""
+import numpy as np
+import pytest
+
+from paper_2001_06111_gb300 import bitruss as bt
+from paper_2001_06111_gb300 import build, synth
+from tests import pins
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def skewed(m, nplant=0):
+    g = synth.chunglu(m // 12, m // 30, m, 2.1, 2.4, seed=m, nplant=nplant, plant_lo=250, plant_hi=300, plant_p=0.9)
+    return g.edges, g.nU, g.nL
+
+
+def uniform(nU, nL, m):
+    k = np.unique(np.random.default_rng(m).integers(0, nU * nL, int(1.1 * m)))
+    k = np.random.default_rng(m).permutation(k)[:m]
+    return np.stack([k // nL, k % nL], 1).astype(np.int32), nU, nL
+
+
+# blooms of many pairs, blooms of few (their state weighs most), skewed graphs by parts
+# with and without a dense block, and graphs of many vertices and no blooms
+GRAPHS = {
+    "biclique": lambda: (pins.biclique(400, 400), 400, 400),
+    "uniform": lambda: uniform(20000, 20000, 2000000),
+    "skewed": lambda: skewed(600000),
+    "planted": lambda: skewed(400000, 2),
+    "sparse": lambda: uniform(400000, 100000, 300000),
+}
+
+
+def taken(call):
+    """Bytes a call on a fresh handle took (its memory pool keeps what it took)."""
+    build.build()
+    with bt.bt_create(0) as warm:  # kernels are loaded once
+        for small in (pins.biclique(3, 3), pins.biclique(60, 60)):
+            bt.bt_decompose_batch(warm, [(small, 60, 60)])
+    free = torch.cuda.mem_get_info()[0]
+    with bt.bt_create(0) as h:
+        call(h)
+        return free - torch.cuda.mem_get_info()[0]
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+def test_estimate_is_an_upper_bound(name):
+    e, nU, nL = GRAPHS[name]()
+    used = taken(lambda h: bt.bt_decompose(h, e, nU, nL))
+    assert used <= bt.bt_estimate_bytes(e, nU, nL)[0]
+
+
+@pytest.mark.parametrize("name", ["biclique", "skewed", "planted"])
+def test_admission_bound_covers_a_batch(name):
+    # the counters' share of a batch's bound is charged once, so several requests of
+    # one kind must be covered by the rest
+    e, nU, nL = GRAPHS[name]()
+    n = 4
+    used = taken(lambda h: bt.bt_decompose_batch(h, [(e, nU, nL)] * n))
+    with bt.Server(0) as srv:
+        info, _ = srv.poll(srv.submit(e, nU, nL), wait=True)
+        counters = 16 * 152 * (nU + nL)
+        assert used <= n * (info["admitted_bytes"] - counters) + counters
+
+
+def test_a_budget_below_the_bound_still_serves():
+    # parts do not fit the budget, the grid's peel does: served as before
+    e, nU, nL = pins.biclique(100, 100), 100, 100
+    least = 201 * 32 + 10000 * 160 + 1000000 * 32 + (64 << 20) + 16 * 152 * 200
+    with bt.Server(0, memory_budget_bytes=least) as srv:
+        info, (_, phi) = srv.poll(srv.submit(e, nU, nL), wait=True)
+    assert info["status"] == bt.BT_OK and (phi == 99 * 99).all() and info["admitted_bytes"] == least
+    with bt.Server(0, memory_budget_bytes=least - 1) as srv:
+        info, _ = srv.poll(srv.submit(e, nU, nL), wait=True)
+    assert info["status"] == bt.BT_ERR_NOMEM
