@@ -744,11 +744,24 @@ __global__ void __launch_bounds__(256) k_emit_light(const __grid_constant__ Emit
 
 }  // namespace
 
+// Whether a kernel whose per-block arrays did not fit the device's memory should be tried
+// with half the blocks: they take 4 (count) and 16 bytes (emit) a block for every
+// vertex of the larger layer (beyond the counters in shared memory), 460 GB for
+// 190M vertices and a block an SM.  A fixed arena has the room it has, and an
+// injected failure is one.
+static bool fewer_blocks(Alloc &al, unsigned &blocks) {
+    if (al.err != cudaErrorMemoryAllocation || al.arena || al.injected || blocks == 1) return false;
+    cudaGetLastError();
+    al.err = cudaSuccess;
+    blocks /= 2;
+    return true;
+}
+
 cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint32_t lo, uint32_t hi) {
     const bool index = o.inc_cnt != nullptr;
     if (hi > g.n) hi = g.n;
     if (lo > hi) lo = hi;
-    const unsigned blocks = (unsigned)num_sms;
+    unsigned blocks = (unsigned)num_sms;
     // ranks below the counters in shared memory (half as many where they have 32
     // bits, for a start vertex of 2^16 middle vertices: its graph has those and more)
     const uint32_t width = g.cnt_n < 0x10000u ? kHot : kHot / 2;
@@ -767,8 +780,10 @@ cudaError_t count_wedges(const Csr &g, CountOut &o, int num_sms, Alloc &al, uint
     a.hi = hi;
     a.vbase = g.vbase;
     a.cold_n = g.cnt_n > width ? g.cnt_n - width : 0u;
-    a.cold = al.get<uint32_t>((size_t)blocks * a.cold_n);
     a.queue = al.get<uint32_t>(1);
+    if (al.err != cudaSuccess) return al.err;
+    while (!(a.cold = al.get<uint32_t>((size_t)blocks * a.cold_n)) && fewer_blocks(al, blocks)) {
+    }
     a.totals = reinterpret_cast<unsigned long long *>(g.totals + 1);
     if (al.err != cudaSuccess) return al.err;
     a.support = reinterpret_cast<unsigned long long *>(o.support);
@@ -836,7 +851,7 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     ix.bloom_off = al.get<uint32_t>(ix.nb + 1);
     ix.pairs = al.get<uint2>(ix.w2);
     ix.inc = al.get<uint2>(ix.links);
-    const unsigned blocks = (unsigned)num_sms;
+    unsigned blocks = (unsigned)num_sms;
     EmitArgs a{};
     a.c.off = g.off;
     a.c.adj = g.adj;
@@ -852,12 +867,19 @@ cudaError_t emit_index(const Csr &g, const CountOut &c, Index &ix, int num_sms, 
     a.c.vbase = g.vbase;
     const uint32_t width = g.cnt_n < 0x10000u ? kHotE : kHotE / 2;  // as in count_wedges
     a.c.cold_n = g.cnt_n > width ? g.cnt_n - width : 0u;
-    a.c.cold = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
     a.c.queue = al.get<uint32_t>(1);
     a.c.assigned = c.assigned;
-    a.word = al.get<unsigned long long>((size_t)blocks * g.cnt_n);
-    a.found = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
     if (al.err != cudaSuccess) return al.err;
+    for (;;) {
+        const size_t held = al.live.size();
+        a.c.cold = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
+        a.word = al.get<unsigned long long>((size_t)blocks * g.cnt_n);
+        a.found = al.get<uint32_t>((size_t)blocks * a.c.cold_n);
+        if (al.err == cudaSuccess) break;
+        if (!fewer_blocks(al, blocks)) return al.err;
+        al.undo_to(held);
+        BT_CUDA(cudaStreamSynchronize(stream));
+    }
     a.cnt_n = g.cnt_n;
     a.bloom_base = bloom_base;
     a.pair_base = pair_base;

@@ -75,3 +75,18 @@ def test_a_budget_below_the_bound_still_serves():
     with bt.Server(0, memory_budget_bytes=least - 1) as srv:
         info, _ = srv.poll(srv.submit(e, nU, nL), wait=True)
     assert info["status"] == bt.BT_ERR_NOMEM
+
+
+def test_counters_of_many_vertices_by_fewer_blocks():
+    # a block an SM would take 365 GB for emit's arrays: ids spread over 150M + 10M
+    # vertices, which changes no vertex's place in the priority order among those
+    # with edges
+    g = synth.chunglu(3000, 2000, 40000, 2.1, 2.4, seed=8)
+    far = g.edges * np.array([[50000, 5000]], dtype=np.int32)
+    with bt.bt_create(0) as h:
+        near = bt.bt_decompose(h, g.edges, g.nU, g.nL)
+        out = bt.bt_decompose(h, far, 150_000_000, 10_000_000)
+        np.testing.assert_array_equal(bt.bt_count_support(h, far, 150_000_000, 10_000_000), near[0])
+    np.testing.assert_array_equal(out[0], near[0])
+    np.testing.assert_array_equal(out[1], near[1])
+    assert out[2] == near[2]
