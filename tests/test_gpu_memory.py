@@ -90,3 +90,51 @@ def test_counters_of_many_vertices_by_fewer_blocks():
     np.testing.assert_array_equal(out[0], near[0])
     np.testing.assert_array_equal(out[1], near[1])
     assert out[2] == near[2]
+
+
+def _decompose(h, g):
+    return bt.bt_decompose(h, g.edges, g.nU, g.nL)[:2]
+
+
+def _batch(h, g):
+    return [x for r in bt.bt_decompose_batch(h, [(g.edges, g.nU, g.nL)] * 2)[0] for x in r]
+
+
+def _progressive(h, g):
+    return bt.bt_decompose_progressive(h, g.edges, g.nU, g.nL, tau=0.5)[:2]
+
+
+# a GPU that is full but for a part of what a call takes when it may: the call runs out of
+# memory somewhere between its first array and its last, and either says so or,
+# where only the parts do not fit, peels by the grid with the same results
+@pytest.mark.parametrize("call", [_decompose, _batch, _progressive])
+def test_calls_on_a_full_gpu(call):
+    g = synth.chunglu(50000, 20000, 600000, 2.1, 2.4, seed=3)
+    want = []
+    used = taken(lambda h: want.extend(call(h, g)))
+    with bt.bt_create(0) as h:
+        call(h, g)
+        launches = bt.bt_profile_read(h)["launches"]
+        bt.bt_set_limits(h, join_cap=1 << 30)
+        for a, b in zip(want, call(h, g)):  # (and the grid's kernels are loaded)
+            np.testing.assert_array_equal(a, b)
+    refused = otherwise = 0
+    for share in np.linspace(0.35, 1.1, 13):
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        full = torch.empty(free - int(share * used), dtype=torch.uint8, device="cuda")
+        with bt.bt_create(0) as h:
+            try:
+                out = call(h, g)
+            except bt.BitrussError as err:
+                assert err.code == bt.BT_ERR_NOMEM
+                refused += 1
+                out = want
+            otherwise += bt.bt_profile_read(h)["launches"] != launches
+            for a, b in zip(want, out):
+                np.testing.assert_array_equal(a, b)
+            del full
+            torch.cuda.empty_cache()
+            for a, b in zip(want, call(h, g)):  # the handle is as good as before
+                np.testing.assert_array_equal(a, b)
+    assert 0 < refused < 13 and otherwise > refused
