@@ -6,6 +6,7 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <new>
 #include <vector>
 
 #include "../../include/bitruss.h"
@@ -142,7 +143,13 @@ struct Alloc {
         }
         err = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
         if (err != cudaSuccess) return nullptr;
-        live.push_back(p);
+        try {
+            live.push_back(p);
+        } catch (const std::bad_alloc &) {  // (no exception may leave a C entry)
+            cudaFreeAsync(p, stream);
+            err = cudaErrorMemoryAllocation;
+            return nullptr;
+        }
         return static_cast<T *>(p);
     }
     void put(void *p) {

@@ -452,9 +452,9 @@ cudaError_t one_part(const Index &ix, const uint64_t *support, PartGraph &g, int
     return cudaGetLastError();
 }
 
-cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
-                            const uint8_t *assigned, bool skip_first, uint64_t first_rounds, PartGraph &g,
-                            int num_sms, Alloc &al) {
+static cudaError_t make_parts(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
+                              const uint8_t *assigned, bool skip_first, uint64_t first_rounds, PartGraph &g,
+                              int num_sms, Alloc &al) {
     const uint64_t m = ix.m, nb = ix.nb;
     const unsigned wide = (unsigned)num_sms * 16;
     g.deep = m;
@@ -577,6 +577,16 @@ cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *sn
     al.put(place);
     al.put(sub);
     return cudaSuccess;
+}
+
+cudaError_t parts_of_ranges(const Index &ix, const uint32_t *part, const int *snap, uint32_t np,
+                            const uint8_t *assigned, bool skip_first, uint64_t first_rounds, PartGraph &g,
+                            int num_sms, Alloc &al) {
+    try {
+        return make_parts(ix, part, snap, np, assigned, skip_first, first_rounds, g, num_sms, al);
+    } catch (const std::bad_alloc &) {  // the host's tables
+        return cudaErrorMemoryAllocation;
+    }
 }
 
 }  // namespace bt
