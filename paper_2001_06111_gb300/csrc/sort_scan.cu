@@ -268,6 +268,10 @@ cudaError_t radix_sort_u32(uint32_t *keys, uint32_t *vals, uint32_t *tk, uint32_
 }
 cudaError_t radix_order_desc_u32(const uint32_t *keys, size_t n, uint32_t *order, uint32_t *sorted, Alloc &al) {
     if (n == 0) return cudaSuccess;
+    if (n == 1) {  // in order as it is (the passes: 0.13 against 0.04 ms)
+        if (sorted) BT_CUDA(cudaMemcpyAsync(sorted, keys, sizeof(uint32_t), cudaMemcpyDeviceToDevice, al.stream));
+        return cudaMemsetAsync(order, 0, sizeof(uint32_t), al.stream);
+    }
     const uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
     uint32_t *hist = al.get<uint32_t>((size_t)256 * ntiles);
     uint32_t *ka = al.get<uint32_t>(n), *va = al.get<uint32_t>(n), *kb = al.get<uint32_t>(n);

@@ -89,3 +89,11 @@ def test_empty_and_errors(h):
     phi = np.zeros(4, np.uint32)
     out = np.zeros(4, np.uint32)
     assert lib.bt_hierarchy(h.ptr, phi.ctypes.data, 4, out.ctypes.data, None, 1 << 7) == bt.BT_ERR_ARG
+
+
+@pytest.mark.parametrize("k", [0, 7, 2**32 - 1])
+def test_one_edge_needs_no_pass(h, k):
+    phi = np.array([k], dtype=np.uint32)
+    order, ps = bt.bt_hierarchy(h, phi)
+    assert order.tolist() == [0] and ps.tolist() == [k]
+    assert bt.bt_profile_read(h)["launches"] == 0
