@@ -674,6 +674,10 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                     }
                     if (!within) {
                         L.label = pno;
+                        // (edges without butterflies still weigh in the first range, so that
+                        // the ranges do not depend on how they are taken out)
+                        const uint32_t gone = pno == first_free && n_zero < a.target ? n_zero : 0u;
+                        total += gone;
                         if (pno + 1u >= a.max_parts || total <= a.target + a.target / 2u) {
                             // the rest is the last part: nothing is left to be told apart
                             for (uint32_t i = gtid; i < v_alive; i += nthreads) {
@@ -689,7 +693,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                             const float grew = (float)(total_jump - total) / (float)picked;
                             aim = fminf(fmaxf((float)a.target / grew, (float)a.target / 32.f), (float)a.target);
                         }
-                        const uint32_t want = aim < 1.f ? 1u : (uint32_t)aim;
+                        const uint32_t want = aim < 1.f + (float)gone ? 1u : (uint32_t)aim - gone;
 #pragma unroll
                         for (uint32_t r = 0; r < kPer; ++r) {
                             // the first class with a weight of at least `want` up to it
@@ -701,7 +705,7 @@ __global__ void __launch_bounds__(peel_threads(kSeg), 1) k_peel(PeelArgs a) {
                         }
                         __syncthreads();
                         L.k = lim = bin_top(s_bin);
-                        picked = s_cum;
+                        picked = s_cum + gone;
                         total_jump = total;
                         ++pno;
                     }

@@ -524,8 +524,9 @@ static cudaError_t make_parts(const Index &ix, const uint32_t *part, const int *
     g.m = he[np];
     g.first_e = skip_first ? he[1] : 0u;
     // the heaviest first; those that one block would be long at by a cluster
-    double lim = kHeavy * (double)lsum / np;
-    if (np < kFewParts) lim = std::min(lim, std::max(kBlockLinks, kHeavy * (double)lsum / kFewParts));
+    const double linked = std::max<double>(1, np - std::count(hr.begin(), hr.begin() + np, 0ull));
+    double lim = kHeavy * (double)lsum / linked;
+    if (linked < kFewParts) lim = std::min(lim, std::max(kBlockLinks, kHeavy * (double)lsum / kFewParts));
     auto heavy = [&](uint32_t p) { return he[p + 1] - he[p] > kBlockEdges || (double)hr[p] > lim; };
     double longest = 0, its_rounds = 0, rounds = (double)first_rounds;
     for (uint32_t p = skip_first; p < np; ++p) {
