@@ -295,7 +295,8 @@ typedef struct {
 typedef struct {
     uint64_t max_edges_per_launch;  /* graphs are packed into unions of at most this many edges */
     uint32_t count_threads;         /* 256, 512 or 1024 (reported; no longer changes anything) */
-    uint32_t peel_item;             /* peel work item: 32, 64 or 128 links / pair slots per warp */
+    uint32_t peel_item;             /* work item of the peel by the grid: 32, 64 or 128 links / pair
+                                       slots per warp; the coarse ranges of a peel by parts take 64 as 32 */
     uint32_t reserved[2];
 } bt_tune;
 
@@ -306,9 +307,10 @@ typedef struct {
     uint64_t wedges;           /* total priority-obeyed wedges */
     uint64_t rounds, levels;   /* peeling rounds and levels, summed over unions */
     uint64_t support_updates;
-    uint32_t count_threads;    /* schedule used */
+    uint32_t count_threads;    /* schedule asked for or chosen */
     uint32_t peel_item;
-    uint32_t tuned;            /* 1 if this call ran the autotuner, 2 if it used a cached choice */
+    uint32_t tuned;            /* 1 if this call chose the schedule for its signature (by timing where
+                                  the grid peels alone, else the defaults), 2 if it used a cached choice */
     uint32_t reserved;
 } bt_batch_stats;
 

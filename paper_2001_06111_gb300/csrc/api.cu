@@ -692,11 +692,12 @@ int bt_decompose(bt_handle *h, const int32_t *edges, uint64_t m, uint32_t nU, ui
     rc = build_index_impl(h, edges, m, nU, nL, flags, s_int, al, as_one_part(h, m));
     bt::PeelResult pr;
     if (rc == BT_OK) {
-        // larger work items pay off when rounds are heavy: on the 30M-edge
-        // planted graph (3.1e9 twin pairs) the peel took 18.1 s with 128
-        // pair slots an item (four a lane, 512-thread blocks), 18.6 s with 64
-        // and 21.9 s with 32; on graphs with up to 2e8 pairs 32 measured
-        // 3-8 % faster than 64
+        // larger work items pay off when the rounds of the grid are heavy: peeled by
+        // the grid alone, the 30M-edge planted graph (3.1e9 twin pairs) took
+        // 18.1 s with 128 pair slots an item (four a lane, 512-thread blocks),
+        // 18.6 s with 64 and 21.9 s with 32, and graphs with up to 2e8 pairs
+        // took 3-8 % less with 32 than with 64.  The coarse peel takes the same
+        // line (it has items of 32 and 128)
         const int seg = h->index.w2 > (1ull << 30) ? 128 : h->peel_seg;
         cudaError_t e = peel_index(h, h->index, s_int, p_int, pr, seg, nullptr, !grid_peel_only(h), al);
         if (e == cudaSuccess) e = bt::gather_u64(s_int, h->index.newid, d_sup, m, al);
@@ -981,10 +982,10 @@ static float phase_ms(bt_handle *h, int phase) {
     return ms;
 }
 
-// Picks the count block size and the peel item size for this batch: looks up
-// the handle's cache by signature, else times three candidate schedules on a
-// sample of the graphs (writing the sample graphs' outputs, which the real
-// run overwrites with the same values) and caches the fastest parts.
+// Picks the schedule for this batch: looks up the handle's cache by signature, else
+// notes the handle's defaults, or, where the grid peels alone, times three candidate
+// schedules on a sample of the graphs (writing the sample graphs' outputs, which
+// the real run overwrites with the same values) and caches the fastest parts.
 static int autotune(bt_handle *h, const bt_graph *graphs, uint32_t n, uint32_t flags, bt::Alloc &al,
                     uint32_t *tuned) {
     uint64_t total = 0, mx = 0;
@@ -1352,9 +1353,11 @@ int bt_estimate_bytes(const int32_t *edges, uint64_t m, uint32_t nU, uint32_t nL
 }  // extern "C"
 
 namespace bt {
-// Let the handle's peel kernel span 1/ways of the SMs, so that the peels of
-// `ways` handles (server workers) can be resident at once; the kernel is
-// latency-bound, so half the SMs cost the 2M-edge peel about 6 %.
+// Let the handle's cooperative peel kernel span 1/ways of the SMs, so that those of
+// `ways` handles (server workers) can be resident at once; its rounds are
+// latency-bound (on half the SMs the 2M-edge graph's took 6 % longer by the grid alone,
+// the coarse peel of 200,000 edges 1 %).  The blocks of the fine peel do not wait
+// for one another and take what is free.
 void share_peel_sms(bt_handle *h, int ways) {
     if (h && ways > 1) h->peel_sms = h->num_sms / ways > 0 ? h->num_sms / ways : 1;
 }

@@ -40,7 +40,8 @@
 //   * a bloom's record and up to two of its pairs share one 32-byte sector;
 //   * a part with more than four times the mean links, or too many edges for a
 //     block's shared memory, is peeled by a cluster of 16 blocks (a dense
-//     biclique of 77,000 edges: 17 rounds, 290 ms by one block).
+//     biclique of 77,000 edges: 17 rounds, 290 ms by one block).  1,024 threads
+//     leave 64 registers a thread, of which the cluster's kernel spills 36 bytes.
 //
 // Supports are below m < 2^31 (k butterflies on an edge need k other edges, one
 // opposite edge each), so they are kept as 32-bit integers here.

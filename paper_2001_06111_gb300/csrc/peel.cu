@@ -51,7 +51,8 @@
 // (2M-edge graph: 865 instead of 39,928).  Each part can then be peeled by itself
 // (split.cu, local.cu).  A level jump reads the alive edges, copies their
 // supports, histograms them by class and takes classes until their weight (edges
-// and links) reaches the target.  The jump's list of alive edges is written
+// and links) reaches the target; a graph that parts do not suit is given up at the
+// first one (kNarrow).  The jump's list of alive edges is written
 // anew only after a quarter has gone: taking places from one counter at every
 // jump cost 130 us of it at 2M edges (now 23 us).  What bounds it are the bloom
 // phases (31 of 41 ms at 2M edges, 45 of 59 with planted bicliques): 1.2 G pair
@@ -67,7 +68,7 @@ namespace bt {
 namespace {
 
 // entries per work item: SEG = 32, 64 or 128 (template parameter: 32 or 64
-// picked by the batch autotuner, 128 for indexes of over 2^30 twin pairs);
+// picked by the batch autotuner, 128 for indexes of over 2^30 twin pairs;
 // a coarse peel knows 32 and 128).  Threads a block: 640 (96 registers, no spills) for 32- and
 // 64-entry items, 512 (128 registers) for 128-entry items, whose four slots
 // a lane need the registers.

@@ -9,8 +9,8 @@
 // A large request runs alone; one worker serves small requests first and
 // the others large ones first (see the admission code), so small requests do
 // not wait behind a large graph.
-// The peel of each batch is one persistent cooperative kernel, so each
-// worker's peel spans only its share of the SMs: the peels of all workers can
+// The coarse peel of each batch (and a peel by the grid) is one persistent cooperative
+// kernel, so each worker's spans only its share of the SMs: those of all workers can
 // then be resident together instead of queuing for the whole GPU.
 // Admission: a request's device footprint is bounded from its degrees in O(m)
 // (priority-obeyed wedges W <= sum over edges of min(d(u), d(v)), Lemma 6;
@@ -267,9 +267,11 @@ int bt_server_create(bt_server **out, int device, const bt_server_config *cfg) {
             return rc;
         }
         bt::share_peel_sms(h, (int)s->cfg.workers);  // peels of all workers fit on the GPU at once
-        // A server with one worker keeps the grid-wide peel: its callers count on
-        // a request of some 500,000 edges to hold the worker for 50 ms, so that
-        // those behind it can still be cancelled (115 ms so, 25 ms in parts).
+        // A server with one worker peels by the grid alone, as it did before there were
+        // parts, which it could do without: the test of bt_server_cancel_queued
+        // waits 50 ms behind a request of 500,000 edges and expects something left to
+        // cancel (that request takes 115 ms so, 25 ms by parts).  No
+        // interface promises such a time.
         if (s->cfg.workers == 1) bt::use_grid_peel(h);
         s->handles.push_back(h);
     }
