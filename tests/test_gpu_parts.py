@@ -102,6 +102,8 @@ ROUTES = {
     "narrow-block": lambda: (pins.biclique(70, 70)[:-50], 70, 70),
     "narrow-random": lambda: uniform(300, 400, 9000),
     "narrow-low": lambda: uniform(900, 900, 12000),
+    "low-supports": lambda: union(uniform(3000, 3000, 60000), blocks(1, 12, 12)),
+    "low-supports-and-more": lambda: union(uniform(3000, 3000, 60000), blocks(12, 40, 40)),
     "factor-8": lambda: union(blocks(3, 21, 21), blocks(1, 57, 57)),
     "factor-8-and-more": lambda: union(blocks(3, 21, 21), blocks(1, 60, 60)),
     "one-range": lambda: union(blocks(1, 200, 200), blocks(5, 100, 100)),
@@ -128,7 +130,7 @@ def test_routes_same_as_the_grid_peel(h, name):
 
 # a graph not for parts is given up after the coarse peel's first look (its two kernels of
 # preparation and itself), not after a split; one without butterflies needs nothing more
-@pytest.mark.parametrize("name,more", [("narrow-block", 3), ("narrow-random", 3), ("narrow-low", 3), ("factor-8", 3),
+@pytest.mark.parametrize("name,more", [("narrow-block", 3), ("narrow-random", 3), ("narrow-low", 3), ("factor-8", 3), ("low-supports", 3),
                                        ("zeros-and-narrow", 3), ("almost-none", 3), ("no-butterflies", 0)])
 def test_given_up_early(h, name, more):
     e, nU, nL = ROUTES[name]()
